@@ -51,7 +51,8 @@ def fp32_ops_general(nL: int, grad: bool, surv: bool) -> int:
 
 
 def fp32_ops_per_node(nL: int, grad: bool, spec: bool) -> int:
-    """Algorithmic FP32 operations (FMA = 1) of the fused kernel per energy node.
+    """Algorithmic FP32 operations (FMA = 1) of the split mapping's and the
+    fits' node kernels per energy node.
 
     Per (node, baseline): double-float phase and two-part reduction mod pi
     2 x 9, sin/cos polynomials 2 x 10 (u = r^2, degree-9 sine 5, degree-8
@@ -71,6 +72,17 @@ def fp32_ops_per_node(nL: int, grad: bool, spec: bool) -> int:
     return nL * per_r + per_node
 
 
+def fp32_ops_anchored(nL: int, grad: bool) -> int:
+    """Algorithmic FP32 operations (FMA = 1) per energy node of the
+    chunk-anchored node kernels (bin and slice mappings): per (node, baseline)
+    two phases by one FMA each from the chunk's anchor 2, sin and cos - 1 of
+    both 22, the third pair by the addition formulas 6 (3 without the
+    gradient), weighted sums 6 (3); per node the offset of 1/E 3, W/E 1 (with
+    the gradient) and the sum of W 4.  Anchors and the additions of a chunk's
+    sums are not counted."""
+    return nL * (36 if grad else 30) + 7 + (1 if grad else 0)
+
+
 # DRAM traffic of one launch of the benchmarked kernels from an ncu capture
 # (dram__bytes_read.sum + dram__bytes_write.sum), per mapping, valid only for
 # the kernel sources it was taken with: reported as null once they change.
@@ -82,10 +94,11 @@ TRAFFIC_CAPTURE = {
                "bytes": 268506880 + 4611584 + 8178176 + 0},
 }
 KERNEL_SOURCES = ["paper_1804_07682_gb300/csrc/common.cuh", "paper_1804_07682_gb300/csrc/fused.cuh",
+                  "paper_1804_07682_gb300/csrc/anchored.cuh",
                   "paper_1804_07682_gb300/csrc/epilogue.cuh", "paper_1804_07682_gb300/csrc/ff_consts.h",
                   "paper_1804_07682_gb300/csrc/slices.cu"]
-KERNEL_NAMES = {"split": "k_fused_split", "slices": "k_fused_bins (slices) + k_slices_reduce",
-                "bins": "k_fused_bins"}
+KERNEL_NAMES = {"split": "k_fused_split", "slices": "k_nodes_multi (slices) + k_slices_reduce",
+                "bins": "k_nodes_multi + k_point_sums"}
 
 
 def kernel_sources_sha256() -> str:
@@ -293,7 +306,7 @@ def side_workloads(api, torch, device, args):
     torch.cuda.synchronize()
     ms = a0.elapsed_time(a1) / reps
     pts = w.points_per_eval()
-    ops = sum(fp32_ops_per_node(1, True, False) * w.nbins * int(n) for n in w.node_counts)
+    ops = sum(fp32_ops_anchored(1, True) * w.nbins * int(n) for n in w.node_counts)
     check = {"scan": (w, N, data.cpu().numpy(), o["chi2"].cpu().numpy(), o["grad"].cpu().numpy())}
     out["scan_64x64_500bins"] = {"scans_per_s": 1e3 / ms, "ms_per_scan": ms, "chi2_grad_evals_per_s": w.npts * 1e3 / ms,
                                  "gpoints_per_s": pts / ms / 1e6, "points_per_scan": pts,
@@ -526,7 +539,8 @@ def side_workloads(api, torch, device, args):
         res[name] = a0.elapsed_time(a1) / 100 * 1e3
     check["nuisance"] = (w, N, data.cpu().numpy(), od["chi2"][0].item(), od["grad"][0].cpu().numpy(),
                          od["grad_eta"][0].cpu().numpy())
-    ops = fp32_ops_per_node(w.nL, True, False) * w.nbins * w.nodes_per_bin
+    ops = (fp32_ops_per_node(w.nL, True, False) if plan.tuning.startswith("mapping=split") else
+           fp32_ops_anchored(w.nL, True)) * w.nbins * w.nodes_per_bin
     out["nuisance_1000x4096"] = {
         "evals_per_s_autograd": 1e6 / res["autograd"], "us_per_eval_autograd": res["autograd"],
         "us_per_eval_autograd_calling_thread": res["autograd_calling_thread"],
@@ -842,12 +856,13 @@ def main():
     kern_avg_ms = kern_ms / max(kern_n, 1)
 
     # roofline of the fused kernel (ALU-bound: FP32 issue)
-    ops = fp32_ops_per_node(w.nL, True, True) * w.nbins * w.nodes_per_bin
+    mapping = plan.tuning.split()[0].split("=")[1]
+    ops = (fp32_ops_per_node(w.nL, True, True) if mapping == "split" else
+           fp32_ops_anchored(w.nL, True)) * w.nbins * w.nodes_per_bin
     achieved_tops = ops / (kern_avg_ms * 1e-3) / 1e12
     peak_tops = SM_COUNT * FP32_LANES * SM_MAX_MHZ * 1e6 / 1e12
     pk, pk_src = peaks()
-    hbm_bytes = 16 * w.nbins * w.nodes_per_bin
-    mapping = plan.tuning.split()[0].split("=")[1]
+    hbm_bytes = (16 if mapping == "split" else 12) * w.nbins * w.nodes_per_bin
     cap = TRAFFIC_CAPTURE.get(mapping, {})
     traffic = cap.get("bytes") if cap.get("sources_sha256") == kernel_sources_sha256() else None
     roofline = {"bound": "alu", "achieved": achieved_tops, "peak": peak_tops, "unit": "TFLOP/s",

@@ -1,0 +1,78 @@
+// anchored_launch.cuh -- choice of the chunk-anchored node kernel: one baseline
+// takes two nodes per packed value, more take 2, 4 or 8 baselines at a time
+// (beyond 8 the nodes are taken again).
+#pragma once
+
+#include <mutex>
+
+#include "anchored.cuh"
+
+namespace gna {
+
+template <int NP, bool GRAD>
+size_t nodes_smem(int block) {
+    return sizeof(f32x2p) * NP * (GRAD ? 6 : 3) * (size_t)block + (size_t)block / 32 * QuadRing<kRingMulti>::kWarpBytes;
+}
+
+inline size_t one_smem(int block) { return (size_t)block / 32 * QuadRing<kRingOne>::kWarpBytes; }
+
+// More than the default 48 KB of dynamic shared memory: opt in once per device and kernel.
+template <auto K>
+cudaError_t allow_smem() {
+    static std::once_flag once[64];
+    static cudaError_t attr[64];
+    int dev = 0;
+    cudaError_t e = cudaGetDevice(&dev);
+    if (e != cudaSuccess) return e;
+    if (dev < 0 || dev >= 64) return cudaErrorInvalidDevice;
+    std::call_once(once[dev], [&] {
+        attr[dev] = cudaFuncSetAttribute(K, cudaFuncAttributeMaxDynamicSharedMemorySize, 72 * 1024);
+    });
+    return attr[dev];
+}
+
+template <int PH, int NP, bool GRAD>
+cudaError_t launch_multi(const BinArgs& a, int grid, int block, cudaStream_t s) {
+    cudaError_t e = allow_smem<k_nodes_multi<PH, NP, GRAD>>();
+    if (e != cudaSuccess) return e;
+    return launch_dependent(k_nodes_multi<PH, NP, GRAD>, a, grid, block, s, nodes_smem<NP, GRAD>(block));
+}
+
+template <int PH, bool GRAD>
+cudaError_t launch_nodes_g(const BinArgs& a, int grid, int block, cudaStream_t s) {
+    if (a.nL <= 1) return launch_dependent(k_nodes_one<PH, GRAD>, a, grid, block, s, one_smem(block));
+    if (a.nL <= 2) return launch_multi<PH, 1, GRAD>(a, grid, block, s);
+    if (a.nL <= 4) return launch_multi<PH, 2, GRAD>(a, grid, block, s);
+    return launch_multi<PH, 4, GRAD>(a, grid, block, s);
+}
+
+template <int PH>
+cudaError_t launch_nodes(bool grad, const BinArgs& a, int grid, int block, cudaStream_t s) {
+    return grad ? launch_nodes_g<PH, true>(a, grid, block, s) : launch_nodes_g<PH, false>(a, grid, block, s);
+}
+
+template <auto K>
+int resident_of(int block, size_t smem) {
+    int n = 0;
+    if (allow_smem<K>() != cudaSuccess) return 1;
+    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, K, block, smem) != cudaSuccess) {
+        cudaGetLastError();
+        return 1;
+    }
+    return n > 0 ? n : 1;
+}
+
+template <int PH, bool GRAD>
+int resident_nodes_g(int nL, int block) {
+    if (nL <= 1) return resident_of<k_nodes_one<PH, GRAD>>(block, one_smem(block));
+    if (nL <= 2) return resident_of<k_nodes_multi<PH, 1, GRAD>>(block, nodes_smem<1, GRAD>(block));
+    if (nL <= 4) return resident_of<k_nodes_multi<PH, 2, GRAD>>(block, nodes_smem<2, GRAD>(block));
+    return resident_of<k_nodes_multi<PH, 4, GRAD>>(block, nodes_smem<4, GRAD>(block));
+}
+
+template <int PH>
+int resident_nodes(int nL, bool grad, int block) {
+    return grad ? resident_nodes_g<PH, true>(nL, block) : resident_nodes_g<PH, false>(nL, block);
+}
+
+}  // namespace gna

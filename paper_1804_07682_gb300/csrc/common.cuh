@@ -34,6 +34,7 @@ struct PointConst {
     double dA13[3];  // d A_ij / d sin^2 theta13
     float Af[3], dA12f[3], dA13f[3];
     float Alo[3];    // A - (double)Af: the amplitudes enter P as hi + lo
+    float cmax;      // largest |c| of the point's phases (rounded up)
 };
 
 // Plan-wide constants passed by value.
@@ -47,6 +48,14 @@ struct BaseConst {
     double wsum_lo;         // sum_r om_r - wsum (exact sum of the FP32 weights)
     int nL;
 };
+
+// Largest |K dm2 L_r| of a point's phases 21 and 32, rounded up (NaN if a splitting is).
+__device__ __forceinline__ float largest_phase(const BaseConst& bc, double dm2_21, double dm2_32) {
+    double kl = 0.0;
+    for (int r = 0; r < bc.nL; r++) kl = bc.kld[r] > kl ? bc.kld[r] : kl;
+    const double a = fabs(dm2_21), b = fabs(dm2_32);
+    return __double2float_ru(kl * ((a >= b || a != a) ? a : b));
+}
 
 // ---------------------------------------------------------------- Kahan --
 struct KahanF {

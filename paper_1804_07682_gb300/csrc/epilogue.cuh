@@ -36,6 +36,7 @@ struct EpiArgs {
     int kind;
     const double* eta;
     double sigma;
+    int penalty;           // eta given and sigma > 0
     const double* data;
     int data_per_point;
     double* mu_out;        // [npts][nbins] or NULL
@@ -44,7 +45,10 @@ struct EpiArgs {
     float2* binvals;       // [npts][nbins][NBV] scratch (double-float values)
     int NBV;               // 1 (chi2), 5 (+ gradient), 15 (+ J^T W J)
     const double* sumW;    // [ngrids][nbins] summed FP32 node weights (mixed modes)
+    const float2* sumWf;   // the same as float pairs
+    float norm_h, norm_l;  // norm as a float pair
     const int* gid;        // [npts] grid of each point, or NULL: every point uses grid 0
+    int corr;              // mixed modes: v[0] needs the two corrections below (node sums with FP32 weights)
     float wsum_lo;               // exact sum of the FP32 weights - the kernel's constant term
     float om_delta[GNA_NLMAX];   // omega_r - om_r (corrections ~1e-8 relative: FP32 suffices)
     double* chi2;          // [npts]
@@ -103,7 +107,7 @@ __device__ inline void bin_epilogue(const EpiArgs& a, int p, int i, const double
         for (int j = 0; j < a.NV; j++) a.binsums[idx * a.NV + j] = v[j];
     double M = v[0];
     const int off = 1 + (a.has_grad ? 4 : 0);
-    if (!a.is64) {
+    if (a.corr) {
         // exact corrections of the FP32 weights: the constant term of P carries
         // wsum_lo times the bin's summed node weights, and with per-baseline
         // sums the rounding of omega_r is undone with those sums
@@ -191,39 +195,47 @@ __device__ inline void bin_epilogue(const EpiArgs& a, int p, int i, const double
 // two short reductions after the last bin instead of one over all bins.
 // Reads go through L2 (__ldcg): other SMs wrote the values.
 
+// NVP >= NBV: the power of two of values that a transposed reduction takes.
+
 // Group g of point p: lane l holds (regs) or loads (binvals) the values of
-// bin 32 g + l; one transposed reduction; lanes holding value lane / 2 store it.
+// bin 32 g + l; one transposed reduction; the first of the 32 / NVP lanes that
+// end up with a value stores it.
+template <int NVP>
 __device__ inline void group_reduce(const EpiArgs& a, int p, int g, int lane, const float2* regs) {
+    constexpr int SH = NVP == 16 ? 1 : 2;
+    static_assert(NVP == 16 || NVP == 8, "8 or 16 values");
     const int i = (g << 5) + lane;
-    float2 v[16];
+    float2 v[NVP];
     if (regs) {
 #pragma unroll
-        for (int j = 0; j < 16; j++) v[j] = (j < a.NBV && i < a.nbins) ? regs[j] : make_float2(0.f, 0.f);
+        for (int j = 0; j < NVP; j++) v[j] = (j < a.NBV && i < a.nbins) ? regs[j] : make_float2(0.f, 0.f);
     } else {
         const float2* bv = a.binvals + ((int64_t)p * a.nbins + i) * a.NBV;
 #pragma unroll
-        for (int j = 0; j < 16; j++) v[j] = (j < a.NBV && i < a.nbins) ? __ldcg(bv + j) : make_float2(0.f, 0.f);
+        for (int j = 0; j < NVP; j++) v[j] = (j < a.NBV && i < a.nbins) ? __ldcg(bv + j) : make_float2(0.f, 0.f);
     }
-    warp_transpose_reduce<16>(v, lane);
-    const int vi = lane >> 1;
-    if ((lane & 1) == 0 && vi < a.NBV) a.gvals[((int64_t)p * a.ngroups + g) * a.NBV + vi] = v[0];
+    warp_transpose_reduce<NVP>(v, lane);
+    const int vi = lane >> SH;
+    if ((lane & ((1 << SH) - 1)) == 0 && vi < a.NBV) a.gvals[((int64_t)p * a.ngroups + g) * a.NBV + vi] = v[0];
 }
 
 // Point p: lane l sums groups l, l + 32, ... in order, then one transposed
 // reduction over the lanes; the point's outputs are written.
+template <int NVP>
 __device__ inline void point_reduce(const EpiArgs& a, int p, int lane) {
-    float2 v[16];
+    constexpr int SH = NVP == 16 ? 1 : 2;
+    float2 v[NVP];
 #pragma unroll
-    for (int j = 0; j < 16; j++) v[j] = make_float2(0.f, 0.f);
+    for (int j = 0; j < NVP; j++) v[j] = make_float2(0.f, 0.f);
     for (int g = lane; g < a.ngroups; g += 32) {
         const float2* gv = a.gvals + ((int64_t)p * a.ngroups + g) * a.NBV;
 #pragma unroll
-        for (int j = 0; j < 15; j++)
+        for (int j = 0; j < (NVP == 16 ? 15 : 5); j++)
             if (j < a.NBV) v[j] = ff_add(v[j], __ldcg(gv + j));
     }
-    warp_transpose_reduce<16>(v, lane);
-    const int vi = lane >> 1;
-    if ((lane & 1) == 0 && vi < a.NBV) {
+    warp_transpose_reduce<NVP>(v, lane);
+    const int vi = lane >> SH;
+    if ((lane & ((1 << SH) - 1)) == 0 && vi < a.NBV) {
         const double tot = (double)v[0].x + (double)v[0].y;
         if (vi == 0) a.chi2[p] = tot;
         else if (vi < 5) {
@@ -234,15 +246,9 @@ __device__ inline void point_reduce(const EpiArgs& a, int p, int lane) {
     }
 }
 
-// The whole group g of point p has its per-bin values ready (whole warp
-// calls): in regs (each lane its bin's values) or in binvals.  Not inlined:
-// its registers stay out of the node loops' allocation.
-static __device__ __noinline__ void group_done(const EpiArgs& a, int p, int g, int lane, const float2* regs) {
-    if (!regs) {
-        __threadfence();
-        __syncwarp();
-    }
-    group_reduce(a, p, g, lane, regs);
+// A group's sums are stored: the last group of the point sums the groups.
+template <int NVP>
+__device__ __forceinline__ void group_counted(const EpiArgs& a, int p, int lane) {
     // every lane that stored a group value makes it visible before lane 0 counts the group
     __threadfence();
     __syncwarp();
@@ -251,8 +257,25 @@ static __device__ __noinline__ void group_done(const EpiArgs& a, int p, int g, i
     lastp = __shfl_sync(0xffffffffu, lastp, 0);
     if (lastp) {
         __threadfence();
-        point_reduce(a, p, lane);
+        point_reduce<NVP>(a, p, lane);
     }
+}
+
+// The whole group g of point p has its per-bin values ready (whole warp
+// calls): in regs (each lane its bin's values) or in binvals.
+template <int NVP>
+__device__ __forceinline__ void group_finish(const EpiArgs& a, int p, int g, int lane, const float2* regs) {
+    if (!regs) {
+        __threadfence();
+        __syncwarp();
+    }
+    group_reduce<NVP>(a, p, g, lane, regs);
+    group_counted<NVP>(a, p, lane);
+}
+
+// Not inlined: its registers stay out of the node loops' allocation.
+static __device__ __noinline__ void group_done(const EpiArgs& a, int p, int g, int lane, const float2* regs) {
+    group_finish<16>(a, p, g, lane, regs);
 }
 
 // Bin i of point p has its per-bin values stored by lane 0 (whole warp calls).
@@ -266,6 +289,107 @@ __device__ inline void bin_done(const EpiArgs& a, int p, int i, int lane) {
     }
     lastg = __shfl_sync(0xffffffffu, lastg, 0);
     if (lastg) group_done(a, p, g, lane, nullptr);
+}
+
+// ------------------------------------------------ chunk-anchored sums ----
+// The epilogue of the anchored node kernels (anchored.cuh): the same steps on
+// a prediction held as a float pair, without FP64 instructions but the
+// conversions of the inputs (a warp-wide FP64 instruction holds an SM
+// quarter's FP64 pipe for 64 cycles: the double epilogue's thirty took half
+// of a scan task's own cost).  The pairs carry 48 bits, the terms formed from
+// them are FP32 as before.
+
+// Inputs of one bin (loadable before the node sums are ready).
+struct BinInput {
+    float2 d;     // data count
+    float2 sumw;  // summed node weights
+    double e;     // nuisance eta_i (0 without nuisances)
+};
+
+__device__ __forceinline__ BinInput bin_input(const EpiArgs& a, int p, int i) {
+    BinInput in;
+    const double d = a.data[a.data_per_point ? (int64_t)p * a.nbins + i : i];
+    split_ff(d, in.d.x, in.d.y);
+    in.sumw = a.sumWf[(a.gid ? (int64_t)a.gid[p] * a.nbins : 0) + i];
+    in.e = a.eta ? a.eta[i] : 0.0;
+    return in;
+}
+
+struct BinSums {
+    float2 M;    // sum_k W_k sum_r omega_r P_r
+    float v[4];  // tangent sums (their sign applied here)
+};
+
+__device__ __forceinline__ float2 ff_norm(float p, float e) {
+    const float h = __fadd_rn(p, e);
+    return make_float2(h, __fsub_rn(e, __fsub_rn(h, p)));
+}
+
+// Bin (p, i): outputs, and the terms to be summed over bins into regs[0..4]
+// (chi^2, gradient).  sp[r]: what to take from sumw for baseline r's sum (with spectra).
+template <bool GRAD>
+__device__ __forceinline__ void bin_terms(const EpiArgs& a, int p, int i, const BinSums& b, const float2* sp,
+                                          const BinInput& in, float2* regs) {
+    const int64_t idx = (int64_t)p * a.nbins + i;
+    constexpr int off = GRAD ? 3 : 1;
+    if (a.binsums) {
+        // kept as float pairs: M, the tangents two by two, the baselines' parts
+        float2* s = reinterpret_cast<float2*>(a.binsums) + idx * a.NV;
+        s[0] = b.M;
+        if constexpr (GRAD) {
+            s[1] = make_float2(b.v[0], b.v[1]);
+            s[2] = make_float2(b.v[2], b.v[3]);
+        }
+        for (int r = 0; r < a.nspec; r++) s[off + r] = sp[r];
+    }
+    if (a.spectra_out) {
+        const double w = (double)in.sumw.x + (double)in.sumw.y;
+        for (int r = 0; r < a.nspec; r++)
+            a.spectra_out[((int64_t)p * a.nL_out + r) * a.nbins + i] = w - ((double)sp[r].x + (double)sp[r].y);
+    }
+    float fh = a.norm_h, fl = a.norm_l;
+    if (a.eta) split_ff(a.norm * (1.0 + in.e), fh, fl);
+    // mu = f M
+    const float pr = __fmul_rn(fh, b.M.x);
+    const float2 mu = ff_norm(pr, __fmaf_rn(fh, b.M.y, __fmaf_rn(fl, b.M.x, __fmaf_rn(fh, b.M.x, -pr))));
+    const float2 dm = ff_add(in.d, make_float2(-mu.x, -mu.y));  // d and mu are close
+    const float tf = dm.x / mu.x;                               // relative residual, 1e-7 is enough
+    float g;
+    float2 term;
+    if (a.kind == GNA_PEARSON) {
+        const float t = __fmul_rn(dm.x, tf);  // (d - mu)^2 / mu
+        term = make_float2(t, __fmaf_rn(dm.y, tf, __fmaf_rn(dm.x, tf, -t)));
+        g = 1.0f - (1.0f + tf) * (1.0f + tf);  // 1 - d^2 / mu^2
+    } else {
+        const float h2 = in.d.x > 0.f ? 2.0f * poisson_h(tf) : 2.0f;
+        const float t = __fmul_rn(h2, mu.x);
+        term = make_float2(t, __fmaf_rn(h2, mu.y, __fmaf_rn(h2, mu.x, -t)));
+        g = -2.0f * tf;  // 2 (1 - d / mu)
+    }
+    const bool pen = a.penalty != 0;
+    if (pen) term = ff_add(term, to_ff(in.e * in.e / (a.sigma * a.sigma)));
+    regs[0] = term;
+    if constexpr (GRAD) {
+#pragma unroll
+        for (int q = 0; q < 4; q++) regs[1 + q] = make_float2(g * (-fh * b.v[q]), 0.f);
+    }
+    if (a.mu_out) a.mu_out[idx] = (double)mu.x + (double)mu.y;
+    if (a.grad_eta_out)
+        a.grad_eta_out[idx] = (double)g * a.norm * ((double)b.M.x + (double)b.M.y) + (pen ? 2.0 * in.e / (a.sigma * a.sigma) : 0.0);
+}
+
+// The group's sums of at most five values in registers, and group_done for them.
+template <bool GRAD>
+__device__ __forceinline__ void group_terms(const EpiArgs& a, int p, int g, int lane, const float2 (&regs)[5]) {
+    float2 r[8];
+#pragma unroll
+    for (int j = 0; j < 8; j++) r[j] = j < (GRAD ? 5 : 1) ? regs[j < 5 ? j : 0] : make_float2(0.f, 0.f);
+    group_reduce<8>(a, p, g, lane, r);
+}
+template <bool GRAD>
+__device__ __forceinline__ void group_done_terms(const EpiArgs& a, int p, int g, int lane, const float2 (&regs)[5]) {
+    group_terms<GRAD>(a, p, g, lane, regs);
+    group_counted<8>(a, p, lane);
 }
 
 }  // namespace gna

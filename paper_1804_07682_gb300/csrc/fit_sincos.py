@@ -1,6 +1,8 @@
 """Generate ff_consts.h: FP32 polynomial coefficients for sin and cos on the
 reduced range |r| <= pi/2 (+ margin) and a 3-part split of pi for the
-Cody-Waite reduction of the oscillation phase modulo pi.
+Cody-Waite reduction of the oscillation phase modulo pi; and the coefficients
+for the chunk-anchored node loops, whose argument is an anchor's phase reduced
+modulo pi (modulo pi/2: the any-channel sums) plus a node's small offset.
 
 Method: weighted least squares on Chebyshev-distributed points, iterated with
 Lawson's reweighting toward the minimax solution, for
@@ -20,6 +22,9 @@ import numpy as np
 R_MAX = math.pi / 2 + 2e-3
 N_SIN = 4  # S1..S4: odd degree 9 (error ~5e-9)
 N_COS = 4  # C1..C4: even degree 8 (error ~5e-8)
+# chunk-anchored loops: (suffix, range, sine terms, cosine terms); the ranges
+# are the reduced anchor's plus the largest offset the kernels allow (anchored.cuh)
+ANCHORED = (("A", math.pi / 2 + 0.25 + 1e-3, 4, 5), ("Q", math.pi / 4 + 0.15 + 1e-3, 3, 4))
 
 # pi to 60 digits (textbook value)
 PI = Fraction("3.14159265358979323846264338327950288419716939937510582097494")
@@ -52,7 +57,7 @@ def fit_sequential(basis, target, weight):
     return np.array(fixed)
 
 
-def fit():
+def fit(R_MAX=R_MAX, N_SIN=N_SIN, N_COS=N_COS):
     t = np.cos(np.linspace(0, np.pi, 6001))  # Chebyshev points on [-1, 1]
     r = 0.5 * (t + 1) * R_MAX
     r = r[r > 1e-3]
@@ -134,6 +139,17 @@ def main():
         out.write("#define GNA_SIN_C%d (%.9ef)\n" % (k + 1, float(c)))
     for k, c in enumerate(cc32):
         out.write("#define GNA_COS_C%d (%.9ef)\n" % (k + 1, float(c)))
+    for suffix, rmax, ns, nc in ANCHORED:
+        ks, kc = fit(rmax, ns, nc)
+        r = np.linspace(-rmax, rmax, 200001)
+        u = r * r
+        e_s = np.abs(r + r * u * sum(float(c) * u ** k for k, c in enumerate(ks)) - np.sin(r)).max()
+        e_c = np.abs(1 + u * sum(float(c) * u ** k for k, c in enumerate(kc)) - np.cos(r)).max()
+        out.write("// Chunk-anchored loops, |r| <= %.6f: polynomial error sin %.2e, cos %.2e.\n" % (rmax, e_s, e_c))
+        for k, c in enumerate(ks):
+            out.write("#define GNA_SIN%s_C%d (%.9ef)\n" % (suffix, k + 1, float(c)))
+        for k, c in enumerate(kc):
+            out.write("#define GNA_COS%s_C%d (%.9ef)\n" % (suffix, k + 1, float(c)))
     out.write("// pi = PI_A + PI_B + PI_C; PI_A and PI_B have 12 significant bits.\n")
     out.write("#define GNA_PI_A (%.17gf)\n" % A)
     out.write("#define GNA_PI_B (%.17gf)\n" % B)

@@ -278,20 +278,57 @@ __global__ void __launch_bounds__(256, GNA_SPLIT_MIN_BLOCKS) k_fused_split(Split
 }
 
 // ---------------------------------------------------------------------------
-// Bin mapping: a warp task is (point p, group b of 32 consecutive bins); lane
-// l owns bin 32 b + l and walks its nodes (grid layout [group][k][lane], so
-// each warp load is 512 contiguous bytes, the next one prefetched).  Each
-// lane finishes its own bin; the warp sums its group and the last group of a
-// point sums the groups.  Warps take tasks from a global counter; tasks are
-// ordered by decreasing node count so that uneven grids balance.
+// Bin mapping (node kernels in anchored.cuh, general.cuh, and for the fits
+// below): a warp task is (point p, group b of 32 consecutive bins); lane l owns
+// bin 32 b + l and walks its nodes.  Each lane finishes its own bin; the warp
+// sums its group and the last group of a point sums the groups.  Warps take
+// tasks from a global counter; tasks are ordered by decreasing node count so
+// that uneven grids balance.
 //
-// Slice mapping (S > 1, one grid shared by all points): the same kernel with
+// Slice mapping (S > 1, one grid shared by all points): the same kernels with
 // each group's nodes cut into S slices of L nodes; task t = (p, b, s) in
 // that order.  A lane keeps its own bin's sums for its slice and stores them
-// as float pairs; k_slices_reduce then sums the slices in order and runs the
+// as float pairs; a second kernel then sums the slices in order and runs the
 // epilogue.  Unlike the split mapping no warp reduction or counter is needed
 // per node range, and the node loop is the same as for whole bins.
+
+// A whole-bin task of the anchored kernels.
+struct BinTask {
+    int p, b, nq;  // point, group, quads of nodes
+    float step;    // largest step of 1/E between neighbouring nodes
+    int64_t quad;  // first quad in the plan's records
+};
+
 struct BinArgs {
+    const float4* grid;   // nodes (general.cuh)
+    const char* rec;      // quads of nodes (anchored.cuh)
+    const int64_t* goff;  // [ngrids] first node of each grid
+    const int* gn;        // [ngrids] Gauss-Legendre order of each grid
+    const int* gid;       // [npts] grid of each point, or NULL: every point uses grid 0
+    const int* tasks;     // [ntasks] p * ngroups + b, in execution order
+    const BinTask* desc;  // [ntasks] the same for the anchored kernels
+    int ntasks, ngroups, nbins;
+    const PointConst* pcs;
+    BaseConst bc;
+    int* counter;  // zeroed before the launch
+    EpiArgs ea;
+    int S, L;      // slices per group and nodes (anchored: quads) per slice (S = 1: whole bins)
+    float2* part;  // slice values [ntasks][NVs][32] (S > 1)
+    int NVs;       // values per slice and bin
+    int nL, spec;  // baselines, per-baseline sums requested
+    const float* step;  // [ngrids][ngroups] largest step of 1/E between neighbouring nodes
+};
+
+// The fits' node kernel (grid layout [group][node][lane], each warp load 512
+// contiguous bytes, the next one prefetched): every node's phases are reduced
+// by themselves and P is formed per node.  Levenberg-Marquardt trajectories
+// amplify any change of rounding -- a trial is accepted when its chi^2 is
+// lower, and from a start far from the minimum single data sets end in
+// another valley (the 64-bit restatement of a batch of 2048 disagreed with it
+// in 0.6 of the norm of chi^2 where one data set did) -- so the fits keep the
+// evaluation whose trajectories users have seen, and the anchored kernels
+// serve everything else.
+struct FitArgs {
     const float4* grid;
     const int64_t* goff;  // [ngrids] float4 offset of each grid
     const int* gn;        // [ngrids] Gauss-Legendre order of each grid
@@ -306,9 +343,10 @@ struct BinArgs {
     float2* part;  // slice values [ntasks][NV][32] (S > 1)
 };
 
-template <int PH, int NL, bool GRAD, bool SPEC>
-__global__ void __launch_bounds__(256) k_fused_bins(BinArgs a) {
-    using M = NodeMath<PH, NL, GRAD, SPEC>;
+template <int PH, int NL>
+__global__ void __launch_bounds__(256) k_fit_bins(FitArgs a) {
+    constexpr bool GRAD = true;
+    using M = NodeMath<PH, NL, GRAD, false>;
     constexpr int NV = M::NV;
     const int lane = threadIdx.x & 31;
     int last_p = -1;
@@ -400,11 +438,11 @@ __global__ void __launch_bounds__(256) k_fused_bins(BinArgs a) {
 // (the kernel preparing the constants): the node kernel's launch and block
 // placement overlap it; the kernel waits with griddepcontrol.wait.
 template <typename Kernel, typename Args>
-cudaError_t launch_dependent(Kernel k, const Args& a, int grid, int block, cudaStream_t s) {
+cudaError_t launch_dependent(Kernel k, const Args& a, int grid, int block, cudaStream_t s, size_t smem = 0) {
     cudaLaunchConfig_t cfg{};
     cfg.gridDim = dim3((unsigned)grid);
     cfg.blockDim = dim3((unsigned)block);
-    cfg.dynamicSmemBytes = 0;
+    cfg.dynamicSmemBytes = smem;
     cfg.stream = s;
     cudaLaunchAttribute at[1];
     at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
@@ -419,9 +457,9 @@ cudaError_t launch_split(const SplitArgs& a, int grid, int block, cudaStream_t s
     return launch_dependent(k_fused_split<PH, NL, GRAD, SPEC>, a, grid, block, s);
 }
 
-template <int PH, int NL, bool GRAD, bool SPEC>
-cudaError_t launch_bins(const BinArgs& a, int grid, int block, cudaStream_t s) {
-    return launch_dependent(k_fused_bins<PH, NL, GRAD, SPEC>, a, grid, block, s);
+template <int PH, int NL>
+cudaError_t launch_fit_bins(const FitArgs& a, int grid, int block, cudaStream_t s) {
+    return launch_dependent(k_fit_bins<PH, NL>, a, grid, block, s);
 }
 
 // Number of values per (point, bin) for the given flags.

@@ -1,4 +1,4 @@
-// fused_f64ph.cu -- explicit instantiations of the fused kernels with the double-precision phase, for 1, 8 and 16 baselines.
+// fused_f64ph.cu -- explicit instantiations of the split-mapping and fit kernels with the double-precision phase, for 1, 8 and 16 baselines.
 #include "dispatch.h"
 #include "fused.cuh"
 namespace gna {
@@ -21,22 +21,11 @@ cudaError_t dispatch_split_ph1(int nl, bool grad, bool spec, const void* args, i
         default: return cudaErrorInvalidValue;
     }
 }
-cudaError_t dispatch_bins_ph1(int nl, bool grad, bool spec, const void* args, int grid, int block, cudaStream_t s) {
-    const BinArgs& a = *static_cast<const BinArgs*>(args);
-    const int key = nl * 4 + (grad ? 2 : 0) + (spec ? 1 : 0);
-    switch (key) {
-        case 4: return launch_bins<1, 1, false, false>(a, grid, block, s);
-        case 5: return launch_bins<1, 1, false, true>(a, grid, block, s);
-        case 6: return launch_bins<1, 1, true, false>(a, grid, block, s);
-        case 7: return launch_bins<1, 1, true, true>(a, grid, block, s);
-        case 32: return launch_bins<1, 8, false, false>(a, grid, block, s);
-        case 33: return launch_bins<1, 8, false, true>(a, grid, block, s);
-        case 34: return launch_bins<1, 8, true, false>(a, grid, block, s);
-        case 35: return launch_bins<1, 8, true, true>(a, grid, block, s);
-        case 64: return launch_bins<1, 16, false, false>(a, grid, block, s);
-        case 65: return launch_bins<1, 16, false, true>(a, grid, block, s);
-        case 66: return launch_bins<1, 16, true, false>(a, grid, block, s);
-        case 67: return launch_bins<1, 16, true, true>(a, grid, block, s);
+cudaError_t dispatch_fit_ph1(int nl, const FitArgs& a, int grid, int block, cudaStream_t s) {
+    switch (nl) {
+        case 1: return launch_fit_bins<1, 1>(a, grid, block, s);
+        case 8: return launch_fit_bins<1, 8>(a, grid, block, s);
+        case 16: return launch_fit_bins<1, 16>(a, grid, block, s);
         default: return cudaErrorInvalidValue;
     }
 }

@@ -1,4 +1,4 @@
-// fused_ff.cu -- explicit instantiations of the fused kernels with the double-float phase, for 1, 2, 4, 8 and 16 baselines.
+// fused_ff.cu -- explicit instantiations of the split-mapping and fit kernels with the double-float phase, for 1, 2, 4, 8 and 16 baselines.
 #include "dispatch.h"
 #include "fused.cuh"
 namespace gna {
@@ -29,30 +29,13 @@ cudaError_t dispatch_split_ph0(int nl, bool grad, bool spec, const void* args, i
         default: return cudaErrorInvalidValue;
     }
 }
-cudaError_t dispatch_bins_ph0(int nl, bool grad, bool spec, const void* args, int grid, int block, cudaStream_t s) {
-    const BinArgs& a = *static_cast<const BinArgs*>(args);
-    const int key = nl * 4 + (grad ? 2 : 0) + (spec ? 1 : 0);
-    switch (key) {
-        case 4: return launch_bins<0, 1, false, false>(a, grid, block, s);
-        case 5: return launch_bins<0, 1, false, true>(a, grid, block, s);
-        case 6: return launch_bins<0, 1, true, false>(a, grid, block, s);
-        case 7: return launch_bins<0, 1, true, true>(a, grid, block, s);
-        case 8: return launch_bins<0, 2, false, false>(a, grid, block, s);
-        case 9: return launch_bins<0, 2, false, true>(a, grid, block, s);
-        case 10: return launch_bins<0, 2, true, false>(a, grid, block, s);
-        case 11: return launch_bins<0, 2, true, true>(a, grid, block, s);
-        case 16: return launch_bins<0, 4, false, false>(a, grid, block, s);
-        case 17: return launch_bins<0, 4, false, true>(a, grid, block, s);
-        case 18: return launch_bins<0, 4, true, false>(a, grid, block, s);
-        case 19: return launch_bins<0, 4, true, true>(a, grid, block, s);
-        case 32: return launch_bins<0, 8, false, false>(a, grid, block, s);
-        case 33: return launch_bins<0, 8, false, true>(a, grid, block, s);
-        case 34: return launch_bins<0, 8, true, false>(a, grid, block, s);
-        case 35: return launch_bins<0, 8, true, true>(a, grid, block, s);
-        case 64: return launch_bins<0, 16, false, false>(a, grid, block, s);
-        case 65: return launch_bins<0, 16, false, true>(a, grid, block, s);
-        case 66: return launch_bins<0, 16, true, false>(a, grid, block, s);
-        case 67: return launch_bins<0, 16, true, true>(a, grid, block, s);
+cudaError_t dispatch_fit_ph0(int nl, const FitArgs& a, int grid, int block, cudaStream_t s) {
+    switch (nl) {
+        case 1: return launch_fit_bins<0, 1>(a, grid, block, s);
+        case 2: return launch_fit_bins<0, 2>(a, grid, block, s);
+        case 4: return launch_fit_bins<0, 4>(a, grid, block, s);
+        case 8: return launch_fit_bins<0, 8>(a, grid, block, s);
+        case 16: return launch_fit_bins<0, 16>(a, grid, block, s);
         default: return cudaErrorInvalidValue;
     }
 }

@@ -129,6 +129,7 @@ __global__ void k_prepare_general(const gna_osc_full* __restrict__ prm, int npts
     split_ff(c21, pc.c21h[r], pc.c21l[r]);
     split_ff(c32, pc.c32h[r], pc.c32l[r]);
     if (r != 0) return;
+    pc.cmax = largest_phase(bc, o.dm2_21, o.dm2_32);
     const bool inside = o.s2_12 > 0.0 && o.s2_12 < 1.0 && o.s2_13 > 0.0 && o.s2_13 < 1.0 && o.s2_23 > 0.0 &&
                         o.s2_23 < 1.0 && isfinite(o.delta_cp) && isfinite(o.dm2_21) && isfinite(o.dm2_32);
     if (!inside && status) atomicExch(status, (int)GNA_EINVAL);

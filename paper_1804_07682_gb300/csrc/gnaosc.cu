@@ -16,6 +16,7 @@
 #include <string>
 #include <vector>
 
+#include "anchored.cuh"
 #include "common.cuh"
 #include "dispatch.h"
 #include "fused.cuh"
@@ -28,11 +29,15 @@ using namespace gna;
 
 namespace gna {
 cudaError_t dispatch_split_ph0(int, bool, bool, const void*, int, int, cudaStream_t);
-cudaError_t dispatch_bins_ph0(int, bool, bool, const void*, int, int, cudaStream_t);
 cudaError_t dispatch_split_ph1(int, bool, bool, const void*, int, int, cudaStream_t);
-cudaError_t dispatch_bins_ph1(int, bool, bool, const void*, int, int, cudaStream_t);
 cudaError_t dispatch_split_ph2(int, bool, bool, const void*, int, int, cudaStream_t);
 cudaError_t dispatch_bins_ph2(int, bool, bool, const void*, int, int, cudaStream_t);
+cudaError_t dispatch_fit_ph0(int, const FitArgs&, int, int, cudaStream_t);
+cudaError_t dispatch_fit_ph1(int, const FitArgs&, int, int, cudaStream_t);
+cudaError_t dispatch_nodes_ph0(bool, const BinArgs&, int, int, cudaStream_t);
+cudaError_t dispatch_nodes_ph1(bool, const BinArgs&, int, int, cudaStream_t);
+int nodes_resident_ctas_ph0(int, bool, int);
+int nodes_resident_ctas_ph1(int, bool, int);
 int split_regs_ph0(int, bool, bool);
 int split_regs_ph1(int, bool, bool);
 int split_regs_ph2(int, bool, bool);
@@ -42,10 +47,15 @@ cudaError_t dispatch_split(int ph, int nl, bool grad, bool spec, const void* arg
     if (ph == 1) return dispatch_split_ph1(nl, grad, spec, args, grid, block, s);
     return dispatch_split_ph2(nl, grad, spec, args, grid, block, s);
 }
-cudaError_t dispatch_bins(int ph, int nl, bool grad, bool spec, const void* args, int grid, int block, cudaStream_t s) {
-    if (ph == 0) return dispatch_bins_ph0(nl, grad, spec, args, grid, block, s);
-    if (ph == 1) return dispatch_bins_ph1(nl, grad, spec, args, grid, block, s);
-    return dispatch_bins_ph2(nl, grad, spec, args, grid, block, s);
+cudaError_t dispatch_nodes(int ph, bool grad, const BinArgs& a, int grid, int block, cudaStream_t s) {
+    return ph == 0 ? dispatch_nodes_ph0(grad, a, grid, block, s) : dispatch_nodes_ph1(grad, a, grid, block, s);
+}
+cudaError_t dispatch_fit(int ph, int nl, const FitArgs& a, int grid, int block, cudaStream_t s) {
+    return ph == 0 ? dispatch_fit_ph0(nl, a, grid, block, s) : dispatch_fit_ph1(nl, a, grid, block, s);
+}
+int nodes_block(int block) { return std::min(block, 128); }
+int nodes_resident_ctas(int ph, int nL, bool grad, int block) {
+    return ph == 0 ? nodes_resident_ctas_ph0(nL, grad, block) : nodes_resident_ctas_ph1(nL, grad, block);
 }
 int split_regs(int ph, int nl, bool grad, bool spec) {
     if (ph == 0) return split_regs_ph0(nl, grad, spec);
@@ -102,6 +112,10 @@ struct gna_plan {
     bool has_split = false, has_bins = false;
     float4* grid_split = nullptr;
     float4* grid_bins = nullptr;
+    // quads of nodes for the anchored kernels (survival chain, mixed precisions,
+    // bin and slice mappings), and their whole-bin tasks
+    char* grid_rec = nullptr;
+    BinTask* d_desc = nullptr;
     double2* grid64_split = nullptr;
     double2* grid64_bins = nullptr;
     double2* plain64 = nullptr;
@@ -112,6 +126,8 @@ struct gna_plan {
     int ngrids = 0, ngroups = 0;
     int* d_tasks = nullptr;
     int ntasks = 0;
+    float* d_step = nullptr;  // [ngrids][ngroups] largest step of 1/E between neighbouring nodes
+    int res_ctas[2] = {0, 0}, res_block[2] = {0, 0};  // resident blocks per SM of the node kernel (without, with gradient)
     // [1 + npts + npts*ngroups (+ npts*nbins, split)]: work counter, groups
     // finished per point, bins finished per group, segments finished per bin
     int* d_counters = nullptr;
@@ -130,7 +146,7 @@ struct gna_plan {
     float2* d_gvals = nullptr;  // [npts][ngroups][15] group sums
     // per-bin node sums of the last evaluation, for epilogue-only re-evaluations
     double* d_binsums = nullptr;  // [npts][nbins][nv_max], or NULL (too large)
-    bool cache_valid = false, cache_grad = false, cache_spec = false;
+    bool cache_valid = false, cache_grad = false, cache_spec = false, cache_split = false;
     double* d_H = nullptr;
     double* d_chi2_tmp = nullptr;
     double* d_grad_tmp = nullptr;
@@ -150,6 +166,7 @@ struct gna_plan {
     // launch shape
     int block = kDefaultBlock, npt = kDefaultNodesPerThread, grid_mult = 0;
     int slice_len = 0;  // slice mapping: nodes per slice (0: chosen from the GPU size)
+    int64_t auto_warps = 0, auto_len = 0;  // the chosen length and the resident warps it was chosen for
     // graphs
     bool use_graph = false;
     cudaGraphExec_t gexec = nullptr;
@@ -195,6 +212,7 @@ struct gna_plan {
     cudaStream_t cp_in = nullptr, cp_out = nullptr;
     size_t in_cap = 0, out_cap = 0;
     double* d_sumW = nullptr;  // [ngrids][nbins]
+    float2* d_sumWf = nullptr;  // the same as float pairs
     double wsum_all_lo = 0.0;  // sum_r (om_r + omlo_r) - wsum: constant term when the weights enter as hi + lo
     // graphs are captured on a plan-owned stream joined to the caller's by events
     cudaStream_t cap_stream = nullptr;
@@ -277,50 +295,84 @@ SplitShape split_shape(const gna_plan* p, bool grad, bool spec) {
 }
 
 
-int value_count(const gna_plan* p, bool grad, bool spec) { return fused_nv(p->nl_inst, grad, spec); }
+// Per-baseline values of one bin's node sums: the split kernels (and
+// GNA_FP64) sum every instantiated baseline, the anchored kernels those of the plan.
+int spectra_count(const gna_plan* p, bool split) { return (split || p->ph == 2) ? p->nl_inst : p->nL; }
+int value_count(const gna_plan* p, bool grad, bool spec, bool split) {
+    return fused_nv(spectra_count(p, split), grad, spec);
+}
 
 int resident_ctas_per_sm(const gna_plan* p, bool grad, bool spec) {
     int per_sm = std::max(1, 1024 / p->block);
-    if (p->mapping == MAP_SPLIT) {
-        const int regs = split_regs(p->ph, p->nl_inst, grad, spec);
-        if (regs > 0) {
-            const int alloc = ((std::max(regs, 32) + 7) / 8) * 8;  // registers are allocated in units of 8
-            per_sm = std::max(1, std::min(65536 / (alloc * p->block), 2048 / p->block));
-        }
+    const int regs = split_regs(p->ph, p->nl_inst, grad, spec);
+    if (regs > 0) {
+        const int alloc = ((std::max(regs, 32) + 7) / 8) * 8;  // registers are allocated in units of 8
+        per_sm = std::max(1, std::min(65536 / (alloc * p->block), 2048 / p->block));
     }
     if (p->grid_mult > 0) per_sm = p->grid_mult;
     return per_sm;
 }
 
+// Resident blocks per SM of the node kernel of the bin and slice mappings
+// (asked of the runtime once per block size).
+int node_ctas_per_sm(gna_plan* p, bool grad, bool surv, int block) {
+    if (p->grid_mult > 0) return p->grid_mult;
+    int& n = p->res_ctas[grad];
+    if (n == 0 || p->res_block[grad] != block) {
+        n = p->general ? general_resident_ctas(p->ph, p->nl_inst, grad, surv, block)
+            : p->ph < 2 ? nodes_resident_ctas(p->ph, p->nL, grad, block)
+                        : std::max(1, 1024 / block);
+        p->res_block[grad] = block;
+    }
+    return n;
+}
+
 // Persistent grid size of the bin mapping (warp-sized work items).
-int grid_size(const gna_plan* p, bool grad, bool spec, int64_t work_items) {
-    int64_t g = (int64_t)p->sm_count * resident_ctas_per_sm(p, grad, spec);
-    g = std::min<int64_t>(g, (work_items * 32 + p->block - 1) / p->block);
+int grid_size(const gna_plan* p, int ctas_per_sm, int block, int64_t work_items) {
+    int64_t g = (int64_t)p->sm_count * ctas_per_sm;
+    g = std::min<int64_t>(g, (work_items * 32 + block - 1) / block);
     return (int)std::max<int64_t>(1, g);
 }
 
-// Slice mapping: S slices of L nodes per group of 32 bins.  The default L
-// gives about two tasks per resident warp (estimate: 16 warps per SM), so
-// that the task counter can even out the warps the schedulers favour.
+// Slice mapping: S slices of L nodes per group of 32 bins.  All tasks take
+// the same time, so the default S is the one whose last round of tasks over
+// the resident warps wastes least: rounds x (nodes of a slice + a task's own
+// cost in nodes).
 struct SliceShape {
     int S, L, ntasks;
 };
 
-SliceShape slice_shape(const gna_plan* p) {
+SliceShape slice_shape(gna_plan* p, int64_t resident_warps) {
     const int n = p->n_uniform;
     const int64_t pg = (int64_t)p->npts * p->ngroups;
+    const int64_t cap = std::max(1, p->slices_cap);
     int64_t L = p->slice_len;
-    if (L <= 0) {
-        const int64_t target = 2LL * 16 * p->sm_count;
-        const int64_t S = std::max<int64_t>(1, (target + pg - 1) / pg);
-        L = (n + S - 1) / S;
+    if (L <= 0 && p->auto_warps == resident_warps) {
+        L = p->auto_len;
+    } else if (L <= 0) {
+        constexpr int64_t kTaskCost = 6, kReduceCost = 16;
+        int64_t best = -1;
+        L = n;
+        for (int64_t S = 1; S <= cap; S++) {
+            const int64_t len = (n + S - 1) / S, used = (n + len - 1) / len;
+            if (used != S) continue;  // same length as a smaller S
+            const int64_t rounds = (pg * S + resident_warps - 1) / resident_warps;
+            const int64_t cost = rounds * (len + kTaskCost) + (S > 1 ? kReduceCost : 0);
+            if (best < 0 || cost < best) {
+                best = cost;
+                L = len;
+            }
+            if (pg * S > 8 * resident_warps) break;
+        }
+        p->auto_warps = resident_warps;
+        p->auto_len = L;
     }
-    if (p->slices_cap <= 1) L = n;
-    else L = std::max<int64_t>(L, (n + p->slices_cap - 1) / p->slices_cap);
+    if (cap <= 1) L = n;
+    else L = std::max<int64_t>(L, (n + cap - 1) / cap);
     L = std::min<int64_t>(std::max<int64_t>(L, 1), n);
     SliceShape sh;
-    sh.L = (int)L;
-    sh.S = (int)((n + L - 1) / L);
+    sh.L = (int)(L + 3) & ~3;  // whole quads of nodes
+    sh.S = (int)((n + sh.L - 1) / sh.L);
     sh.ntasks = (int)(pg * sh.S);
     return sh;
 }
@@ -342,12 +394,15 @@ struct EvalReq {
 
 // Epilogue arguments of one evaluation (outputs of q; NV node sums per bin
 // laid out for the grad / spec flags).
-EpiArgs make_epi(const gna_plan* plan, const EvalReq& q, bool grad, bool spec, int NV) {
+EpiArgs make_epi(const gna_plan* plan, const EvalReq& q, bool grad, bool spec, int NV, bool split) {
     EpiArgs ea{};
     ea.is64 = plan->ph == 2;
+    // the split kernel's mixed node sums carry the FP32 weights' rounding; the
+    // anchored kernels' are formed without it
+    ea.corr = plan->ph < 2 && split;
     ea.NV = NV;
     ea.has_grad = grad;
-    ea.nspec = spec ? plan->nl_inst : 0;
+    ea.nspec = spec ? spectra_count(plan, split) : 0;
     ea.nL_out = plan->nL;
     ea.npts = plan->npts;
     ea.nbins = plan->nbins;
@@ -355,6 +410,7 @@ EpiArgs make_epi(const gna_plan* plan, const EvalReq& q, bool grad, bool spec, i
     ea.kind = plan->kind;
     ea.eta = q.eta;
     ea.sigma = q.sigma;
+    ea.penalty = q.eta && q.sigma > 0.0;
     ea.data = q.data;
     ea.data_per_point = q.dpp;
     ea.mu_out = q.mu;
@@ -363,6 +419,8 @@ EpiArgs make_epi(const gna_plan* plan, const EvalReq& q, bool grad, bool spec, i
     ea.binvals = plan->d_binvals;
     ea.NBV = q.H ? 15 : (grad ? 5 : 1);
     ea.sumW = plan->d_sumW;
+    ea.sumWf = plan->d_sumWf;
+    split_ff(plan->norm, ea.norm_h, ea.norm_l);
     ea.gid = plan->d_gid;
     // the kernel's constant term is wsum; the exact one is sum_r om_r when the
     // per-baseline sums carry the weight correction (or one baseline), else
@@ -381,22 +439,69 @@ EpiArgs make_epi(const gna_plan* plan, const EvalReq& q, bool grad, bool spec, i
     return ea;
 }
 
+// Slice mapping of the fits and the any-channel chain: a slice length for
+// about two tasks per resident warp (16 per SM).
+SliceShape fixed_slice_shape(const gna_plan* p) {
+    const int n = p->n_uniform;
+    const int64_t pg = (int64_t)p->npts * p->ngroups;
+    int64_t L = p->slice_len;
+    if (L <= 0) {
+        const int64_t target = 2LL * 16 * p->sm_count;
+        const int64_t S = std::max<int64_t>(1, (target + pg - 1) / pg);
+        L = (n + S - 1) / S;
+    }
+    if (p->slices_cap <= 1) L = n;
+    else L = std::max<int64_t>(L, (n + p->slices_cap - 1) / p->slices_cap);
+    L = std::min<int64_t>(std::max<int64_t>(L, 1), n);
+    SliceShape sh;
+    sh.L = (int)L;
+    sh.S = (int)((n + L - 1) / L);
+    sh.ntasks = (int)(pg * sh.S);
+    return sh;
+}
+
+// The node pass of one fit iteration (mixed precisions, bin and slice
+// mappings; the constants and counters are prepared).
+gna_status enqueue_fit_nodes(gna_plan* plan, const EpiArgs& ea, cudaStream_t s, int* nl) {
+    SliceShape ssh{1, 0, plan->ntasks};
+    if (plan->mapping == MAP_SLICES) {
+        ssh = fixed_slice_shape(plan);
+        if ((int64_t)plan->npts * plan->ngroups * ssh.S >= (1LL << 31)) return fail(plan, GNA_ESHAPE, "too many slice tasks");
+    }
+    const bool sliced = ssh.S > 1;
+    const int per_sm = plan->grid_mult > 0 ? plan->grid_mult : std::max(1, 1024 / plan->block);
+    FitArgs a{plan->grid_bins, plan->d_goff, plan->d_gn, plan->d_gid, plan->d_tasks, ssh.ntasks,
+              plan->ngroups, plan->nbins, plan->d_pc, plan->bc, plan->d_counters, ea,
+              ssh.S, ssh.L, sliced ? plan->d_slices : nullptr};
+    CU(dispatch_fit(plan->ph, plan->nl_inst, a, grid_size(plan, per_sm, plan->block, ssh.ntasks), plan->block, s));
+    if (sliced) {
+        CU(launch_fit_slices_reduce(plan->d_slices, ssh.S, ea, plan->npts, s));
+        (*nl)++;
+    }
+    return GNA_OK;
+}
+
 // Enqueue one fused evaluation; counts kernel launches into *launches.
 gna_status enqueue_eval(gna_plan* plan, const EvalReq& q, cudaStream_t s, int* launches) {
     const bool grad = q.grad || q.grad_eta || q.H;
     const bool spec = q.spectra != nullptr;
+    const bool split = plan->mapping == MAP_SPLIT;
+    const bool fit = q.H && plan->ph < 2 && !split;  // the fits' own node kernel (fused.cuh)
+    const bool plain_sums = split || fit;
     int nl = 0;
-    const int NV = value_count(plan, grad, spec);
+    const int NV = value_count(plan, grad, spec, plain_sums);
     SplitShape sh{};
-    if (plan->mapping == MAP_SPLIT) {
+    if (split) {
         sh = split_shape(plan, grad, spec);
         if ((size_t)plan->npts * plan->nbins * sh.maxseg * NV > plan->part_cap)
             return fail(plan, GNA_ESHAPE, "launch shape needs %lld partials, capacity %zu",
                         (long long)plan->npts * plan->nbins * sh.maxseg * NV, plan->part_cap);
     }
     SliceShape ssh{1, 0, plan->ntasks};
-    if (plan->mapping == MAP_SLICES) {
-        ssh = slice_shape(plan);
+    const int nblock = plan->ph < 2 ? nodes_block(plan->block) : plan->block;
+    const int ctas = split ? 0 : node_ctas_per_sm(plan, grad, false, nblock);
+    if (plan->mapping == MAP_SLICES && !fit) {
+        ssh = slice_shape(plan, (int64_t)plan->sm_count * ctas * (nblock / 32));
         if ((int64_t)plan->npts * plan->ngroups * ssh.S >= (1LL << 31)) return fail(plan, GNA_ESHAPE, "too many slice tasks");
     }
     // work counter, per-point and per-bin arrival counters: zeroed by the
@@ -405,7 +510,7 @@ gna_status enqueue_eval(gna_plan* plan, const EvalReq& q, cudaStream_t s, int* l
                          (plan->mapping == MAP_SPLIT ? (int64_t)plan->npts * plan->nbins : 0);
     CU(launch_prepare(q.params, plan->npts, plan->bc, plan->d_pc, s, plan->d_counters, ncnt, plan->d_status));
     nl++;
-    EpiArgs ea = make_epi(plan, q, grad, spec, NV);
+    EpiArgs ea = make_epi(plan, q, grad, spec, NV, plain_sums);
     // keep the node sums for epilogue-only re-evaluations (not in fits)
     ea.binsums = q.H ? nullptr : plan->d_binsums;
     cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
@@ -425,27 +530,27 @@ gna_status enqueue_eval(gna_plan* plan, const EvalReq& q, cudaStream_t s, int* l
                           plan->d_pc, plan->bc, (double*)plan->d_part, ea};
             CU(dispatch_split(2, plan->nl_inst, grad, spec, &a, sh.grid, plan->block, s));
         }
-    } else if (plan->mapping == MAP_SLICES) {
-        const int g = grid_size(plan, grad, spec, ssh.ntasks);
-        const bool sliced = ssh.S > 1;
-        BinArgs a{plan->grid_bins, plan->d_goff, plan->d_gn, plan->d_gid, plan->d_tasks, ssh.ntasks,
-                  plan->ngroups, plan->nbins, plan->d_pc, plan->bc, plan->d_counters, ea,
-                  ssh.S, ssh.L, sliced ? plan->d_slices : nullptr};
-        CU(dispatch_bins(plan->ph, plan->nl_inst, grad, spec, &a, g, plan->block, s));
-        if (sliced) {
-            CU(launch_slices_reduce(plan->d_slices, ssh.S, NV, ea, plan->npts, s));
-            nl++;
-        }
+    } else if (fit) {
+        TRY(enqueue_fit_nodes(plan, ea, s, &nl));
     } else {
-        const int g = grid_size(plan, grad, spec, plan->ntasks);
+        const int g = grid_size(plan, ctas, nblock, ssh.ntasks);
         if (plan->ph < 2) {
-            BinArgs a{plan->grid_bins, plan->d_goff, plan->d_gn, plan->d_gid, plan->d_tasks, plan->ntasks,
-                      plan->ngroups, plan->nbins, plan->d_pc, plan->bc, plan->d_counters, ea, 1, 0, nullptr};
-            CU(dispatch_bins(plan->ph, plan->nl_inst, grad, spec, &a, g, plan->block, s));
+            const bool sliced = ssh.S > 1;
+            const int NVs = 3 + (grad ? 3 : 0) + (spec ? plan->nL : 0);
+            BinArgs a{nullptr, plan->grid_rec, plan->d_goff, plan->d_gn, plan->d_gid, nullptr, plan->d_desc, ssh.ntasks,
+                      plan->ngroups, plan->nbins, plan->d_pc, plan->bc, plan->d_counters, ea,
+                      ssh.S, ssh.L / 4, sliced ? plan->d_slices : nullptr, NVs, plan->nL, spec, plan->d_step};
+            CU(dispatch_nodes(plan->ph, grad, a, g, nblock, s));
+            if (sliced) {
+                CU(launch_slices_reduce(plan->d_slices, ssh.S, NVs, ea, plan->d_pc, plan->npts, s));
+            } else {
+                CU(launch_point_sums(ea, s));
+            }
+            nl++;
         } else {
             BinArgs64 a{plan->grid64_bins, plan->d_goff, plan->d_gn, plan->d_gid, plan->d_tasks, plan->ntasks,
                         plan->ngroups, plan->nbins, plan->d_pc, plan->bc, plan->d_counters, ea};
-            CU(dispatch_bins(2, plan->nl_inst, grad, spec, &a, g, plan->block, s));
+            CU(dispatch_bins_ph2(plan->nl_inst, grad, spec, &a, g, nblock, s));
         }
     }
     nl++;
@@ -457,6 +562,7 @@ gna_status enqueue_eval(gna_plan* plan, const EvalReq& q, cudaStream_t s, int* l
         plan->cache_valid = true;
         plan->cache_grad = grad;
         plan->cache_spec = spec;
+        plan->cache_split = split;
     }
     *launches = nl;
     return GNA_OK;
@@ -469,32 +575,32 @@ gna_status enqueue_eval_general(gna_plan* plan, const EvalReq& q, cudaStream_t s
     const bool surv = plan->g_alpha == plan->g_beta;  // survival channel: phases modulo pi/2 (general.cuh)
     const int NV = gen_nv(grad);
     SliceShape ssh{1, 0, plan->ntasks};
+    const int ctas = node_ctas_per_sm(plan, grad, surv, plan->block);
     if (plan->mapping == MAP_SLICES) {
-        ssh = slice_shape(plan);
+        ssh = fixed_slice_shape(plan);
         if ((int64_t)plan->npts * plan->ngroups * ssh.S >= (1LL << 31)) return fail(plan, GNA_ESHAPE, "too many slice tasks");
     }
     const int64_t ncnt = 1 + (int64_t)plan->npts * (1 + plan->ngroups);
     CU(launch_prepare_general(q.pfull, plan->npts, plan->bc, plan->g_alpha, plan->g_beta, plan->g_anti, plan->d_pc,
                               plan->d_gc, plan->d_counters, ncnt, plan->d_status, s));
-    EpiArgs ea = make_epi(plan, q, grad, false, NV);
+    EpiArgs ea = make_epi(plan, q, grad, false, NV, false);
     ea.NBV = q.H ? kGenNBVFit : (grad ? 7 : 1);  // chi2, the six-parameter gradient terms, J^T W J
     ea.binsums = nullptr;
     const bool sliced = ssh.S > 1;
-    int64_t g = (int64_t)plan->sm_count * general_resident_ctas(plan->ph, plan->nl_inst, grad, surv, plan->block);
-    g = std::max<int64_t>(1, std::min<int64_t>(g, ((int64_t)ssh.ntasks * 32 + plan->block - 1) / plan->block));
+    const int g = grid_size(plan, ctas, plan->block, ssh.ntasks);
     if (plan->ph == 2) {
         GenArgs64 ga64{BinArgs64{plan->grid64_bins, plan->d_goff, plan->d_gn, plan->d_gid, plan->d_tasks, plan->ntasks,
                                  plan->ngroups, plan->nbins, plan->d_pc, plan->bc, plan->d_counters, ea},
                        plan->d_gc};
-        CU(dispatch_general64(plan->nl_inst, grad, ga64, (int)g, plan->block, s));
+        CU(dispatch_general64(plan->nl_inst, grad, ga64, g, plan->block, s));
         *launches = 2;
         return GNA_OK;
     }
-    GenArgs ga{BinArgs{plan->grid_bins, plan->d_goff, plan->d_gn, plan->d_gid, plan->d_tasks, ssh.ntasks,
+    GenArgs ga{BinArgs{plan->grid_bins, nullptr, plan->d_goff, plan->d_gn, plan->d_gid, plan->d_tasks, nullptr, ssh.ntasks,
                        plan->ngroups, plan->nbins, plan->d_pc, plan->bc, plan->d_counters, ea, ssh.S, ssh.L,
-                       sliced ? plan->d_slices : nullptr},
+                       sliced ? plan->d_slices : nullptr, NV, plan->nL, 0, plan->d_step},
                plan->d_gc};
-    CU(dispatch_general(plan->ph, plan->nl_inst, grad, surv, ga, (int)g, plan->block, s));
+    CU(dispatch_general(plan->ph, plan->nl_inst, grad, surv, ga, g, plan->block, s));
     *launches = 2;
     if (sliced) {
         CU(launch_slices_reduce_general(plan->d_slices, ssh.S, NV, ea, plan->d_gc, plan->npts, s));
@@ -934,6 +1040,13 @@ static gna_status plan_build(gna_plan* plan, const gna_plan_desc* d, cudaStream_
         gid[p] = (int)(std::lower_bound(gn.begin(), gn.end(), plan->counts[p]) - gn.begin());
     const int nbins_pad = ngroups * 32;
     // grid offsets of the bins layout (the split layout is one bin-major grid)
+    const bool quads = plan->ph < 2 && !plan->general;  // nodes also stored in quads
+    std::vector<int64_t> qoff(plan->ngrids);            // first quad of each grid
+    int64_t nquads = 0;
+    for (int g = 0; g < plan->ngrids; g++) {
+        qoff[g] = nquads;
+        nquads += (int64_t)ngroups * ((gn[g] + 3) / 4);
+    }
     std::vector<int64_t> goff(plan->ngrids);
     int64_t off = 0;
     for (int g = 0; g < plan->ngrids; g++) {
@@ -957,6 +1070,7 @@ static gna_status plan_build(gna_plan* plan, const gna_plan_desc* d, cudaStream_
     }
     if (plan->has_bins) {
         if (plan->ph < 2) TRY(dalloc(plan, &plan->grid_bins, len_bins));
+        if (quads) TRY(dalloc(plan, &plan->grid_rec, nquads * kQuadBytes));
         if (want64) TRY(dalloc(plan, &plan->grid64_bins, len_bins));
     }
     // plain chain: one bin-major {1/E, W} grid per distinct node count (the
@@ -998,25 +1112,44 @@ static gna_status plan_build(gna_plan* plan, const gna_plan_desc* d, cudaStream_
     if (plan->has_split) {
         const int n = plan->n_uniform;
         CU(launch_build_grid(d->nbins, d->nbins, plan->d_edges, n, glx + gl_off[n], glw + gl_off[n], plan->e_scale, 0,
-                             plan->grid_split, plan->grid64_split, plan->plain64, s));
+                             plan->grid_split, nullptr, plan->grid64_split, plan->plain64, s));
     }
     if (plan->has_bins)
         for (int g = 0; g < plan->ngrids; g++) {
             const int n = gn[g];
             CU(launch_build_grid(d->nbins, nbins_pad, plan->d_edges, n, glx + gl_off[n], glw + gl_off[n],
                                  plan->e_scale, 1, plan->grid_bins ? plan->grid_bins + goff[g] : nullptr,
+                                 quads ? plan->grid_rec + qoff[g] * kQuadBytes : nullptr,
                                  plan->grid64_bins ? plan->grid64_bins + goff[g] : nullptr,
                                  (plan->plain64 && !plan->has_split) ? plan->plain64 + plain_goff[g] : nullptr, s));
         }
     if (plain_alias) plan->plain64 = plan->grid64_split;
     if (plan->ph < 2) {
         TRY(dalloc(plan, &plan->d_sumW, (size_t)plan->ngrids * d->nbins));
+        TRY(dalloc(plan, &plan->d_sumWf, (size_t)plan->ngrids * d->nbins));
         for (int g = 0; g < plan->ngrids; g++) {
-            if (plan->has_split)
-                CU(launch_sum_weights(plan->grid_split, d->nbins, gn[g], 0, plan->d_sumW + (size_t)g * d->nbins, s));
-            else
-                CU(launch_sum_weights(plan->grid_bins + goff[g], d->nbins, gn[g], 1, plan->d_sumW + (size_t)g * d->nbins, s));
+            double* sw = plan->d_sumW + (size_t)g * d->nbins;
+            float2* swf = plan->d_sumWf + (size_t)g * d->nbins;
+            if (plan->has_split) CU(launch_sum_weights(plan->grid_split, d->nbins, gn[g], 0, sw, swf, s));
+            else CU(launch_sum_weights(plan->grid_bins + goff[g], d->nbins, gn[g], 1, sw, swf, s));
         }
+    }
+    std::vector<float> step;  // (copied from below: lives until the stream is synchronised)
+    std::vector<BinTask> desc;
+    if (plan->has_bins && plan->ph < 2) {
+        // neighbouring zeros of P_n are less than pi / (n + 1/2) apart in
+        // theta, x = cos theta, so the nodes of a bin of half width h are less
+        // than h pi / (n + 1/2) apart in E and 1/E_low^2 times that in 1/E
+        step.resize((size_t)plan->ngrids * ngroups);
+        for (int g = 0; g < plan->ngrids; g++)
+            for (int b = 0; b < ngroups; b++) {
+                double w = 0.0;
+                for (int i = b * 32; i < std::min(d->nbins, (b + 1) * 32); i++)
+                    w = std::max(w, 0.5 * (d->edges[i + 1] - d->edges[i]) / (d->edges[i] * d->edges[i]));
+                step[(size_t)g * ngroups + b] = (float)(w * M_PI / (gn[g] + 0.5));
+            }
+        TRY(dalloc(plan, &plan->d_step, step.size()));
+        CU(cudaMemcpyAsync(plan->d_step, step.data(), sizeof(float) * step.size(), cudaMemcpyHostToDevice, s));
     }
     CU(cudaStreamCreateWithFlags(&plan->cap_stream, cudaStreamNonBlocking));
     // task list (bins mapping): (point, group) ordered by decreasing node count
@@ -1032,13 +1165,23 @@ static gna_status plan_build(gna_plan* plan, const gna_plan_desc* d, cudaStream_
         plan->ntasks = (int)tasks.size();
         TRY(dalloc(plan, &plan->d_tasks, tasks.size()));
         CU(cudaMemcpyAsync(plan->d_tasks, tasks.data(), sizeof(int) * tasks.size(), cudaMemcpyHostToDevice, s));
+        if (quads) {
+            desc.reserve(tasks.size());
+            for (int p : order) {
+                const int g = gid[p], nq = (gn[g] + 3) / 4;
+                for (int b = 0; b < ngroups; b++)
+                    desc.push_back(BinTask{p, b, nq, step[(size_t)g * ngroups + b], qoff[g] + (int64_t)b * nq});
+            }
+            TRY(dalloc(plan, &plan->d_desc, desc.size()));
+            CU(cudaMemcpyAsync(plan->d_desc, desc.data(), sizeof(BinTask) * desc.size(), cudaMemcpyHostToDevice, s));
+        }
     }
     plan->ncounters = 1 + (int64_t)d->npts * (1 + ngroups) + (plan->has_split ? (int64_t)d->npts * d->nbins : 0);
     TRY(dalloc(plan, &plan->d_counters, plan->ncounters));
     // scratch
     TRY(dalloc(plan, &plan->d_pc, d->npts));
     if (plan->general) TRY(dalloc(plan, &plan->d_gc, d->npts));
-    const int nv_max = std::max(fused_nv(plan->nl_inst, true, true), plan->general ? gen_nv(true) : 0);
+    const int nv_max = std::max(fused_nv(plan->nl_inst, true, true), plan->general ? gen_nv(true) : 0) + 1;
     if (plan->has_split) {
         // ranges are at least 128 nodes long, so a bin meets at most ceil(n / 128) + 1 of
         // them; the slot count is capped so that the partials stay within 256 M values
@@ -1257,14 +1400,15 @@ gna_status gna_chain_eval_cached(gna_plan* plan, const double* eta, double sigma
     if (out->grad_eta && !eta) return fail(plan, GNA_EINVAL, "grad_eta needs eta");
     cudaStream_t s = (cudaStream_t)stream;
     plan->last_stream = s;
-    const int NV = value_count(plan, plan->cache_grad, plan->cache_spec);
+    const int NV = value_count(plan, plan->cache_grad, plan->cache_spec, plan->cache_split);
     EvalReq q{nullptr, eta, sigma_eta, data, data_per_point, out->chi2, out->grad, out->grad_eta, out->mu, out->spectra,
               nullptr};
-    EpiArgs ea = make_epi(plan, q, plan->cache_grad, plan->cache_spec, NV);
+    EpiArgs ea = make_epi(plan, q, plan->cache_grad, plan->cache_spec, NV, plan->cache_split);
     ea.NBV = out->grad ? 5 : 1;  // the tangent terms are summed over bins only when asked for
     ea.binsums = nullptr;
     CU(cudaMemsetAsync(plan->d_counters, 0, sizeof(int) * (1 + (size_t)plan->npts * (1 + plan->ngroups)), s));
-    CU(launch_cached_epilogue(plan->d_binsums, ea, s));
+    if (plan->ph < 2 && !plan->cache_split) CU(launch_cached_terms((const float2*)plan->d_binsums, ea, s));
+    else CU(launch_cached_epilogue(plan->d_binsums, ea, s));
     plan->last_launches = 1;
     return GNA_OK;
 }
@@ -1651,6 +1795,7 @@ gna_status gna_plan_autotune(gna_plan* plan, const gna_osc* params, const double
     std::vector<std::string> cand;
     const int blocks[3] = {64, 128, 256};
     char t[96];
+    const bool nodes128 = plan->ph < 2;  // the bin and slice kernels take blocks of at most 128 threads
     if (plan->has_split) {
         // block size only changes how the equal ranges sit on the SMs; the
         // minimum range length matters only for workloads smaller than the GPU
@@ -1663,14 +1808,21 @@ gna_status gna_plan_autotune(gna_plan* plan, const gna_osc* params, const double
     }
     if (plan->has_bins)
         for (int b : blocks) {
+            if (nodes128 && b > 128) continue;
             snprintf(t, sizeof(t), "mapping=bins block=%d nodes=1", b);
             cand.push_back(t);
         }
     if (plan->has_bins && plan->uniform && plan->ph < 2 && plan->slices_cap > 1) {
-        // slice lengths for about 1, 2 and 4 tasks per resident warp
+        // the chosen slice length, and lengths for about 1, 2 and 4 tasks per
+        // 16 warps on each SM
         const int64_t pg = (int64_t)plan->npts * plan->ngroups;
-        for (int b : {128, 256})
-            for (int tpw : {1, 2, 4}) {
+        for (int b : {64, 128})
+            for (int tpw : {0, 1, 2, 4}) {
+                if (tpw == 0) {
+                    snprintf(t, sizeof(t), "mapping=slices block=%d slice=0", b);
+                    cand.push_back(t);
+                    continue;
+                }
                 const int64_t S = std::max<int64_t>(1, ((int64_t)tpw * 16 * plan->sm_count + pg - 1) / pg);
                 const int64_t L = (plan->n_uniform + S - 1) / S;
                 snprintf(t, sizeof(t), "mapping=slices block=%d slice=%lld", b, (long long)L);

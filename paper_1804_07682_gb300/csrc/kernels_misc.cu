@@ -70,6 +70,7 @@ __global__ void k_prepare_points(const gna_osc* __restrict__ prm, int npts, Base
             pc.dA12f[j] = (float)d12[j];
             pc.dA13f[j] = (float)d13[j];
         }
+        pc.cmax = largest_phase(bc, o.dm2_21, o.dm2_32);
     }
 }
 
@@ -152,10 +153,13 @@ cudaError_t launch_gl(int n, double* x, double* w, double* tmp_ab /*[2n]*/, cuda
 // 1/E split into two floats, W = (b_i-a_i)/2 w_k S(E_ik e_scale) with the
 // reactor shape S(E) = exp(0.87 - 0.16 E - 0.091 E^2), and W/E.  Layout 0:
 // bin-major (node k of bin i at i*n + k); layout 1: groups of 32 bins,
-// node k of bin i at ((i/32) n + k) 32 + i%32, padded bins have W = 0.
+// node k of bin i at ((i/32) n + k) 32 + i%32, padded bins have W = 0.  rec
+// (layout 1): the same order in quads of nodes, per group and quad three rows of
+// 32 float4 (one per bin): 1/E hi, W, 1/E lo of the quad's nodes; an order's
+// last quad is filled with its last node and W = 0.
 __global__ void k_build_grid(int nbins, int nbins_pad, const double* __restrict__ edges, int n, const double* __restrict__ x,
                              const double* __restrict__ w, double e_scale, int layout, float4* __restrict__ ff,
-                             double2* __restrict__ d64, double2* __restrict__ plain64) {
+                             char* __restrict__ rec, double2* __restrict__ d64, double2* __restrict__ plain64) {
     const int64_t idx = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     if (idx >= (int64_t)nbins_pad * n) return;
     const int i = (int)(idx / n);
@@ -175,6 +179,17 @@ __global__ void k_build_grid(int nbins, int nbins_pad, const double* __restrict_
         split_ff(invE, hi, lo);
         ff[pos] = make_float4(hi, lo, (float)Wd, (float)(Wd * invE));
     }
+    if (rec) {
+        float hi, lo;
+        split_ff(invE, hi, lo);
+        float* q = reinterpret_cast<float*>(rec + ((int64_t)(i >> 5) * ((n + 3) >> 2) + (k >> 2)) * (3 * 512)) + (i & 31) * 4;
+        const int last = (k == n - 1) ? 3 : (k & 3);
+        for (int u = k & 3; u <= last; u++) {
+            q[u] = hi;
+            q[128 + u] = u == (k & 3) ? (float)Wd : 0.f;
+            q[256 + u] = lo;
+        }
+    }
     if (d64) d64[pos] = make_double2(invE, Wd);
     if (plain64 && i < nbins) plain64[idx] = make_double2(invE, Wd);
 }
@@ -182,7 +197,8 @@ __global__ void k_build_grid(int nbins, int nbins_pad, const double* __restrict_
 // Sum of the FP32 node weights of each bin, in double (for the epilogue's
 // exact correction of the constant term): one warp per bin, lane l takes
 // nodes l, l + 32, ... (coalesced in layout 0), then a fixed-order butterfly.
-__global__ void k_sum_weights(const float4* __restrict__ grid, int nbins, int n, int layout, double* __restrict__ out) {
+__global__ void k_sum_weights(const float4* __restrict__ grid, int nbins, int n, int layout, double* __restrict__ out,
+                              float2* __restrict__ outf) {
     const int i = (int)(((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5);
     const int lane = threadIdx.x & 31;
     if (i >= nbins) return;
@@ -193,19 +209,24 @@ __global__ void k_sum_weights(const float4* __restrict__ grid, int nbins, int n,
     }
 #pragma unroll
     for (int o = 16; o >= 1; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
-    if (lane == 0) out[i] = s;
+    if (lane == 0) {
+        out[i] = s;
+        split_ff(s, outf[i].x, outf[i].y);
+    }
 }
 
-cudaError_t launch_sum_weights(const float4* grid, int nbins, int n, int layout, double* out, cudaStream_t s) {
-    k_sum_weights<<<(unsigned)(((int64_t)nbins * 32 + 255) / 256), 256, 0, s>>>(grid, nbins, n, layout, out);
+cudaError_t launch_sum_weights(const float4* grid, int nbins, int n, int layout, double* out, float2* outf,
+                               cudaStream_t s) {
+    k_sum_weights<<<(unsigned)(((int64_t)nbins * 32 + 255) / 256), 256, 0, s>>>(grid, nbins, n, layout, out, outf);
     return cudaGetLastError();
 }
 
 cudaError_t launch_build_grid(int nbins, int nbins_pad, const double* edges, int n, const double* x, const double* w,
-                              double e_scale, int layout, float4* ff, double2* d64, double2* plain64, cudaStream_t s) {
+                              double e_scale, int layout, float4* ff, char* rec, double2* d64, double2* plain64,
+                              cudaStream_t s) {
     const int64_t total = (int64_t)nbins_pad * n;
     const int64_t blocks = (total + 255) / 256;
-    k_build_grid<<<(unsigned)blocks, 256, 0, s>>>(nbins, nbins_pad, edges, n, x, w, e_scale, layout, ff, d64, plain64);
+    k_build_grid<<<(unsigned)blocks, 256, 0, s>>>(nbins, nbins_pad, edges, n, x, w, e_scale, layout, ff, rec, d64, plain64);
     return cudaGetLastError();
 }
 

@@ -84,8 +84,10 @@ cudaError_t launch_prepare(const gna_osc* prm, int npts, const BaseConst& bc, Po
                            int* zero = nullptr, int64_t nz = 0, int* status = nullptr);
 cudaError_t launch_gl(int n, double* x, double* w, double* tmp_ab, cudaStream_t s);
 cudaError_t launch_build_grid(int nbins, int nbins_pad, const double* edges, int n, const double* x, const double* w,
-                              double e_scale, int layout, float4* ff, double2* d64, double2* plain64, cudaStream_t s);
-cudaError_t launch_sum_weights(const float4* grid, int nbins, int n, int layout, double* out, cudaStream_t s);
+                              double e_scale, int layout, float4* ff, char* rec, double2* d64, double2* plain64,
+                              cudaStream_t s);
+cudaError_t launch_sum_weights(const float4* grid, int nbins, int n, int layout, double* out, float2* outf,
+                               cudaStream_t s);
 // The plain chain's kernels for one chunk of points: OscProb (+ tangents),
 // weights, bin integration, chi^2 (4 launches, 6 with the tangents).
 cudaError_t launch_plain_chunk(const PlainArgs& a, const PlainChi2Args& ca, cudaStream_t s);

@@ -234,6 +234,7 @@ extern "C" gna_status gna_chain_eval_noalloc(int nbins, int n, const double* E, 
     a.sumW = reinterpret_cast<double*>(base + kOffSumW);
     gna::EpiArgs& ea = a.ea;
     ea.is64 = 0;
+    ea.corr = 1;
     ea.NV = 5;
     ea.has_grad = 1;
     ea.nspec = 0;

@@ -1053,3 +1053,37 @@ def test_general_fits_match_oracle(api, prec):
         # directions and no statistical errors exist to measure them in
         assert rel(P[j], th) < (1e-7 if prec == "fp64" else 1e-3), (j, P[j], th)
     plan.close()
+
+
+# ------------------------------------------- chunk-anchored node kernels
+@pytest.mark.parametrize("prec", ["f64phase", "ff"])
+@pytest.mark.parametrize("mapping", ["bins", "slices"])
+@pytest.mark.parametrize("nL", [1, 2, 3, 5, 9])
+@pytest.mark.parametrize("n,edges", [(1, (2.0, 9.0)), (3, (2.0, 9.0)), (4, (2.0, 9.0)), (5, (3.0, 3.4)), (33, (3.0, 3.4)),
+                                     (130, (3.0, 3.4)), (67, (0.6, 12.0))])
+def test_anchored_chunks(api, prec, mapping, nL, n, edges):
+    # orders around a quad and a chunk of nodes; fine grids (3-3.4 MeV: long
+    # chunks), coarse ones (2-9 MeV with up to 5 nodes: every phase reduced)
+    # and one that has both and lengths between (0.6-12 MeV); baselines below,
+    # at and beyond the packed instantiations; 37 bins: a ragged group
+    rng = np.random.default_rng(nL + n)
+    e = np.linspace(edges[0], edges[1], 38)
+    L = rng.uniform(1.0, 60.0, nL)
+    theta = np.array(wl.TRUTH) * 1.03
+    Nn = oracle.norm_for_total(e, n, L, wl.TRUTH)
+    data = wl.poisson_data(Nn * (oracle.baseline_weights(L) @ oracle.binned(e, n, L, wl.TRUTH)), 7)
+    ref = oracle.chain(e, n, L, theta, Nn, data, wl.POISSON)
+    plan = api.Plan(e, L, nodes_per_bin=n, norm=Nn, prec=prec, kind="poisson", mapping=mapping)
+    if mapping == "slices":
+        plan.tuning = "slice=16"
+    p, d = plan.params_tensor(theta), dev(data)
+    out = plan.eval(p, d, grad=True, mu=True, spectra=True)
+    alone = plan.eval(p, d, grad=False)
+    torch.cuda.synchronize()
+    plan.status()
+    assert rel(out["mu"][0].cpu().numpy(), ref["mu"]) < 1e-6
+    assert rel(out["spectra"][0].cpu().numpy(), ref["mu_rb"]) < 1e-6
+    assert normrel(out["grad"][0].cpu().numpy(), ref["grad"][:4]) < 1e-4
+    for o in (out, alone):  # few nodes per bin: the scaled bound (see the module's head)
+        check_chi2(o["chi2"][0].item(), ref, data, wl.POISSON, 1e-6, tag="anchored %d %d" % (nL, n), plain=False)
+    plan.close()
