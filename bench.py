@@ -36,18 +36,14 @@ PEAKS_FILE = os.path.join(ROOT, "MEASURED_PEAKS.json")
 SM_COUNT, FP32_LANES, SM_MAX_MHZ = 152, 128, 2070.0
 
 
-def fp32_ops_general(nL: int, grad: bool, surv: bool) -> int:
-    """Algorithmic FP32 operations per energy node of the any-channel node
-    kernel: per (node, baseline) the phases reduced modulo pi and their
-    sin/cos 38, angle addition 4, sin^2, sin cos and cos^2 of three phases 9,
-    their weighted sums over the baselines 9 (18 with hi + lo weights for
-    several baselines; none for one baseline, whose weight is exactly 1),
-    with the gradient cos^2 - sin^2 3 and two more weighted sums per phase 6;
-    per node the Kahan product-sums of 9 (15) values, 4 each.  Survival
-    channels (alpha = beta) reduce the phases modulo pi/2 instead (11 each)
-    with quadrant swaps (3 each): 10 more per (node, baseline)."""
-    per_r = 51 + (18 if nL > 1 else 0) + (9 if grad else 0) + (10 if surv else 0)
-    return nL * per_r + (60 if grad else 36)
+def fp32_ops_general(nL: int, grad: bool) -> int:
+    """Algorithmic FP32 operations (FMA = 1) per energy node of the any-channel
+    chain's chunk-anchored node kernels: per (node, baseline) two phases by one
+    FMA each from the chunk's anchor 2, sin and cos - 1 of both 20, the third
+    pair by the addition formulas 6, weighted sums 6 (12 with the gradient);
+    per node the offset of 1/E 3, W/E 1, the sum of W 4 and of W/E 1 (with the
+    gradient).  Anchors and the additions of a chunk's sums are not counted."""
+    return nL * (40 if grad else 34) + 8 + (1 if grad else 0)
 
 
 def fp32_ops_per_node(nL: int, grad: bool, spec: bool) -> int:
@@ -372,7 +368,7 @@ def side_workloads(api, torch, device, args):
     a1.record(stream)
     torch.cuda.synchronize()
     ms = a0.elapsed_time(a1) / reps
-    ops = sum(fp32_ops_general(1, True, False) * w.nbins * int(n) for n in w.node_counts)  # appearance
+    ops = sum(fp32_ops_general(1, True) * w.nbins * int(n) for n in w.node_counts)
     check["scan_numu_nue"] = (w, Ng, datag.cpu().numpy(), og["chi2"].cpu().numpy(), og["grad"].cpu().numpy(), th6)
     out["scan_64x64_500bins_numu_nue"] = {
         "scans_per_s": 1e3 / ms, "ms_per_scan": ms, "chi2_grad_evals_per_s": w.npts * 1e3 / ms,

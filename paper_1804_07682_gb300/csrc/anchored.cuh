@@ -98,15 +98,35 @@ __device__ __forceinline__ f32x2p ff_add2(f32x2p a, f32x2p b) {
 // Compensated sum of the two lanes' values (s + n).
 struct Kahan2 {
     f32x2 s, n;
-    __device__ __forceinline__ void zero() { s = n = f32x2{0.f, 0.f}; }
     __device__ __forceinline__ void add(f32x2 x) {
         const f32x2 y = add2(x, n);
         const f32x2 t = add2(s, y);
         n = add2(y, sub2(s, t));
         s = t;
     }
+};
+
+// Sum of a chunk's weights to about 2^-40 of itself, four operations a value:
+// s starts at a bias far above the weights, so that the fast form of the
+// error-free sum holds from the first one on (weights grow along a bin's
+// start), and the errors are summed in n.
+struct WeightSum {
+    float bias;
+    f32x2 s, n;
+    __device__ __forceinline__ void start(f32x2 w) {
+        bias = 4096.0f * w.x;
+        s = dup2(bias);
+        n = f32x2{0.f, 0.f};
+    }
+    __device__ __forceinline__ void add(f32x2 x) {
+        const f32x2 t = add2(s, x);
+        n = add2(n, add2(sub2(s, t), x));
+        s = t;
+    }
     // both lanes, as a float pair
-    __device__ __forceinline__ float2 total() const { return ff_add(make_float2(s.x, n.x), make_float2(s.y, n.y)); }
+    __device__ __forceinline__ float2 total() const {
+        return ff_add(make_float2(__fsub_rn(s.x, bias), n.x), make_float2(__fsub_rn(s.y, bias), n.y));
+    }
 };
 
 // s = sin r, h = cos r - 1 on |r| <= pi/2 + kSwing, for N packed arguments
@@ -337,18 +357,18 @@ __device__ __forceinline__ float2 spectrum_part(const PointConst* pc, const floa
     return ff_add(s, ff_mul(0.5f * pc->Af[2], 0.5f * pc->Alo[2], T[2]));
 }
 
-// A bin's prediction and tangents from its sums (the order of fused.cuh).
+// A bin's prediction and its derivatives from its sums.
 template <bool GRAD>
-__device__ __forceinline__ BinSums bin_sums(const PointConst* pc, float2 sumw, const TaskSums& q) {
-    BinSums b;
+__device__ __forceinline__ BinSums<GRAD ? 4 : 0> bin_sums(const PointConst* pc, float2 sumw, const TaskSums& q) {
+    BinSums<GRAD ? 4 : 0> b;
     const float2 x = spectrum_part(pc, q.T);
     b.M = ff_add(sumw, make_float2(-x.x, -x.y));
     if constexpr (GRAD) {
-        const float t0 = 0.5f * q.T[0].x, t1 = 0.5f * q.T[1].x, t2 = 0.5f * q.T[2].x;
-        b.v[0] = fmaf(pc->dA12f[2], t2, fmaf(pc->dA12f[1], t1, pc->dA12f[0] * t0));
-        b.v[1] = fmaf(pc->dA13f[2], t2, fmaf(pc->dA13f[1], t1, pc->dA13f[0] * t0));
-        b.v[2] = fmaf(pc->Af[1], q.N[1], pc->Af[0] * q.N[0]);
-        b.v[3] = fmaf(pc->Af[2], q.N[2], pc->Af[1] * q.N[1]);
+        const float t0 = -0.5f * q.T[0].x, t1 = -0.5f * q.T[1].x, t2 = -0.5f * q.T[2].x;
+        b.d[0] = fmaf(pc->dA12f[2], t2, fmaf(pc->dA12f[1], t1, pc->dA12f[0] * t0));
+        b.d[1] = fmaf(pc->dA13f[2], t2, fmaf(pc->dA13f[1], t1, pc->dA13f[0] * t0));
+        b.d[2] = -fmaf(pc->Af[1], q.N[1], pc->Af[0] * q.N[0]);
+        b.d[3] = -fmaf(pc->Af[2], q.N[2], pc->Af[1] * q.N[1]);
     }
     return b;
 }
@@ -372,9 +392,10 @@ template <bool GRAD>
 __device__ __forceinline__ void finish_bins(const BinArgs& a, int p, int b, const TaskSums& q, const float2* sp,
                                             const BinInput& in, int lane) {
     const int i = b * 32 + lane;
-    float2 regs[5];
-    if (i < a.nbins) bin_terms<GRAD>(a.ea, p, i, bin_sums<GRAD>(a.pcs + p, in.sumw, q), sp, in, regs);
-    group_terms<GRAD>(a.ea, p, b, lane, regs);
+    constexpr int NG = GRAD ? 4 : 0;
+    float2 regs[1 + NG];
+    if (i < a.nbins) bin_terms<NG>(a.ea, p, i, bin_sums<GRAD>(a.pcs + p, in.sumw, q), sp, in, regs);
+    group_terms<NG>(a.ea, p, b, lane, regs);
 }
 
 // ------------------------------------------------ several baselines ------
@@ -586,8 +607,9 @@ __global__ void __maxnreg__(NP == 4 ? 168 : 128) k_nodes_multi(BinArgs a) {
                     const unsigned par = x.anchor(pc, r0, an.x, an.y);
                     const f32x2 nah = dup2(-an.x), nal = dup2(-an.y);
                     if (kb < k.nq) an = load_anchor(k, kb, min(step, k.nq - kb));
-                    Kahan2 w;
-                    w.zero();
+                    WeightSum w;
+                    in.wait();
+                    w.start(in.pair(0).w);
 #pragma unroll 1
                     for (int j = ka; j < kb; j++) {
                         in.wait();
@@ -765,8 +787,9 @@ __global__ void __maxnreg__(112) k_nodes_one(BinArgs a) {
                     x.a32 = dup2(phase<PH, true>(pc, 0, true, an.x, an.y, q32));
                     const f32x2 nah = dup2(-an.x), nal = dup2(-an.y);
                     if (kb < k.nq) an = load_anchor(k, kb, min(step, k.nq - kb));
-                    Kahan2 w;
-                    w.zero();
+                    WeightSum w;
+                    in.wait();
+                    w.start(in.pair(0).w);
 #pragma unroll 1
                     for (int j = ka; j < kb; j++) {
                         in.wait();

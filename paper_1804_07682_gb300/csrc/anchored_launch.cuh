@@ -6,6 +6,7 @@
 #include <mutex>
 
 #include "anchored.cuh"
+#include "slices.cuh"
 
 namespace gna {
 
@@ -14,26 +15,13 @@ size_t nodes_smem(int block) {
     return sizeof(f32x2p) * NP * (GRAD ? 6 : 3) * (size_t)block + (size_t)block / 32 * QuadRing<kRingMulti>::kWarpBytes;
 }
 
-inline size_t one_smem(int block) { return (size_t)block / 32 * QuadRing<kRingOne>::kWarpBytes; }
+constexpr size_t kNodesSmem = 72 * 1024;  // the most a block of 128 threads takes
 
-// More than the default 48 KB of dynamic shared memory: opt in once per device and kernel.
-template <auto K>
-cudaError_t allow_smem() {
-    static std::once_flag once[64];
-    static cudaError_t attr[64];
-    int dev = 0;
-    cudaError_t e = cudaGetDevice(&dev);
-    if (e != cudaSuccess) return e;
-    if (dev < 0 || dev >= 64) return cudaErrorInvalidDevice;
-    std::call_once(once[dev], [&] {
-        attr[dev] = cudaFuncSetAttribute(K, cudaFuncAttributeMaxDynamicSharedMemorySize, 72 * 1024);
-    });
-    return attr[dev];
-}
+inline size_t one_smem(int block) { return (size_t)block / 32 * QuadRing<kRingOne>::kWarpBytes; }
 
 template <int PH, int NP, bool GRAD>
 cudaError_t launch_multi(const BinArgs& a, int grid, int block, cudaStream_t s) {
-    cudaError_t e = allow_smem<k_nodes_multi<PH, NP, GRAD>>();
+    cudaError_t e = allow_smem<k_nodes_multi<PH, NP, GRAD>>(kNodesSmem);
     if (e != cudaSuccess) return e;
     return launch_dependent(k_nodes_multi<PH, NP, GRAD>, a, grid, block, s, nodes_smem<NP, GRAD>(block));
 }
@@ -54,7 +42,7 @@ cudaError_t launch_nodes(bool grad, const BinArgs& a, int grid, int block, cudaS
 template <auto K>
 int resident_of(int block, size_t smem) {
     int n = 0;
-    if (allow_smem<K>() != cudaSuccess) return 1;
+    if (allow_smem<K>(kNodesSmem) != cudaSuccess) return 1;
     if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, K, block, smem) != cudaSuccess) {
         cudaGetLastError();
         return 1;

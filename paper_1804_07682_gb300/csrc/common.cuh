@@ -44,6 +44,7 @@ struct BaseConst {
     float wkl[GNA_NLMAX];   // 2 omega_r K L_r: d sin^2 D / d dm2 = sin 2D K L / E
     double omd[GNA_NLMAX];  // omega_r (FP64)
     double kld[GNA_NLMAX];  // K L_r (FP64)
+    double klmax;           // largest K L_r
     float wsum;             // sum_r om_r rounded to FP32
     double wsum_lo;         // sum_r om_r - wsum (exact sum of the FP32 weights)
     int nL;
@@ -51,10 +52,8 @@ struct BaseConst {
 
 // Largest |K dm2 L_r| of a point's phases 21 and 32, rounded up (NaN if a splitting is).
 __device__ __forceinline__ float largest_phase(const BaseConst& bc, double dm2_21, double dm2_32) {
-    double kl = 0.0;
-    for (int r = 0; r < bc.nL; r++) kl = bc.kld[r] > kl ? bc.kld[r] : kl;
     const double a = fabs(dm2_21), b = fabs(dm2_32);
-    return __double2float_ru(kl * ((a >= b || a != a) ? a : b));
+    return __double2float_ru(bc.klmax * ((a >= b || a != a) ? a : b));
 }
 
 // ---------------------------------------------------------------- Kahan --

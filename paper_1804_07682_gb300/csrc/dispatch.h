@@ -22,7 +22,7 @@ struct BinArgs;
 struct FitArgs;
 cudaError_t dispatch_fit(int ph, int nl, const FitArgs& a, int grid, int block, cudaStream_t s);
 cudaError_t launch_fit_slices_reduce(const float2* part, int S, const EpiArgs& ea, int npts, cudaStream_t s);
-cudaError_t launch_point_sums(const EpiArgs& ea, cudaStream_t s);
+cudaError_t launch_point_sums(int npar, const EpiArgs& ea, cudaStream_t s);  // npar: 4 or 6
 cudaError_t launch_cached_terms(const float2* sums, const EpiArgs& ea, cudaStream_t s);
 cudaError_t dispatch_nodes(int ph, bool grad, const BinArgs& a, int grid, int block, cudaStream_t s);
 int nodes_block(int block);

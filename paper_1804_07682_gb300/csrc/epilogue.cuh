@@ -220,8 +220,9 @@ __device__ inline void group_reduce(const EpiArgs& a, int p, int g, int lane, co
 }
 
 // Point p: lane l sums groups l, l + 32, ... in order, then one transposed
-// reduction over the lanes; the point's outputs are written.
-template <int NVP>
+// reduction over the lanes; the point's outputs are written (NG: gradient
+// components per point).
+template <int NVP, int NG = 4>
 __device__ inline void point_reduce(const EpiArgs& a, int p, int lane) {
     constexpr int SH = NVP == 16 ? 1 : 2;
     float2 v[NVP];
@@ -230,7 +231,7 @@ __device__ inline void point_reduce(const EpiArgs& a, int p, int lane) {
     for (int g = lane; g < a.ngroups; g += 32) {
         const float2* gv = a.gvals + ((int64_t)p * a.ngroups + g) * a.NBV;
 #pragma unroll
-        for (int j = 0; j < (NVP == 16 ? 15 : 5); j++)
+        for (int j = 0; j < (NVP == 16 ? 15 : 1 + NG); j++)
             if (j < a.NBV) v[j] = ff_add(v[j], __ldcg(gv + j));
     }
     warp_transpose_reduce<NVP>(v, lane);
@@ -238,8 +239,8 @@ __device__ inline void point_reduce(const EpiArgs& a, int p, int lane) {
     if ((lane & ((1 << SH) - 1)) == 0 && vi < a.NBV) {
         const double tot = (double)v[0].x + (double)v[0].y;
         if (vi == 0) a.chi2[p] = tot;
-        else if (vi < 5) {
-            if (a.grad) a.grad[(int64_t)p * 4 + vi - 1] = tot;
+        else if (vi < 1 + NG) {
+            if (a.grad) a.grad[(int64_t)p * NG + vi - 1] = tot;
         } else if (a.H) {
             a.H[(int64_t)p * 10 + vi - 5] = tot;
         }
@@ -247,7 +248,7 @@ __device__ inline void point_reduce(const EpiArgs& a, int p, int lane) {
 }
 
 // A group's sums are stored: the last group of the point sums the groups.
-template <int NVP>
+template <int NVP, int NG = 4>
 __device__ __forceinline__ void group_counted(const EpiArgs& a, int p, int lane) {
     // every lane that stored a group value makes it visible before lane 0 counts the group
     __threadfence();
@@ -257,7 +258,7 @@ __device__ __forceinline__ void group_counted(const EpiArgs& a, int p, int lane)
     lastp = __shfl_sync(0xffffffffu, lastp, 0);
     if (lastp) {
         __threadfence();
-        point_reduce<NVP>(a, p, lane);
+        point_reduce<NVP, NG>(a, p, lane);
     }
 }
 
@@ -315,9 +316,10 @@ __device__ __forceinline__ BinInput bin_input(const EpiArgs& a, int p, int i) {
     return in;
 }
 
+template <int NG>
 struct BinSums {
-    float2 M;    // sum_k W_k sum_r omega_r P_r
-    float v[4];  // tangent sums (their sign applied here)
+    float2 M;                  // sum_k W_k sum_r omega_r P_r
+    float d[NG > 0 ? NG : 1];  // its derivatives
 };
 
 __device__ __forceinline__ float2 ff_norm(float p, float e) {
@@ -325,22 +327,19 @@ __device__ __forceinline__ float2 ff_norm(float p, float e) {
     return make_float2(h, __fsub_rn(e, __fsub_rn(h, p)));
 }
 
-// Bin (p, i): outputs, and the terms to be summed over bins into regs[0..4]
+// Bin (p, i): outputs, and the terms to be summed over bins into regs[0..NG]
 // (chi^2, gradient).  sp[r]: what to take from sumw for baseline r's sum (with spectra).
-template <bool GRAD>
-__device__ __forceinline__ void bin_terms(const EpiArgs& a, int p, int i, const BinSums& b, const float2* sp,
+template <int NG>
+__device__ __forceinline__ void bin_terms(const EpiArgs& a, int p, int i, const BinSums<NG>& b, const float2* sp,
                                           const BinInput& in, float2* regs) {
     const int64_t idx = (int64_t)p * a.nbins + i;
-    constexpr int off = GRAD ? 3 : 1;
     if (a.binsums) {
-        // kept as float pairs: M, the tangents two by two, the baselines' parts
+        // kept as float pairs: M, the derivatives two by two, the baselines' parts
         float2* s = reinterpret_cast<float2*>(a.binsums) + idx * a.NV;
         s[0] = b.M;
-        if constexpr (GRAD) {
-            s[1] = make_float2(b.v[0], b.v[1]);
-            s[2] = make_float2(b.v[2], b.v[3]);
-        }
-        for (int r = 0; r < a.nspec; r++) s[off + r] = sp[r];
+#pragma unroll
+        for (int q = 0; q < NG; q += 2) s[1 + q / 2] = make_float2(b.d[q], b.d[q + 1]);
+        for (int r = 0; r < a.nspec; r++) s[1 + NG / 2 + r] = sp[r];
     }
     if (a.spectra_out) {
         const double w = (double)in.sumw.x + (double)in.sumw.y;
@@ -369,27 +368,25 @@ __device__ __forceinline__ void bin_terms(const EpiArgs& a, int p, int i, const 
     const bool pen = a.penalty != 0;
     if (pen) term = ff_add(term, to_ff(in.e * in.e / (a.sigma * a.sigma)));
     regs[0] = term;
-    if constexpr (GRAD) {
 #pragma unroll
-        for (int q = 0; q < 4; q++) regs[1 + q] = make_float2(g * (-fh * b.v[q]), 0.f);
-    }
+    for (int q = 0; q < NG; q++) regs[1 + q] = make_float2(g * (fh * b.d[q]), 0.f);
     if (a.mu_out) a.mu_out[idx] = (double)mu.x + (double)mu.y;
     if (a.grad_eta_out)
         a.grad_eta_out[idx] = (double)g * a.norm * ((double)b.M.x + (double)b.M.y) + (pen ? 2.0 * in.e / (a.sigma * a.sigma) : 0.0);
 }
 
-// The group's sums of at most five values in registers, and group_done for them.
-template <bool GRAD>
-__device__ __forceinline__ void group_terms(const EpiArgs& a, int p, int g, int lane, const float2 (&regs)[5]) {
+// The group's sums of 1 + NG values in registers, and group_done for them.
+template <int NG>
+__device__ __forceinline__ void group_terms(const EpiArgs& a, int p, int g, int lane, const float2 (&regs)[1 + NG]) {
     float2 r[8];
 #pragma unroll
-    for (int j = 0; j < 8; j++) r[j] = j < (GRAD ? 5 : 1) ? regs[j < 5 ? j : 0] : make_float2(0.f, 0.f);
+    for (int j = 0; j < 8; j++) r[j] = j <= NG ? regs[j <= NG ? j : 0] : make_float2(0.f, 0.f);
     group_reduce<8>(a, p, g, lane, r);
 }
-template <bool GRAD>
-__device__ __forceinline__ void group_done_terms(const EpiArgs& a, int p, int g, int lane, const float2 (&regs)[5]) {
-    group_terms<GRAD>(a, p, g, lane, regs);
-    group_counted<8>(a, p, lane);
+template <int NG>
+__device__ __forceinline__ void group_done_terms(const EpiArgs& a, int p, int g, int lane, const float2 (&regs)[1 + NG]) {
+    group_terms<NG>(a, p, g, lane, regs);
+    group_counted<8, NG>(a, p, lane);
 }
 
 }  // namespace gna

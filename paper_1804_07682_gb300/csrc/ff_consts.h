@@ -21,14 +21,15 @@
 #define GNA_COSA_C3 (-1.388737932e-03f)
 #define GNA_COSA_C4 (2.471726839e-05f)
 #define GNA_COSA_C5 (-2.540818400e-07f)
-// Chunk-anchored loops, |r| <= 0.936398: polynomial error sin 8.69e-09, cos 5.80e-10.
-#define GNA_SINQ_C1 (-1.666662097e-01f)
-#define GNA_SINQ_C2 (8.330608718e-03f)
-#define GNA_SINQ_C3 (-1.935162727e-04f)
-#define GNA_COSQ_C1 (-5.000000000e-01f)
-#define GNA_COSQ_C2 (4.166660830e-02f)
-#define GNA_COSQ_C3 (-1.388576464e-03f)
-#define GNA_COSQ_C4 (2.428173866e-05f)
+// Chunk-anchored loops, |r| <= 1.186398: polynomial error sin 2.28e-10, cos 3.68e-09.
+#define GNA_SINQ_C1 (-1.666666567e-01f)
+#define GNA_SINQ_C2 (8.333275095e-03f)
+#define GNA_SINQ_C3 (-1.982997928e-04f)
+#define GNA_SINQ_C4 (2.666453838e-06f)
+#define GNA_COSQ_C1 (-4.999999404e-01f)
+#define GNA_COSQ_C2 (4.166620970e-02f)
+#define GNA_COSQ_C3 (-1.387852593e-03f)
+#define GNA_COSQ_C4 (2.389178371e-05f)
 // pi = PI_A + PI_B + PI_C; PI_A and PI_B have 12 significant bits.
 #define GNA_PI_A (3.140625f)
 #define GNA_PI_B (0.00096750259399414062f)

@@ -24,7 +24,7 @@ N_SIN = 4  # S1..S4: odd degree 9 (error ~5e-9)
 N_COS = 4  # C1..C4: even degree 8 (error ~5e-8)
 # chunk-anchored loops: (suffix, range, sine terms, cosine terms); the ranges
 # are the reduced anchor's plus the largest offset the kernels allow (anchored.cuh)
-ANCHORED = (("A", math.pi / 2 + 0.25 + 1e-3, 4, 5), ("Q", math.pi / 4 + 0.15 + 1e-3, 3, 4))
+ANCHORED = (("A", math.pi / 2 + 0.25 + 1e-3, 4, 5), ("Q", math.pi / 4 + 0.4 + 1e-3, 4, 4))
 
 # pi to 60 digits (textbook value)
 PI = Fraction("3.14159265358979323846264338327950288419716939937510582097494")

@@ -5,6 +5,8 @@
 #include <mutex>
 
 #include "general.cuh"
+#include "general_nodes.cuh"
+#include "slices.cuh"
 
 namespace gna {
 
@@ -97,6 +99,8 @@ __device__ void general_coefficients(const gna_osc_full& o, int alpha, int beta,
         gc.b[k] = sb * X.im.v;
         gc.af[k] = (float)gc.a[k];
         gc.bf[k] = (float)gc.b[k];
+        gc.alo[k] = (float)(gc.a[k] - (double)gc.af[k]);
+        gc.blo[k] = (float)(gc.b[k] - (double)gc.bf[k]);
         for (int q = 0; q < 4; q++) {
             gc.da[q][k] = -4.0 * X.re.d[q];
             gc.db[q][k] = sb * X.im.d[q];
@@ -156,26 +160,26 @@ cudaError_t launch_prepare_general(const gna_osc_full* prm, int npts, const Base
 }
 
 // ------------------------------------------------------------ launchers ----
-template <int PH, int NL, bool GRAD, bool SURV>
-static cudaError_t launch_gen(const GenArgs& a, int grid, int block, cudaStream_t s) {
-    return launch_dependent(k_fused_bins_gen<PH, NL, GRAD, SURV>, a, grid, block, s);
-}
-
+// Fits.
 template <int PH, int NL>
-static cudaError_t launch_gen_nl(bool grad, bool surv, const GenArgs& a, int grid, int block, cudaStream_t s) {
-    if (grad) return surv ? launch_gen<PH, NL, true, true>(a, grid, block, s) : launch_gen<PH, NL, true, false>(a, grid, block, s);
-    return surv ? launch_gen<PH, NL, false, true>(a, grid, block, s) : launch_gen<PH, NL, false, false>(a, grid, block, s);
+static cudaError_t launch_gen_fit(bool surv, const GenArgs& a, int grid, int block, cudaStream_t s) {
+    return surv ? launch_dependent(k_fit_bins_gen<PH, NL, true>, a, grid, block, s)
+                : launch_dependent(k_fit_bins_gen<PH, NL, false>, a, grid, block, s);
 }
 
 template <int PH>
-static cudaError_t dispatch_gen_ph(int nl, bool grad, bool surv, const GenArgs& a, int grid, int block, cudaStream_t s) {
+static cudaError_t dispatch_gen_fit(int nl, bool surv, const GenArgs& a, int grid, int block, cudaStream_t s) {
     switch (nl) {
-        case 1: return launch_gen_nl<PH, 1>(grad, surv, a, grid, block, s);
-        case 2: return launch_gen_nl<PH, 2>(grad, surv, a, grid, block, s);
-        case 4: return launch_gen_nl<PH, 4>(grad, surv, a, grid, block, s);
-        case 8: return launch_gen_nl<PH, 8>(grad, surv, a, grid, block, s);
+        case 1: return launch_gen_fit<PH, 1>(surv, a, grid, block, s);
+        case 2: return launch_gen_fit<PH, 2>(surv, a, grid, block, s);
+        case 4: return launch_gen_fit<PH, 4>(surv, a, grid, block, s);
+        case 8: return launch_gen_fit<PH, 8>(surv, a, grid, block, s);
         default: return cudaErrorInvalidValue;
     }
+}
+
+cudaError_t dispatch_general_fit(int ph, int nl, bool surv, const GenArgs& a, int grid, int block, cudaStream_t s) {
+    return ph == 0 ? dispatch_gen_fit<0>(nl, surv, a, grid, block, s) : dispatch_gen_fit<1>(nl, surv, a, grid, block, s);
 }
 
 template <typename Kernel>
@@ -188,21 +192,64 @@ static int occupancy(Kernel k, int block) {
     return n > 0 ? n : 1;
 }
 
-template <int PH, int NL>
-static int resident_gen_nl(bool grad, bool surv, int block) {
-    if (grad) return surv ? occupancy(k_fused_bins_gen<PH, NL, true, true>, block) : occupancy(k_fused_bins_gen<PH, NL, true, false>, block);
-    return surv ? occupancy(k_fused_bins_gen<PH, NL, false, true>, block) : occupancy(k_fused_bins_gen<PH, NL, false, false>, block);
-}
-
 template <int PH>
-static int resident_gen_ph(int nl, bool grad, bool surv, int block) {
+static int fit_ctas(int nl, bool surv, int block) {
     switch (nl) {
-        case 1: return resident_gen_nl<PH, 1>(grad, surv, block);
-        case 2: return resident_gen_nl<PH, 2>(grad, surv, block);
-        case 4: return resident_gen_nl<PH, 4>(grad, surv, block);
-        case 8: return resident_gen_nl<PH, 8>(grad, surv, block);
+        case 1: return surv ? occupancy(k_fit_bins_gen<PH, 1, true>, block) : occupancy(k_fit_bins_gen<PH, 1, false>, block);
+        case 2: return surv ? occupancy(k_fit_bins_gen<PH, 2, true>, block) : occupancy(k_fit_bins_gen<PH, 2, false>, block);
+        case 4: return surv ? occupancy(k_fit_bins_gen<PH, 4, true>, block) : occupancy(k_fit_bins_gen<PH, 4, false>, block);
+        case 8: return surv ? occupancy(k_fit_bins_gen<PH, 8, true>, block) : occupancy(k_fit_bins_gen<PH, 8, false>, block);
         default: return 1;
     }
+}
+int general_fit_ctas(int ph, int nl, bool surv, int block) {
+    return ph == 0 ? fit_ctas<0>(nl, surv, block) : fit_ctas<1>(nl, surv, block);
+}
+
+// Evaluations: one baseline takes two nodes per packed value, more take two or
+// four baselines at a time.
+constexpr size_t kGenSmem = 72 * 1024;  // the most a block of 128 threads takes
+template <int NP, bool GRAD>
+static size_t gen_smem(int block) {
+    return sizeof(f32x2p) * NP * gen_sums(GRAD) * (size_t)block + (size_t)block / 32 * QuadRing<kRingMulti>::kWarpBytes;
+}
+static size_t gen_one_smem(int block) { return (size_t)block / 32 * QuadRing<kRingOne>::kWarpBytes; }
+
+template <int PH, int NP, bool GRAD>
+static cudaError_t launch_gen_multi(const GenArgs& a, int grid, int block, cudaStream_t s) {
+    cudaError_t e = allow_smem<k_gen_multi<PH, NP, GRAD>>(kGenSmem);
+    if (e != cudaSuccess) return e;
+    return launch_dependent(k_gen_multi<PH, NP, GRAD>, a, grid, block, s, gen_smem<NP, GRAD>(block));
+}
+
+template <int PH, bool GRAD>
+static cudaError_t launch_gen(const GenArgs& a, int grid, int block, cudaStream_t s) {
+    if (a.b.nL <= 1) return launch_dependent(k_gen_one<PH, GRAD>, a, grid, block, s, gen_one_smem(block));
+    if (a.b.nL <= 2) return launch_gen_multi<PH, 1, GRAD>(a, grid, block, s);
+    return launch_gen_multi<PH, 2, GRAD>(a, grid, block, s);
+}
+
+cudaError_t dispatch_general(int ph, bool grad, const GenArgs& a, int grid, int block, cudaStream_t s) {
+    if (ph == 0) return grad ? launch_gen<0, true>(a, grid, block, s) : launch_gen<0, false>(a, grid, block, s);
+    if (ph == 1) return grad ? launch_gen<1, true>(a, grid, block, s) : launch_gen<1, false>(a, grid, block, s);
+    return cudaErrorInvalidValue;
+}
+
+template <auto K>
+static int resident_of(int block, size_t smem) {
+    int n = 0;
+    if (allow_smem<K>(kGenSmem) != cudaSuccess) return 1;
+    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, K, block, smem) != cudaSuccess) {
+        cudaGetLastError();
+        return 1;
+    }
+    return n > 0 ? n : 1;
+}
+template <int PH, bool GRAD>
+static int resident_gen(int nL, int block) {
+    if (nL <= 1) return resident_of<k_gen_one<PH, GRAD>>(block, gen_one_smem(block));
+    if (nL <= 2) return resident_of<k_gen_multi<PH, 1, GRAD>>(block, gen_smem<1, GRAD>(block));
+    return resident_of<k_gen_multi<PH, 2, GRAD>>(block, gen_smem<2, GRAD>(block));
 }
 
 static int resident_gen64(int nl, bool grad, int block) {
@@ -226,9 +273,10 @@ static int resident_gen64(int nl, bool grad, int block) {
     return n > 0 ? n : 1;
 }
 
-int general_resident_ctas(int ph, int nl, bool grad, bool surv, int block) {
+int general_resident_ctas(int ph, int nl, int nL, bool grad, int block) {
     if (ph == 2) return resident_gen64(nl, grad, block);
-    return ph == 0 ? resident_gen_ph<0>(nl, grad, surv, block) : resident_gen_ph<1>(nl, grad, surv, block);
+    if (ph == 0) return grad ? resident_gen<0, true>(nL, block) : resident_gen<0, false>(nL, block);
+    return grad ? resident_gen<1, true>(nL, block) : resident_gen<1, false>(nL, block);
 }
 
 template <int NL, bool GRAD>
@@ -251,39 +299,29 @@ cudaError_t dispatch_general64(int nl, bool grad, const GenArgs64& a, int grid, 
     }
 }
 
-cudaError_t dispatch_general(int ph, int nl, bool grad, bool surv, const GenArgs& a, int grid, int block,
-                             cudaStream_t s) {
-    if (ph == 0) return dispatch_gen_ph<0>(nl, grad, surv, a, grid, block, s);
-    if (ph == 1) return dispatch_gen_ph<1>(nl, grad, surv, a, grid, block, s);
-    return cudaErrorInvalidValue;
+template <int NVM, int W>
+static cudaError_t launch_gen_reduce(const float2* part, int S, int NV, const EpiArgs& ea, const GenConst* gc, int npts,
+                                     cudaStream_t s) {
+    cudaError_t e = allow_smem<k_gen_slices_reduce<NVM, W>>(sizeof(float2) * (W + 1) * NVM * 32);
+    if (e != cudaSuccess) return e;
+    return launch_blocks(k_gen_slices_reduce<NVM, W>, (int64_t)npts * ea.ngroups, W * 32,
+                         sizeof(float2) * (W + 1) * NV * 32, s, part, S, NV, ea, gc);
 }
 
 cudaError_t launch_slices_reduce_general(const float2* part, int S, int NV, const EpiArgs& ea, const GenConst* gc,
                                          int npts, cudaStream_t s) {
-    constexpr int W = 24;
-    if (NV != gen_nv(false) && NV != gen_nv(true)) return cudaErrorInvalidValue;
-    static std::once_flag once[64];
-    static cudaError_t attr[64];
-    int dev = 0;
-    cudaError_t e = cudaGetDevice(&dev);
+    if (NV == gen_sums(false)) return launch_gen_reduce<6, 32>(part, S, NV, ea, gc, npts, s);
+    if (NV == gen_sums(true)) return launch_gen_reduce<12, 24>(part, S, NV, ea, gc, npts, s);
+    return cudaErrorInvalidValue;
+}
+
+cudaError_t launch_fit_slices_reduce_general(const float2* part, int S, const EpiArgs& ea, const GenConst* gc, int npts,
+                                             cudaStream_t s) {
+    constexpr int W = 24, NV = gen_nv(true);
+    constexpr size_t smem = sizeof(float2) * W * NV * 32 + sizeof(double) * NV * 32;
+    cudaError_t e = allow_smem<k_fit_slices_reduce_gen<W>>(smem);
     if (e != cudaSuccess) return e;
-    if (dev < 0 || dev >= 64) return cudaErrorInvalidDevice;
-    std::call_once(once[dev], [&] {
-        attr[dev] = cudaFuncSetAttribute(k_slices_reduce_gen<W>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                         (int)(sizeof(float2) * W * gen_nv(true) * 32 + sizeof(double) * gen_nv(true) * 32));
-    });
-    if (attr[dev] != cudaSuccess) return attr[dev];
-    cudaLaunchConfig_t cfg{};
-    cfg.gridDim = dim3((unsigned)((int64_t)npts * ea.ngroups));
-    cfg.blockDim = dim3(W * 32);
-    cfg.dynamicSmemBytes = sizeof(float2) * W * NV * 32 + sizeof(double) * NV * 32;
-    cfg.stream = s;
-    cudaLaunchAttribute at[1];
-    at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-    at[0].val.programmaticStreamSerializationAllowed = 1;
-    cfg.attrs = at;
-    cfg.numAttrs = 1;
-    return cudaLaunchKernelEx(&cfg, k_slices_reduce_gen<W>, part, S, NV, ea, gc);
+    return launch_blocks(k_fit_slices_reduce_gen<W>, (int64_t)npts * ea.ngroups, W * 32, smem, s, part, S, NV, ea, gc);
 }
 
 }  // namespace gna

@@ -50,6 +50,7 @@ struct GenConst {
     // FP32 copies for the gradient terms (FP64 instructions run at 1/64 of
     // the FP32 rate on this part; the gradient is held to 1e-4)
     float af[3], bf[3], daf[4][3], dbf[4][3];
+    float alo[3], blo[3];  // a - (double)af, b - (double)bf
     // sum_r omega_r as the mixed node pass applies the FP32 weights (hi + lo)
     double wsum;
 };
@@ -116,8 +117,9 @@ __device__ __forceinline__ void sincos_quadrant(float r, bool odd, float& s, flo
 // quadrant swaps, so that cos x near its zeros (the cos^2 sums there) keeps
 // its relative accuracy; other channels reduce modulo pi (P stays well above
 // the cos^2 errors there).
-template <int PH, int NL, bool GRAD, bool SURV>
+template <int PH, int NL, bool SURV>
 struct NodeMathGen {
+    static constexpr bool GRAD = true;
     static constexpr int NV = gen_nv(GRAD);
     // with several baselines the weights enter as hi + lo (no bias from the
     // FP32 rounding of omega_r)
@@ -341,11 +343,12 @@ static __device__ __noinline__ void gen_group_done(const EpiArgs& a, int p, int 
     }
 }
 
-// Node kernel of the general channel, bin and slice mappings: the task scheme
-// and node loop of k_fused_bins with the channel-free sums above.
-template <int PH, int NL, bool GRAD, bool SURV>
-__global__ void __launch_bounds__(256) k_fused_bins_gen(GenArgs ga) {
-    using M = NodeMathGen<PH, NL, GRAD, SURV>;
+// Node kernel of the general channel's fits, bin and slice mappings: the task
+// scheme and node loop of k_fit_bins (and its reason) with the channel-free
+// sums above.  Evaluations use the kernels of general_nodes.cuh.
+template <int PH, int NL, bool SURV>
+__global__ void __launch_bounds__(256) k_fit_bins_gen(GenArgs ga) {
+    using M = NodeMathGen<PH, NL, SURV>;
     constexpr int NV = M::NV;
     const BinArgs& a = ga.b;
     const int lane = threadIdx.x & 31;
@@ -425,10 +428,10 @@ __global__ void __launch_bounds__(256) k_fused_bins_gen(GenArgs ga) {
 }
 
 // Slice sums of the general channel (NV = 9 or 15 values), in slice order,
-// then the epilogue and the group and point reductions: k_slices_reduce with
-// the general epilogue.
+// then the epilogue and the group and point reductions: k_fit_slices_reduce
+// with the general epilogue.
 template <int W>
-__global__ void __launch_bounds__(W * 32) k_slices_reduce_gen(const float2* __restrict__ part, int S, int NV,
+__global__ void __launch_bounds__(W * 32) k_fit_slices_reduce_gen(const float2* __restrict__ part, int S, int NV,
                                                                EpiArgs ea, const GenConst* __restrict__ gc) {
     constexpr int NVM = gen_nv(true);
     extern __shared__ float2 red[];  // [W][NV][32], then [NV][32] doubles
@@ -621,11 +624,16 @@ __global__ void __launch_bounds__(256) k_fused64_bins_gen(GenArgs64 ga) {
 cudaError_t launch_prepare_general(const gna_osc_full* prm, int npts, const BaseConst& bc, int alpha, int beta,
                                    int anti, PointConst* out, GenConst* gout, int* zero, int64_t nz, int* status,
                                    cudaStream_t s);
-cudaError_t dispatch_general(int ph, int nl, bool grad, bool surv, const GenArgs& a, int grid, int block,
-                             cudaStream_t s);
-int general_resident_ctas(int ph, int nl, bool grad, bool surv, int block);
-cudaError_t dispatch_general64(int nl, bool grad, const GenArgs64& a, int grid, int block, cudaStream_t s);
+// node kernel of an evaluation (ph 0 or 1; blocks of at most 128 threads)
+cudaError_t dispatch_general(int ph, bool grad, const GenArgs& a, int grid, int block, cudaStream_t s);
+int general_resident_ctas(int ph, int nl, int nL, bool grad, int block);
 cudaError_t launch_slices_reduce_general(const float2* part, int S, int NV, const EpiArgs& ea, const GenConst* gc,
                                          int npts, cudaStream_t s);
+// of a fit's iteration (ph 0 or 1)
+cudaError_t dispatch_general_fit(int ph, int nl, bool surv, const GenArgs& a, int grid, int block, cudaStream_t s);
+int general_fit_ctas(int ph, int nl, bool surv, int block);
+cudaError_t launch_fit_slices_reduce_general(const float2* part, int S, const EpiArgs& ea, const GenConst* gc, int npts,
+                                             cudaStream_t s);
+cudaError_t dispatch_general64(int nl, bool grad, const GenArgs64& a, int grid, int block, cudaStream_t s);
 
 }  // namespace gna

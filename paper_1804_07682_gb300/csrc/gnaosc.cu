@@ -22,6 +22,7 @@
 #include "fused.cuh"
 #include "fused64.cuh"
 #include "general.cuh"
+#include "general_nodes.cuh"
 #include "gnaosc.h"
 #include "misc.h"
 
@@ -315,11 +316,11 @@ int resident_ctas_per_sm(const gna_plan* p, bool grad, bool spec) {
 
 // Resident blocks per SM of the node kernel of the bin and slice mappings
 // (asked of the runtime once per block size).
-int node_ctas_per_sm(gna_plan* p, bool grad, bool surv, int block) {
+int node_ctas_per_sm(gna_plan* p, bool grad, int block) {
     if (p->grid_mult > 0) return p->grid_mult;
     int& n = p->res_ctas[grad];
     if (n == 0 || p->res_block[grad] != block) {
-        n = p->general ? general_resident_ctas(p->ph, p->nl_inst, grad, surv, block)
+        n = p->general ? general_resident_ctas(p->ph, p->nl_inst, p->nL, grad, block)
             : p->ph < 2 ? nodes_resident_ctas(p->ph, p->nL, grad, block)
                         : std::max(1, 1024 / block);
         p->res_block[grad] = block;
@@ -439,8 +440,8 @@ EpiArgs make_epi(const gna_plan* plan, const EvalReq& q, bool grad, bool spec, i
     return ea;
 }
 
-// Slice mapping of the fits and the any-channel chain: a slice length for
-// about two tasks per resident warp (16 per SM).
+// Slice mapping of the fits: a slice length for about two tasks per resident
+// warp (16 per SM).
 SliceShape fixed_slice_shape(const gna_plan* p) {
     const int n = p->n_uniform;
     const int64_t pg = (int64_t)p->npts * p->ngroups;
@@ -499,7 +500,7 @@ gna_status enqueue_eval(gna_plan* plan, const EvalReq& q, cudaStream_t s, int* l
     }
     SliceShape ssh{1, 0, plan->ntasks};
     const int nblock = plan->ph < 2 ? nodes_block(plan->block) : plan->block;
-    const int ctas = split ? 0 : node_ctas_per_sm(plan, grad, false, nblock);
+    const int ctas = split ? 0 : node_ctas_per_sm(plan, grad, nblock);
     if (plan->mapping == MAP_SLICES && !fit) {
         ssh = slice_shape(plan, (int64_t)plan->sm_count * ctas * (nblock / 32));
         if ((int64_t)plan->npts * plan->ngroups * ssh.S >= (1LL << 31)) return fail(plan, GNA_ESHAPE, "too many slice tasks");
@@ -544,7 +545,7 @@ gna_status enqueue_eval(gna_plan* plan, const EvalReq& q, cudaStream_t s, int* l
             if (sliced) {
                 CU(launch_slices_reduce(plan->d_slices, ssh.S, NVs, ea, plan->d_pc, plan->npts, s));
             } else {
-                CU(launch_point_sums(ea, s));
+                CU(launch_point_sums(4, ea, s));
             }
             nl++;
         } else {
@@ -572,12 +573,14 @@ gna_status enqueue_eval(gna_plan* plan, const EvalReq& q, cudaStream_t s, int* l
 // q.H set for the fits' J^T W J); counts kernel launches into *launches.
 gna_status enqueue_eval_general(gna_plan* plan, const EvalReq& q, cudaStream_t s, int* launches) {
     const bool grad = q.grad || q.grad_eta || q.H;
-    const bool surv = plan->g_alpha == plan->g_beta;  // survival channel: phases modulo pi/2 (general.cuh)
-    const int NV = gen_nv(grad);
+    const bool fit = q.H && plan->ph < 2;           // the fits' own node kernel (general.cuh)
+    const bool surv = plan->g_alpha == plan->g_beta;  // survival channel: the fits reduce phases modulo pi/2
+    const int NV = fit ? gen_nv(true) : gen_sums(grad);
+    const int nblock = (plan->ph < 2 && !fit) ? nodes_block(plan->block) : plan->block;
+    const int ctas = fit ? general_fit_ctas(plan->ph, plan->nl_inst, surv, nblock) : node_ctas_per_sm(plan, grad, nblock);
     SliceShape ssh{1, 0, plan->ntasks};
-    const int ctas = node_ctas_per_sm(plan, grad, surv, plan->block);
     if (plan->mapping == MAP_SLICES) {
-        ssh = fixed_slice_shape(plan);
+        ssh = fit ? fixed_slice_shape(plan) : slice_shape(plan, (int64_t)plan->sm_count * ctas * (nblock / 32));
         if ((int64_t)plan->npts * plan->ngroups * ssh.S >= (1LL << 31)) return fail(plan, GNA_ESHAPE, "too many slice tasks");
     }
     const int64_t ncnt = 1 + (int64_t)plan->npts * (1 + plan->ngroups);
@@ -587,25 +590,29 @@ gna_status enqueue_eval_general(gna_plan* plan, const EvalReq& q, cudaStream_t s
     ea.NBV = q.H ? kGenNBVFit : (grad ? 7 : 1);  // chi2, the six-parameter gradient terms, J^T W J
     ea.binsums = nullptr;
     const bool sliced = ssh.S > 1;
-    const int g = grid_size(plan, ctas, plan->block, ssh.ntasks);
+    const int g = grid_size(plan, ctas, nblock, ssh.ntasks);
+    *launches = 2;
     if (plan->ph == 2) {
         GenArgs64 ga64{BinArgs64{plan->grid64_bins, plan->d_goff, plan->d_gn, plan->d_gid, plan->d_tasks, plan->ntasks,
                                  plan->ngroups, plan->nbins, plan->d_pc, plan->bc, plan->d_counters, ea},
                        plan->d_gc};
-        CU(dispatch_general64(plan->nl_inst, grad, ga64, g, plan->block, s));
-        *launches = 2;
+        CU(dispatch_general64(plan->nl_inst, grad, ga64, g, nblock, s));
         return GNA_OK;
     }
-    GenArgs ga{BinArgs{plan->grid_bins, nullptr, plan->d_goff, plan->d_gn, plan->d_gid, plan->d_tasks, nullptr, ssh.ntasks,
-                       plan->ngroups, plan->nbins, plan->d_pc, plan->bc, plan->d_counters, ea, ssh.S, ssh.L,
-                       sliced ? plan->d_slices : nullptr, NV, plan->nL, 0, plan->d_step},
+    GenArgs ga{BinArgs{plan->grid_bins, plan->grid_rec, plan->d_goff, plan->d_gn, plan->d_gid, plan->d_tasks, plan->d_desc,
+                       ssh.ntasks, plan->ngroups, plan->nbins, plan->d_pc, plan->bc, plan->d_counters, ea, ssh.S,
+                       fit ? ssh.L : ssh.L / 4, sliced ? plan->d_slices : nullptr, NV, plan->nL, 0, plan->d_step},
                plan->d_gc};
-    CU(dispatch_general(plan->ph, plan->nl_inst, grad, surv, ga, g, plan->block, s));
-    *launches = 2;
-    if (sliced) {
-        CU(launch_slices_reduce_general(plan->d_slices, ssh.S, NV, ea, plan->d_gc, plan->npts, s));
-        *launches = 3;
+    if (fit) {
+        CU(dispatch_general_fit(plan->ph, plan->nl_inst, surv, ga, g, nblock, s));
+        if (sliced) CU(launch_fit_slices_reduce_general(plan->d_slices, ssh.S, ea, plan->d_gc, plan->npts, s));
+        *launches = sliced ? 3 : 2;
+        return GNA_OK;
     }
+    CU(dispatch_general(plan->ph, grad, ga, g, nblock, s));
+    if (sliced) CU(launch_slices_reduce_general(plan->d_slices, ssh.S, NV, ea, plan->d_gc, plan->npts, s));
+    else CU(launch_point_sums(6, ea, s));
+    *launches = 3;
     return GNA_OK;
 }
 
@@ -988,6 +995,7 @@ static gna_status plan_build(gna_plan* plan, const gna_plan_desc* d, cudaStream_
     for (int r = 0; r < d->nL; r++) {
         bc.omd[r] = plan->omega[r];
         bc.kld[r] = GNA_K_PHASE * d->L[r];
+        bc.klmax = std::max(bc.klmax, bc.kld[r]);
         bc.om[r] = (float)plan->omega[r];
         bc.omlo[r] = (float)(plan->omega[r] - (double)bc.om[r]);
         bc.wkl[r] = (float)(2.0 * plan->omega[r] * bc.kld[r]);
@@ -1040,7 +1048,7 @@ static gna_status plan_build(gna_plan* plan, const gna_plan_desc* d, cudaStream_
         gid[p] = (int)(std::lower_bound(gn.begin(), gn.end(), plan->counts[p]) - gn.begin());
     const int nbins_pad = ngroups * 32;
     // grid offsets of the bins layout (the split layout is one bin-major grid)
-    const bool quads = plan->ph < 2 && !plan->general;  // nodes also stored in quads
+    const bool quads = plan->ph < 2;  // nodes also stored in quads
     std::vector<int64_t> qoff(plan->ngrids);            // first quad of each grid
     int64_t nquads = 0;
     for (int g = 0; g < plan->ngrids; g++) {
@@ -1843,11 +1851,14 @@ gna_status gna_plan_autotune_general(gna_plan* plan, const gna_osc_full* params,
     std::vector<std::string> cand;
     char t[96];
     for (int b : {64, 128, 256}) {
+        if (plan->ph < 2 && b > 128) continue;  // the mixed kernels take blocks of at most 128 threads
         if (plan->mapping == MAP_BINS) {
             snprintf(t, sizeof(t), "mapping=bins block=%d", b);
             cand.push_back(t);
         } else {
             const int64_t pg = (int64_t)plan->npts * plan->ngroups;
+            snprintf(t, sizeof(t), "mapping=slices block=%d slice=0", b);
+            cand.push_back(t);
             for (int tpw : {1, 2, 4}) {
                 const int64_t S = std::max<int64_t>(1, ((int64_t)tpw * 16 * plan->sm_count + pg - 1) / pg);
                 const int64_t L = std::min<int64_t>(plan->n_uniform, (plan->n_uniform + S - 1) / S);

@@ -8,109 +8,40 @@
 #include "anchored.cuh"
 #include "dispatch.h"
 #include "epilogue.cuh"
+#include "slices.cuh"
 
 namespace gna {
 
-// One block of W warps per (point, group).  Warp w sums slices w, w + W, ...
-// in order for every value (lane l: bin 32 g + l; the loads of a slice for
-// all values are in flight together); the warps' sums are then added in warp
-// order through shared memory, one value per warp, and warp 0 runs the
-// epilogue of the group.  The fixed order makes the result independent of
-// timing.  NVM bounds the value count so that the per-lane arrays stay in
-// registers: 32 warps for up to 6 values, 24 for up to 14, 16 beyond.
+// One block of W warps per (point, group); warp 0 runs the epilogue of the
+// group: 32 warps for up to 6 values, 24 for up to 14, 16 beyond.
 template <int NVM, int W>
 __global__ void __launch_bounds__(W * 32) k_slices_reduce(const float2* __restrict__ part, int S, int NV, EpiArgs ea,
                                                           const PointConst* __restrict__ pcs) {
-    extern __shared__ float2 red[];  // [W][NV][32], then [NV][32]
-    float2* fin = red + W * NV * 32;
-    const int pg = blockIdx.x;
-    const int p = pg / ea.ngroups;
-    const int g = pg - p * ea.ngroups;
-    const int w = threadIdx.x >> 5;
-    const int lane = threadIdx.x & 31;
-    // the next evaluation's first kernel may be placed now; it waits for this
-    // kernel to complete before it touches anything
-    asm volatile("griddepcontrol.launch_dependents;");
-    float2 acc[NVM];
-#pragma unroll
-    for (int v = 0; v < NVM; v++) acc[v] = make_float2(0.f, 0.f);
+    const int p = blockIdx.x / ea.ngroups, g = blockIdx.x - p * ea.ngroups;
+    const int w = threadIdx.x >> 5, lane = threadIdx.x & 31;
     // the epilogue's inputs do not depend on the node kernel: load them first
     const int i = g * 32 + lane;
     BinInput in;
     if (w == 0) in = bin_input(ea, p, min(i, ea.nbins - 1));
-    // launched as a programmatic dependent of the node kernel: the blocks may
-    // be resident before it ends; wait (in hardware) until it has completed
-    // and its writes are visible
-    asm volatile("griddepcontrol.wait;" ::: "memory");
-    const float2* base = part + (int64_t)pg * S * NV * 32 + lane;
-    const int64_t stride = (int64_t)NV * 32;
-    for (int sl = w; sl < S; sl += W) {
-        const float2* src = base + sl * stride;
-        float2 t[NVM];
-#pragma unroll
-        for (int v = 0; v < NVM; v++) t[v] = (v < NV) ? __ldg(src + v * 32) : make_float2(0.f, 0.f);
-#pragma unroll
-        for (int v = 0; v < NVM; v++)
-            if (v < NV) acc[v] = ff_add(acc[v], t[v]);
-    }
-#pragma unroll
-    for (int v = 0; v < NVM; v++)
-        if (v < NV) red[(w * NV + v) * 32 + lane] = acc[v];
-    __syncthreads();
-    const int used = min(W, S);  // warps that had a slice
-    for (int v = w; v < NV; v += W) {
-        float2 sum = red[v * 32 + lane];
-        for (int k = 1; k < used; k++) sum = ff_add(sum, red[(k * NV + v) * 32 + lane]);
-        fin[v * 32 + lane] = sum;
-    }
-    __syncthreads();
+    const float2* fin = sum_slices<NVM, W>(part, S, NV, w, lane);
     if (w == 0) {
         // the task sums T, N (anchored.cuh), then the per-baseline parts
         TaskSums q;
         float2 sp[GNA_NLMAX];
-        float2 regs[5];
         for (int j = 0; j < 3; j++) q.T[j] = fin[j * 32 + lane];
         const int from = ea.has_grad ? 6 : 3;
         for (int r = 0; r < ea.nspec; r++) sp[r] = fin[(from + r) * 32 + lane];
         if (ea.has_grad) {
             for (int j = 0; j < 3; j++) q.N[j] = fin[(3 + j) * 32 + lane].x + fin[(3 + j) * 32 + lane].y;
-            if (i < ea.nbins) bin_terms<true>(ea, p, i, bin_sums<true>(pcs + p, in.sumw, q), sp, in, regs);
-            group_done_terms<true>(ea, p, g, lane, regs);
+            float2 regs[5];
+            if (i < ea.nbins) bin_terms<4>(ea, p, i, bin_sums<true>(pcs + p, in.sumw, q), sp, in, regs);
+            group_done_terms<4>(ea, p, g, lane, regs);
         } else {
-            if (i < ea.nbins) bin_terms<false>(ea, p, i, bin_sums<false>(pcs + p, in.sumw, q), sp, in, regs);
-            group_done_terms<false>(ea, p, g, lane, regs);
+            float2 regs[1];
+            if (i < ea.nbins) bin_terms<0>(ea, p, i, bin_sums<false>(pcs + p, in.sumw, q), sp, in, regs);
+            group_done_terms<0>(ea, p, g, lane, regs);
         }
     }
-}
-
-// More than the default 48 KB of dynamic shared memory: opt in once per device.
-template <auto K>
-cudaError_t allow_smem(size_t bytes) {
-    static std::once_flag once[64];
-    static cudaError_t attr[64];
-    int dev = 0;
-    cudaError_t e = cudaGetDevice(&dev);
-    if (e != cudaSuccess) return e;
-    if (dev < 0 || dev >= 64) return cudaErrorInvalidDevice;
-    std::call_once(once[dev], [&] {
-        attr[dev] = cudaFuncSetAttribute(K, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
-    });
-    return attr[dev];
-}
-
-template <typename... Args>
-cudaError_t launch_blocks(void (*k)(Args...), int64_t blocks, int threads, size_t smem, cudaStream_t s, Args... args) {
-    cudaLaunchConfig_t cfg{};
-    cfg.gridDim = dim3((unsigned)blocks);
-    cfg.blockDim = dim3(threads);
-    cfg.dynamicSmemBytes = smem;
-    cfg.stream = s;
-    cudaLaunchAttribute at[1];
-    at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-    at[0].val.programmaticStreamSerializationAllowed = 1;
-    cfg.attrs = at;
-    cfg.numAttrs = 1;
-    return cudaLaunchKernelEx(&cfg, k, args...);
 }
 
 template <int NVM, int W>
@@ -194,20 +125,21 @@ cudaError_t launch_fit_slices_reduce(const float2* part, int S, const EpiArgs& e
 
 // After whole-bin tasks of the anchored kernels: one warp per point sums its
 // groups and writes its outputs.
+template <int NG>
 __global__ void __launch_bounds__(256) k_point_sums(EpiArgs ea) {
     asm volatile("griddepcontrol.launch_dependents;");
     const int p = (int)(((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5);
     asm volatile("griddepcontrol.wait;" ::: "memory");
-    if (p < ea.npts) point_reduce<8>(ea, p, threadIdx.x & 31);
+    if (p < ea.npts) point_reduce<8, NG>(ea, p, threadIdx.x & 31);
 }
 
-cudaError_t launch_point_sums(const EpiArgs& ea, cudaStream_t s) {
-    return launch_blocks(k_point_sums, ((int64_t)ea.npts * 32 + 255) / 256, 256, 0, s, ea);
+cudaError_t launch_point_sums(int npar, const EpiArgs& ea, cudaStream_t s) {
+    return launch_blocks(npar == 6 ? k_point_sums<6> : k_point_sums<4>, ((int64_t)ea.npts * 32 + 255) / 256, 256, 0, s, ea);
 }
 
 // Epilogue-only evaluation (steps a7-a9) on the node sums an evaluation in
 // the anchored kernels kept (as k_cached_epilogue below).
-template <bool GRAD>
+template <int NG>
 __global__ void __launch_bounds__(256) k_cached_terms(const float2* __restrict__ sums, EpiArgs ea) {
     const int64_t wid = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
     const int lane = threadIdx.x & 31;
@@ -215,26 +147,25 @@ __global__ void __launch_bounds__(256) k_cached_terms(const float2* __restrict__
     const int p = (int)(wid / ea.ngroups);
     const int g = (int)(wid - (int64_t)p * ea.ngroups);
     const int i = g * 32 + lane;
-    float2 regs[5];
+    float2 regs[1 + NG];
     if (i < ea.nbins) {
         const float2* src = sums + ((int64_t)p * ea.nbins + i) * ea.NV;
-        BinSums b;
+        BinSums<NG> b;
         b.M = src[0];
-        if (GRAD) {
-            b.v[0] = src[1].x;
-            b.v[1] = src[1].y;
-            b.v[2] = src[2].x;
-            b.v[3] = src[2].y;
+#pragma unroll
+        for (int q = 0; q < NG; q += 2) {
+            b.d[q] = src[1 + q / 2].x;
+            b.d[q + 1] = src[1 + q / 2].y;
         }
-        bin_terms<GRAD>(ea, p, i, b, src + (GRAD ? 3 : 1), bin_input(ea, p, i), regs);
+        bin_terms<NG>(ea, p, i, b, src + 1 + NG / 2, bin_input(ea, p, i), regs);
     }
-    group_done_terms<GRAD>(ea, p, g, lane, regs);
+    group_done_terms<NG>(ea, p, g, lane, regs);
 }
 
 cudaError_t launch_cached_terms(const float2* sums, const EpiArgs& ea, cudaStream_t s) {
     const unsigned blocks = (unsigned)(((int64_t)ea.npts * ea.ngroups * 32 + 255) / 256);
-    if (ea.has_grad) k_cached_terms<true><<<blocks, 256, 0, s>>>(sums, ea);
-    else k_cached_terms<false><<<blocks, 256, 0, s>>>(sums, ea);
+    if (ea.has_grad) k_cached_terms<4><<<blocks, 256, 0, s>>>(sums, ea);
+    else k_cached_terms<0><<<blocks, 256, 0, s>>>(sums, ea);
     return cudaGetLastError();
 }
 

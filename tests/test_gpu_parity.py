@@ -1087,3 +1087,38 @@ def test_anchored_chunks(api, prec, mapping, nL, n, edges):
     for o in (out, alone):  # few nodes per bin: the scaled bound (see the module's head)
         check_chi2(o["chi2"][0].item(), ref, data, wl.POISSON, 1e-6, tag="anchored %d %d" % (nL, n), plain=False)
     plan.close()
+
+
+@pytest.mark.parametrize("prec", ["f64phase", "ff"])
+@pytest.mark.parametrize("nL", [1, 2, 3, 5])
+@pytest.mark.parametrize("channel", [("mu", "e", False), ("mu", "mu", True), ("e", "tau", False)])
+@pytest.mark.parametrize("n,edges", [(1, (600.0, 4000.0)), (3, (600.0, 4000.0)), (5, (1500.0, 2000.0)), (34, (1500.0, 2000.0)),
+                                     (131, (1500.0, 2000.0)), (21, (150.0, 3000.0))])
+def test_general_anchored_chunks(api, prec, nL, channel, n, edges):
+    # as test_anchored_chunks for the any-channel node kernels: single nodes,
+    # quads, chunks and ragged ends, coarse and fine grids, both mappings
+    rng = np.random.default_rng(nL + n)
+    e = np.linspace(edges[0], edges[1], 38)
+    L = np.array([810.0, 295.0, 735.0, 700.0, 280.0])[:nL]
+    th = np.array(THETA_FULL) * 1.02
+    a, b, anti = channel
+    mu_rb, _ = oracle.binned_general(e, n, L, THETA_FULL, a, b, anti, 1e-3)
+    M = oracle.baseline_weights(L) @ mu_rb
+    Nn = 1e4 / M.sum()
+    data = wl.poisson_data(Nn * M, 3)
+    ref = oracle.chain_general(e, n, L, th, Nn, data, a, b, anti, 1, None, 0.0, 1e-3)
+    for mapping in ("bins", "slices"):
+        plan = api.Plan(e, L, nodes_per_bin=n, norm=Nn, e_scale=1e-3, prec=prec, kind="poisson", channel=channel,
+                        mapping="bins" if mapping == "bins" else None)
+        if mapping == "slices":
+            plan.tuning = "slice=16"
+        p, d = plan.params_tensor(th), dev(data)
+        out = plan.eval_general(p, d, grad=True, mu=True)
+        alone = plan.eval_general(p, d, grad=False)
+        torch.cuda.synchronize()
+        plan.status()
+        assert rel(out["mu"][0].cpu().numpy(), ref["mu"]) < 1e-6
+        assert normrel(out["grad"][0].cpu().numpy(), ref["grad"][:6]) < 1e-4
+        for o in (out, alone):
+            check_chi2(o["chi2"][0].item(), ref, data, wl.POISSON, 1e-6, tag="general anchored %d %d" % (nL, n), plain=False)
+        plan.close()
