@@ -148,9 +148,10 @@ struct BinArgs64 {
     EpiArgs ea;
 };
 
-template <int NL, bool GRAD, bool SPEC>
-__global__ void __launch_bounds__(256) k_fused64_bins(BinArgs64 a) {
-    using M = NodeMath64<NL, GRAD, SPEC>;
+// The fits' kernel (see k_fit_bins; evaluations use nodes64.cuh).
+template <int NL>
+__global__ void __launch_bounds__(256) k_fit64_bins(BinArgs64 a) {
+    using M = NodeMath64<NL, true, false>;
     constexpr int NV = M::NV;
     const int lane = threadIdx.x & 31;
     int last_p = -1;
@@ -187,9 +188,9 @@ cudaError_t launch_split64(const SplitArgs64& a, int grid, int block, cudaStream
     return cudaGetLastError();
 }
 
-template <int NL, bool GRAD, bool SPEC>
-cudaError_t launch_bins64(const BinArgs64& a, int grid, int block, cudaStream_t s) {
-    k_fused64_bins<NL, GRAD, SPEC><<<grid, block, 0, s>>>(a);
+template <int NL>
+cudaError_t launch_fit_bins64(const BinArgs64& a, int grid, int block, cudaStream_t s) {
+    k_fit64_bins<NL><<<grid, block, 0, s>>>(a);
     return cudaGetLastError();
 }
 

@@ -21,22 +21,11 @@ cudaError_t dispatch_split_ph2(int nl, bool grad, bool spec, const void* args, i
         default: return cudaErrorInvalidValue;
     }
 }
-cudaError_t dispatch_bins_ph2(int nl, bool grad, bool spec, const void* args, int grid, int block, cudaStream_t s) {
-    const BinArgs64& a = *static_cast<const BinArgs64*>(args);
-    const int key = nl * 4 + (grad ? 2 : 0) + (spec ? 1 : 0);
-    switch (key) {
-        case 4: return launch_bins64<1, false, false>(a, grid, block, s);
-        case 5: return launch_bins64<1, false, true>(a, grid, block, s);
-        case 6: return launch_bins64<1, true, false>(a, grid, block, s);
-        case 7: return launch_bins64<1, true, true>(a, grid, block, s);
-        case 32: return launch_bins64<8, false, false>(a, grid, block, s);
-        case 33: return launch_bins64<8, false, true>(a, grid, block, s);
-        case 34: return launch_bins64<8, true, false>(a, grid, block, s);
-        case 35: return launch_bins64<8, true, true>(a, grid, block, s);
-        case 64: return launch_bins64<16, false, false>(a, grid, block, s);
-        case 65: return launch_bins64<16, false, true>(a, grid, block, s);
-        case 66: return launch_bins64<16, true, false>(a, grid, block, s);
-        case 67: return launch_bins64<16, true, true>(a, grid, block, s);
+cudaError_t dispatch_fit_ph2(int nl, const BinArgs64& a, int grid, int block, cudaStream_t s) {
+    switch (nl) {
+        case 1: return launch_fit_bins64<1>(a, grid, block, s);
+        case 8: return launch_fit_bins64<8>(a, grid, block, s);
+        case 16: return launch_fit_bins64<16>(a, grid, block, s);
         default: return cudaErrorInvalidValue;
     }
 }

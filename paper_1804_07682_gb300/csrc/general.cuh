@@ -491,8 +491,9 @@ __global__ void __launch_bounds__(W * 32) k_fit_slices_reduce_gen(const float2* 
 // The same sums with every step in double (phases reduced modulo pi in
 // double, CUDA's double sincos), for the bin mapping on the double grids
 // {1/E, W}.
-template <int NL, bool GRAD>
+template <int NL>
 struct NodeMathGen64 {
+    static constexpr bool GRAD = true;
     // the sums of the mixed variant, then sum_k W_k (the delta_ab term; the
     // mixed precisions take it from the plan's per-bin weight sums)
     static constexpr int NV = GRAD ? 13 : 7;
@@ -586,9 +587,9 @@ __device__ inline void gen_bin_epilogue64(const EpiArgs& a, const GenConst& c, i
     if (a.grad_eta_out) a.grad_eta_out[idx] = gd * a.norm * M + (pen ? 2.0 * e / (a.sigma * a.sigma) : 0.0);
 }
 
-template <int NL, bool GRAD>
-__global__ void __launch_bounds__(256) k_fused64_bins_gen(GenArgs64 ga) {
-    using M = NodeMathGen64<NL, GRAD>;
+template <int NL>
+__global__ void __launch_bounds__(256) k_fit64_bins_gen(GenArgs64 ga) {
+    using M = NodeMathGen64<NL>;
     constexpr int NV = M::NV;
     const BinArgs64& a = ga.b;
     const int lane = threadIdx.x & 31;
@@ -626,7 +627,7 @@ cudaError_t launch_prepare_general(const gna_osc_full* prm, int npts, const Base
                                    cudaStream_t s);
 // node kernel of an evaluation (ph 0 or 1; blocks of at most 128 threads)
 cudaError_t dispatch_general(int ph, bool grad, const GenArgs& a, int grid, int block, cudaStream_t s);
-int general_resident_ctas(int ph, int nl, int nL, bool grad, int block);
+int general_resident_ctas(int ph, int nL, bool grad, int block);
 cudaError_t launch_slices_reduce_general(const float2* part, int S, int NV, const EpiArgs& ea, const GenConst* gc,
                                          int npts, cudaStream_t s);
 // of a fit's iteration (ph 0 or 1)
@@ -634,6 +635,7 @@ cudaError_t dispatch_general_fit(int ph, int nl, bool surv, const GenArgs& a, in
 int general_fit_ctas(int ph, int nl, bool surv, int block);
 cudaError_t launch_fit_slices_reduce_general(const float2* part, int S, const EpiArgs& ea, const GenConst* gc, int npts,
                                              cudaStream_t s);
-cudaError_t dispatch_general64(int nl, bool grad, const GenArgs64& a, int grid, int block, cudaStream_t s);
+cudaError_t dispatch_general_fit64(int nl, const GenArgs64& a, int grid, int block, cudaStream_t s);
+int general_fit_ctas64(int nl, int block);
 
 }  // namespace gna

@@ -25,6 +25,7 @@
 #include "general_nodes.cuh"
 #include "gnaosc.h"
 #include "misc.h"
+#include "nodes64.cuh"
 
 using namespace gna;
 
@@ -32,7 +33,7 @@ namespace gna {
 cudaError_t dispatch_split_ph0(int, bool, bool, const void*, int, int, cudaStream_t);
 cudaError_t dispatch_split_ph1(int, bool, bool, const void*, int, int, cudaStream_t);
 cudaError_t dispatch_split_ph2(int, bool, bool, const void*, int, int, cudaStream_t);
-cudaError_t dispatch_bins_ph2(int, bool, bool, const void*, int, int, cudaStream_t);
+cudaError_t dispatch_fit_ph2(int, const BinArgs64&, int, int, cudaStream_t);
 cudaError_t dispatch_fit_ph0(int, const FitArgs&, int, int, cudaStream_t);
 cudaError_t dispatch_fit_ph1(int, const FitArgs&, int, int, cudaStream_t);
 cudaError_t dispatch_nodes_ph0(bool, const BinArgs&, int, int, cudaStream_t);
@@ -101,6 +102,9 @@ struct gna_plan {
     double norm = 1.0, e_scale = 1.0;
     int prec = GNA_MIXED_FFPHASE, kind = GNA_PEARSON, flags = 0, max_datasets = 0;
     int mapping = MAP_SPLIT;
+    // GNA_FP64 plans evaluate by bins (nodes64.cuh); their fits use the split
+    // mapping where it was the default and none was asked for
+    bool fit_split = false;
     int sm_count = 0;
     // any-channel plans (GNA_PLAN_GENERAL): P(g_alpha -> g_beta), antineutrinos
     // when g_anti; their coefficients are prepared per point into d_gc
@@ -296,9 +300,9 @@ SplitShape split_shape(const gna_plan* p, bool grad, bool spec) {
 }
 
 
-// Per-baseline values of one bin's node sums: the split kernels (and
-// GNA_FP64) sum every instantiated baseline, the anchored kernels those of the plan.
-int spectra_count(const gna_plan* p, bool split) { return (split || p->ph == 2) ? p->nl_inst : p->nL; }
+// Per-baseline values of one bin's node sums: the split and fit kernels sum
+// every instantiated baseline, the others those of the plan.
+int spectra_count(const gna_plan* p, bool split) { return split ? p->nl_inst : p->nL; }
 int value_count(const gna_plan* p, bool grad, bool spec, bool split) {
     return fused_nv(spectra_count(p, split), grad, spec);
 }
@@ -314,15 +318,13 @@ int resident_ctas_per_sm(const gna_plan* p, bool grad, bool spec) {
     return per_sm;
 }
 
-// Resident blocks per SM of the node kernel of the bin and slice mappings
-// (asked of the runtime once per block size).
+// Resident blocks per SM of the mixed-precision node kernels of the bin and
+// slice mappings (asked of the runtime once per block size).
 int node_ctas_per_sm(gna_plan* p, bool grad, int block) {
     if (p->grid_mult > 0) return p->grid_mult;
     int& n = p->res_ctas[grad];
     if (n == 0 || p->res_block[grad] != block) {
-        n = p->general ? general_resident_ctas(p->ph, p->nl_inst, p->nL, grad, block)
-            : p->ph < 2 ? nodes_resident_ctas(p->ph, p->nL, grad, block)
-                        : std::max(1, 1024 / block);
+        n = p->general ? general_resident_ctas(p->ph, p->nL, grad, block) : nodes_resident_ctas(p->ph, p->nL, grad, block);
         p->res_block[grad] = block;
     }
     return n;
@@ -343,7 +345,10 @@ struct SliceShape {
     int S, L, ntasks;
 };
 
-SliceShape slice_shape(gna_plan* p, int64_t resident_warps) {
+// in nodes of the mixed-precision kernels
+constexpr int64_t kTaskCost = 6, kReduceCost = 16;
+
+SliceShape slice_shape(gna_plan* p, int64_t resident_warps, int64_t task_cost, int64_t reduce_cost) {
     const int n = p->n_uniform;
     const int64_t pg = (int64_t)p->npts * p->ngroups;
     const int64_t cap = std::max(1, p->slices_cap);
@@ -351,14 +356,13 @@ SliceShape slice_shape(gna_plan* p, int64_t resident_warps) {
     if (L <= 0 && p->auto_warps == resident_warps) {
         L = p->auto_len;
     } else if (L <= 0) {
-        constexpr int64_t kTaskCost = 6, kReduceCost = 16;
         int64_t best = -1;
         L = n;
         for (int64_t S = 1; S <= cap; S++) {
             const int64_t len = (n + S - 1) / S, used = (n + len - 1) / len;
             if (used != S) continue;  // same length as a smaller S
             const int64_t rounds = (pg * S + resident_warps - 1) / resident_warps;
-            const int64_t cost = rounds * (len + kTaskCost) + (S > 1 ? kReduceCost : 0);
+            const int64_t cost = rounds * (len + task_cost) + (S > 1 ? reduce_cost : 0);
             if (best < 0 || cost < best) {
                 best = cost;
                 L = len;
@@ -482,12 +486,38 @@ gna_status enqueue_fit_nodes(gna_plan* plan, const EpiArgs& ea, cudaStream_t s, 
     return GNA_OK;
 }
 
+// Node pass (and slice reduction) of a GNA_FP64 evaluation of either chain by
+// bins.  The FP64 pipe's latency takes about four warps per SM quarter to
+// cover (1000 x 16384 x 8: 18.2 ms with one, 14.1 with two, 12.7 with three,
+// 12.1 with four), so the bins of a uniform grid are cut until there are about
+// that many tasks; a task's own cost (the anchor of its chunk) is that of
+// about three nodes.
+gna_status enqueue_nodes64(gna_plan* plan, const EpiArgs& ea, bool grad, bool spec, cudaStream_t s, int* nl) {
+    constexpr int kBlock = 128, kCtas = 4;
+    SliceShape ssh{1, 0, plan->ntasks};
+    if (plan->uniform) ssh = slice_shape(plan, 16LL * plan->sm_count, 3, 2);
+    if ((int64_t)plan->npts * plan->ngroups * ssh.S >= (1LL << 31)) return fail(plan, GNA_ESHAPE, "too many slice tasks");
+    const bool sliced = ssh.S > 1;
+    const int NVs = sums64(plan->general, grad) + (spec ? plan->nL : 0);
+    Args64 a{plan->grid64_bins, plan->d_goff, plan->d_gn, plan->d_gid, plan->d_tasks, ssh.ntasks, plan->ngroups, plan->nbins,
+             plan->d_pc, plan->d_gc, plan->bc, plan->d_counters, ea, ssh.S, ssh.L, sliced ? (double*)plan->d_slices : nullptr,
+             NVs, plan->nL, spec, plan->d_step};
+    const int grid = grid_size(plan, plan->grid_mult > 0 ? plan->grid_mult : kCtas, kBlock, ssh.ntasks);
+    CU(launch_nodes64(plan->general, grad, a, grid, kBlock, s));
+    if (sliced) {
+        CU(launch_slices_reduce64(plan->general, grad, (double*)plan->d_slices, ssh.S, NVs, ea, plan->d_pc, plan->d_gc,
+                                  plan->npts, s));
+        (*nl)++;
+    }
+    return GNA_OK;
+}
+
 // Enqueue one fused evaluation; counts kernel launches into *launches.
 gna_status enqueue_eval(gna_plan* plan, const EvalReq& q, cudaStream_t s, int* launches) {
     const bool grad = q.grad || q.grad_eta || q.H;
     const bool spec = q.spectra != nullptr;
-    const bool split = plan->mapping == MAP_SPLIT;
-    const bool fit = q.H && plan->ph < 2 && !split;  // the fits' own node kernel (fused.cuh)
+    const bool split = plan->mapping == MAP_SPLIT || (q.H && plan->fit_split);
+    const bool fit = q.H && !split;  // the fits' own node kernels (fused.cuh, fused64.cuh)
     const bool plain_sums = split || fit;
     int nl = 0;
     const int NV = value_count(plan, grad, spec, plain_sums);
@@ -500,15 +530,15 @@ gna_status enqueue_eval(gna_plan* plan, const EvalReq& q, cudaStream_t s, int* l
     }
     SliceShape ssh{1, 0, plan->ntasks};
     const int nblock = plan->ph < 2 ? nodes_block(plan->block) : plan->block;
-    const int ctas = split ? 0 : node_ctas_per_sm(plan, grad, nblock);
+    const int ctas = split || plan->ph == 2 ? 0 : node_ctas_per_sm(plan, grad, nblock);
     if (plan->mapping == MAP_SLICES && !fit) {
-        ssh = slice_shape(plan, (int64_t)plan->sm_count * ctas * (nblock / 32));
+        ssh = slice_shape(plan, (int64_t)plan->sm_count * ctas * (nblock / 32), kTaskCost, kReduceCost);
         if ((int64_t)plan->npts * plan->ngroups * ssh.S >= (1LL << 31)) return fail(plan, GNA_ESHAPE, "too many slice tasks");
     }
     // work counter, per-point and per-bin arrival counters: zeroed by the
     // kernel that prepares the per-point constants
     const int64_t ncnt = 1 + (int64_t)plan->npts * (1 + plan->ngroups) +
-                         (plan->mapping == MAP_SPLIT ? (int64_t)plan->npts * plan->nbins : 0);
+                         (split ? (int64_t)plan->npts * plan->nbins : 0);
     CU(launch_prepare(q.params, plan->npts, plan->bc, plan->d_pc, s, plan->d_counters, ncnt, plan->d_status));
     nl++;
     EpiArgs ea = make_epi(plan, q, grad, spec, NV, plain_sums);
@@ -520,7 +550,7 @@ gna_status enqueue_eval(gna_plan* plan, const EvalReq& q, cudaStream_t s, int* l
     if (plan->profile && cap == cudaStreamCaptureStatusNone)
         timed = (plan->prof_seen++ % plan->prof_every) == 0 && plan->prof_n < (int)plan->prof_ev.size() / 2;
     if (timed) CU(cudaEventRecord(plan->prof_ev[2 * plan->prof_n], s));
-    if (plan->mapping == MAP_SPLIT) {
+    if (split) {
         if (plan->ph < 2) {
             const int gstep = (int)(32 % ((int64_t)plan->nbins * plan->n_uniform));
             SplitArgs a{plan->grid_split, plan->nbins, plan->n_uniform, plan->npts, sh.per, sh.maxseg, gstep,
@@ -531,28 +561,26 @@ gna_status enqueue_eval(gna_plan* plan, const EvalReq& q, cudaStream_t s, int* l
                           plan->d_pc, plan->bc, (double*)plan->d_part, ea};
             CU(dispatch_split(2, plan->nl_inst, grad, spec, &a, sh.grid, plan->block, s));
         }
-    } else if (fit) {
+    } else if (fit && plan->ph < 2) {
         TRY(enqueue_fit_nodes(plan, ea, s, &nl));
+    } else if (fit) {
+        BinArgs64 a{plan->grid64_bins, plan->d_goff, plan->d_gn, plan->d_gid, plan->d_tasks, plan->ntasks,
+                    plan->ngroups, plan->nbins, plan->d_pc, plan->bc, plan->d_counters, ea};
+        const int per_sm = plan->grid_mult > 0 ? plan->grid_mult : std::max(1, 1024 / plan->block);
+        CU(dispatch_fit_ph2(plan->nl_inst, a, grid_size(plan, per_sm, plan->block, plan->ntasks), plan->block, s));
+    } else if (plan->ph == 2) {
+        TRY(enqueue_nodes64(plan, ea, grad, spec, s, &nl));
     } else {
         const int g = grid_size(plan, ctas, nblock, ssh.ntasks);
-        if (plan->ph < 2) {
-            const bool sliced = ssh.S > 1;
-            const int NVs = 3 + (grad ? 3 : 0) + (spec ? plan->nL : 0);
-            BinArgs a{nullptr, plan->grid_rec, plan->d_goff, plan->d_gn, plan->d_gid, nullptr, plan->d_desc, ssh.ntasks,
-                      plan->ngroups, plan->nbins, plan->d_pc, plan->bc, plan->d_counters, ea,
-                      ssh.S, ssh.L / 4, sliced ? plan->d_slices : nullptr, NVs, plan->nL, spec, plan->d_step};
-            CU(dispatch_nodes(plan->ph, grad, a, g, nblock, s));
-            if (sliced) {
-                CU(launch_slices_reduce(plan->d_slices, ssh.S, NVs, ea, plan->d_pc, plan->npts, s));
-            } else {
-                CU(launch_point_sums(4, ea, s));
-            }
-            nl++;
-        } else {
-            BinArgs64 a{plan->grid64_bins, plan->d_goff, plan->d_gn, plan->d_gid, plan->d_tasks, plan->ntasks,
-                        plan->ngroups, plan->nbins, plan->d_pc, plan->bc, plan->d_counters, ea};
-            CU(dispatch_bins_ph2(plan->nl_inst, grad, spec, &a, g, nblock, s));
-        }
+        const bool sliced = ssh.S > 1;
+        const int NVs = 3 + (grad ? 3 : 0) + (spec ? plan->nL : 0);
+        BinArgs a{nullptr, plan->grid_rec, plan->d_goff, plan->d_gn, plan->d_gid, nullptr, plan->d_desc, ssh.ntasks,
+                  plan->ngroups, plan->nbins, plan->d_pc, plan->bc, plan->d_counters, ea,
+                  ssh.S, ssh.L / 4, sliced ? plan->d_slices : nullptr, NVs, plan->nL, spec, plan->d_step};
+        CU(dispatch_nodes(plan->ph, grad, a, g, nblock, s));
+        if (sliced) CU(launch_slices_reduce(plan->d_slices, ssh.S, NVs, ea, plan->d_pc, plan->npts, s));
+        else CU(launch_point_sums(4, ea, s));
+        nl++;
     }
     nl++;
     if (timed) {
@@ -573,14 +601,16 @@ gna_status enqueue_eval(gna_plan* plan, const EvalReq& q, cudaStream_t s, int* l
 // q.H set for the fits' J^T W J); counts kernel launches into *launches.
 gna_status enqueue_eval_general(gna_plan* plan, const EvalReq& q, cudaStream_t s, int* launches) {
     const bool grad = q.grad || q.grad_eta || q.H;
-    const bool fit = q.H && plan->ph < 2;           // the fits' own node kernel (general.cuh)
+    const bool fit = q.H != nullptr;                  // the fits' own node kernels (general.cuh)
     const bool surv = plan->g_alpha == plan->g_beta;  // survival channel: the fits reduce phases modulo pi/2
     const int NV = fit ? gen_nv(true) : gen_sums(grad);
     const int nblock = (plan->ph < 2 && !fit) ? nodes_block(plan->block) : plan->block;
-    const int ctas = fit ? general_fit_ctas(plan->ph, plan->nl_inst, surv, nblock) : node_ctas_per_sm(plan, grad, nblock);
+    const int ctas = plan->ph == 2 ? general_fit_ctas64(plan->nl_inst, nblock)
+                     : fit         ? general_fit_ctas(plan->ph, plan->nl_inst, surv, nblock)
+                                   : node_ctas_per_sm(plan, grad, nblock);
     SliceShape ssh{1, 0, plan->ntasks};
     if (plan->mapping == MAP_SLICES) {
-        ssh = fit ? fixed_slice_shape(plan) : slice_shape(plan, (int64_t)plan->sm_count * ctas * (nblock / 32));
+        ssh = fit ? fixed_slice_shape(plan) : slice_shape(plan, (int64_t)plan->sm_count * ctas * (nblock / 32), kTaskCost, kReduceCost);
         if ((int64_t)plan->npts * plan->ngroups * ssh.S >= (1LL << 31)) return fail(plan, GNA_ESHAPE, "too many slice tasks");
     }
     const int64_t ncnt = 1 + (int64_t)plan->npts * (1 + plan->ngroups);
@@ -592,11 +622,17 @@ gna_status enqueue_eval_general(gna_plan* plan, const EvalReq& q, cudaStream_t s
     const bool sliced = ssh.S > 1;
     const int g = grid_size(plan, ctas, nblock, ssh.ntasks);
     *launches = 2;
+    if (plan->ph == 2 && !fit) {
+        int nl = 2;
+        TRY(enqueue_nodes64(plan, ea, grad, false, s, &nl));
+        *launches = nl;
+        return GNA_OK;
+    }
     if (plan->ph == 2) {
         GenArgs64 ga64{BinArgs64{plan->grid64_bins, plan->d_goff, plan->d_gn, plan->d_gid, plan->d_tasks, plan->ntasks,
                                  plan->ngroups, plan->nbins, plan->d_pc, plan->bc, plan->d_counters, ea},
                        plan->d_gc};
-        CU(dispatch_general64(plan->nl_inst, grad, ga64, g, nblock, s));
+        CU(dispatch_general_fit64(plan->nl_inst, ga64, g, nblock, s));
         return GNA_OK;
     }
     GenArgs ga{BinArgs{plan->grid_bins, plan->grid_rec, plan->d_goff, plan->d_gn, plan->d_gid, plan->d_tasks, plan->d_desc,
@@ -1026,6 +1062,11 @@ static gna_status plan_build(gna_plan* plan, const gna_plan_desc* d, cudaStream_
     else if (plan->uniform && (plan->n_uniform >= 1024 || (int64_t)d->npts * ngroups < 16LL * plan->sm_count))
         plan->mapping = MAP_SPLIT;
     else plan->mapping = MAP_BINS;
+    const bool was_split = plan->mapping == MAP_SPLIT;
+    if (plan->ph == 2 && was_split && !(d->flags & GNA_PLAN_FORCE_SPLIT)) {
+        plan->mapping = MAP_BINS;
+        plan->fit_split = true;
+    }
     const bool forced = plan->general ||
                         (d->flags & (GNA_PLAN_FORCE_SPLIT | GNA_PLAN_FORCE_BINS | GNA_PLAN_FORCE_SLICES)) != 0;
     const bool small = plan->uniform && (int64_t)d->nbins * plan->n_uniform <= (1LL << 20) &&
@@ -1034,7 +1075,7 @@ static gna_status plan_build(gna_plan* plan, const gna_plan_desc* d, cudaStream_
     // nodes), so that the autotuner can compare the two
     const bool keep_split = plan->mapping == MAP_SLICES && !forced &&
                             (int64_t)d->nbins * plan->n_uniform <= (1LL << 26);
-    plan->has_split = plan->mapping == MAP_SPLIT || (!forced && small) || keep_split;
+    plan->has_split = was_split || (!forced && small) || keep_split;
     plan->has_bins = plan->mapping == MAP_BINS || plan->mapping == MAP_SLICES || (!forced && small);
     // one grid per distinct node count: the bins and weights depend on nothing
     // else, so points with the same count share one grid (read once from HBM
@@ -1144,7 +1185,7 @@ static gna_status plan_build(gna_plan* plan, const gna_plan_desc* d, cudaStream_
     }
     std::vector<float> step;  // (copied from below: lives until the stream is synchronised)
     std::vector<BinTask> desc;
-    if (plan->has_bins && plan->ph < 2) {
+    if (plan->has_bins) {
         // neighbouring zeros of P_n are less than pi / (n + 1/2) apart in
         // theta, x = cos theta, so the nodes of a bin of half width h are less
         // than h pi / (n + 1/2) apart in E and 1/E_low^2 times that in 1/E
@@ -1189,7 +1230,7 @@ static gna_status plan_build(gna_plan* plan, const gna_plan_desc* d, cudaStream_
     // scratch
     TRY(dalloc(plan, &plan->d_pc, d->npts));
     if (plan->general) TRY(dalloc(plan, &plan->d_gc, d->npts));
-    const int nv_max = std::max(fused_nv(plan->nl_inst, true, true), plan->general ? gen_nv(true) : 0) + 1;
+    const int nv_max = std::max(fused_nv(plan->nl_inst, true, true) + 2, plan->general ? gen_nv(true) : 0);
     if (plan->has_split) {
         // ranges are at least 128 nodes long, so a bin meets at most ceil(n / 128) + 1 of
         // them; the slot count is capped so that the partials stay within 256 M values
@@ -1200,11 +1241,12 @@ static gna_status plan_build(gna_plan* plan, const gna_plan_desc* d, cudaStream_
         plan->part_cap = (size_t)pairs * plan->maxseg_cap * nv_max;
         TRY(dalloc(plan, (double**)&plan->d_part, plan->part_cap));
     }
-    if (slices_ok && plan->has_bins) {
-        // slices per group: up to 8 tasks per resident warp, at least 16 nodes per slice
+    if (plan->uniform && plan->has_bins) {
+        // slices per group: up to 8 tasks per resident warp, at least 16 nodes per
+        // slice (GNA_FP64: eight tasks per SM quarter, four nodes)
         const int64_t pg = (int64_t)d->npts * ngroups;
-        const int64_t by_tasks = (8 * warps_est + pg - 1) / pg;
-        const int64_t by_len = std::max<int64_t>(1, plan->n_uniform / 16);
+        const int64_t by_tasks = ((plan->ph == 2 ? 32LL * plan->sm_count : 8 * warps_est) + pg - 1) / pg;
+        const int64_t by_len = std::max<int64_t>(1, plan->n_uniform / (plan->ph == 2 ? 4 : 16));
         plan->slices_cap = (int)std::max<int64_t>(1, std::min(by_tasks, by_len));
         if (plan->slices_cap > 1)
             TRY(dalloc(plan, &plan->d_slices, (size_t)pg * plan->slices_cap * nv_max * 32));
@@ -1754,6 +1796,7 @@ gna_status gna_plan_set_tuning(gna_plan* plan, const char* text) {
     plan->npt = npt;
     plan->grid_mult = gm;
     plan->mapping = mapping;
+    if (m) plan->fit_split = false;
     plan->slice_len = sl;
     destroy_graph(plan);
     return GNA_OK;

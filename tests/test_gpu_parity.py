@@ -1122,3 +1122,58 @@ def test_general_anchored_chunks(api, prec, nL, channel, n, edges):
         for o in (out, alone):
             check_chi2(o["chi2"][0].item(), ref, data, wl.POISSON, 1e-6, tag="general anchored %d %d" % (nL, n), plain=False)
         plan.close()
+
+
+@pytest.mark.parametrize("nL", [1, 3, 9])
+@pytest.mark.parametrize("n,edges", [(1, (2.0, 9.0)), (3, (2.0, 9.0)), (5, (3.0, 3.4)), (33, (3.0, 3.4)), (130, (3.0, 3.4)),
+                                     (1000, (3.0, 3.4)), (67, (0.6, 12.0))])
+def test_fp64_anchored_chunks(api, nL, n, edges):
+    # GNA_FP64: sincos per node (coarse grids), both lengths of polynomial
+    # (0.6-12 MeV has all three), whole bins and slices
+    rng = np.random.default_rng(nL + n)
+    e = np.linspace(edges[0], edges[1], 38)
+    L = rng.uniform(1.0, 60.0, nL)
+    theta = np.array(wl.TRUTH) * 1.03
+    Nn = oracle.norm_for_total(e, n, L, wl.TRUTH)
+    data = wl.poisson_data(Nn * (oracle.baseline_weights(L) @ oracle.binned(e, n, L, wl.TRUTH)), 7)
+    ref = oracle.chain(e, n, L, theta, Nn, data, wl.POISSON)
+    for npts in (1, 40):
+        plan = api.Plan(e, L, nodes_per_bin=n, npts=npts, norm=Nn, prec="fp64", kind="poisson")
+        p, d = plan.params_tensor(np.repeat(theta[None], npts, 0)), dev(data)
+        out = plan.eval(p, d, grad=True, mu=True, spectra=True)
+        alone = plan.eval(p, d, grad=False)
+        torch.cuda.synchronize()
+        plan.status()
+        q = npts - 1
+        assert rel(out["mu"][q].cpu().numpy(), ref["mu"]) < 1e-9
+        assert rel(out["spectra"][q].cpu().numpy(), ref["mu_rb"]) < 1e-9
+        assert normrel(out["grad"][q].cpu().numpy(), ref["grad"][:4]) < 1e-9
+        for o in (out, alone):
+            check_chi2(o["chi2"][q].item(), ref, data, wl.POISSON, 1e-9, tag="fp64 anchored %d %d" % (nL, n), plain=False)
+        plan.close()
+
+
+@pytest.mark.parametrize("nL", [1, 3])
+@pytest.mark.parametrize("channel", [("mu", "e", False), ("mu", "mu", True)])
+@pytest.mark.parametrize("n,edges", [(1, (600.0, 4000.0)), (5, (1500.0, 2000.0)), (131, (1500.0, 2000.0)), (21, (150.0, 3000.0))])
+def test_fp64_general_anchored_chunks(api, nL, channel, n, edges):
+    e = np.linspace(edges[0], edges[1], 38)
+    L = np.array([810.0, 295.0, 735.0])[:nL]
+    th = np.array(THETA_FULL) * 1.02
+    a, b, anti = channel
+    mu_rb, _ = oracle.binned_general(e, n, L, THETA_FULL, a, b, anti, 1e-3)
+    M = oracle.baseline_weights(L) @ mu_rb
+    Nn = 1e4 / M.sum()
+    data = wl.poisson_data(Nn * M, 3)
+    ref = oracle.chain_general(e, n, L, th, Nn, data, a, b, anti, 1, None, 0.0, 1e-3)
+    plan = api.Plan(e, L, nodes_per_bin=n, norm=Nn, e_scale=1e-3, prec="fp64", kind="poisson", channel=channel)
+    p, d = plan.params_tensor(th), dev(data)
+    out = plan.eval_general(p, d, grad=True, mu=True)
+    alone = plan.eval_general(p, d, grad=False)
+    torch.cuda.synchronize()
+    plan.status()
+    assert rel(out["mu"][0].cpu().numpy(), ref["mu"]) < 1e-9
+    assert normrel(out["grad"][0].cpu().numpy(), ref["grad"][:6]) < 1e-9
+    for o in (out, alone):
+        check_chi2(o["chi2"][0].item(), ref, data, wl.POISSON, 1e-9, tag="fp64 general %d %d" % (nL, n), plain=False)
+    plan.close()
