@@ -26,6 +26,7 @@
 #include "gnaosc.h"
 #include "misc.h"
 #include "nodes64.cuh"
+#include "oscprob.h"
 
 using namespace gna;
 
@@ -760,6 +761,8 @@ static gna_status ee_constants(const double* L, int nL, const gna_osc* p, OscCon
         split_ff(oc.c32[r], oc.c32h[r], oc.c32l[r]);
         split_ff(oc.c21[r] + oc.c32[r], oc.c31h[r], oc.c31l[r]);
     }
+    const double cr[3] = {-oc.A[0], -oc.A[1], -oc.A[2]}, ci[3] = {0.0, 0.0, 0.0};
+    turn_constants(oc.c21, oc.c32, nL, 1.0, cr, ci, oc.t);
     return GNA_OK;
 }
 
@@ -950,6 +953,7 @@ gna_status gna_oscprob(const double* E, int64_t n, const double* L, int nL, int 
             split_ff(cq[q], oc.ch[q][r], oc.cl[q][r]);
         }
     }
+    turn_constants(oc.c[0], oc.c[2], nL, oc.dab, oc.cr, oc.ci, oc.t);
     cudaError_t e = launch_oscgen(E, n, oc, prec, P_out, (cudaStream_t)stream);
     return e == cudaSuccess ? GNA_OK : GNA_ECUDA;
 }

@@ -377,80 +377,6 @@ cudaError_t launch_plain_chunk(const PlainArgs& a, const PlainChi2Args& ca, cuda
     return cudaGetLastError();
 }
 
-// -------------------------------------------------- element-wise OscProb --
-// FP64: P[r][k] = 1 - sum_ij A_ij sin^2(c_ij,r / E_k), CUDA double sin.
-__global__ void k_oscprob64(const double* __restrict__ E, int64_t n, OscConst oc, double* __restrict__ P) {
-    const int64_t k = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (k >= n) return;
-    const double e = 1.0 / E[k];
-    for (int r = 0; r < oc.nL; r++) {
-        const double s21 = sin(oc.c21[r] * e), s32 = sin(oc.c32[r] * e), s31 = sin((oc.c21[r] + oc.c32[r]) * e);
-        P[(int64_t)r * n + k] = 1.0 - oc.A[0] * s21 * s21 - oc.A[1] * s31 * s31 - oc.A[2] * s32 * s32;
-    }
-}
-
-// Mixed: each phase reduced modulo pi/2 (quadrant parity q), sin r by the
-// FP32 polynomial; sin^2(phase) = s^2 for even q, 1 - s^2 for odd q.  The
-// dominant term is written as (1 - A21) + A21 s^2 for odd q so that P stays
-// accurate to a few ulp where it is smallest.
-template <int PH>
-__device__ __forceinline__ float reduce_half_pi(float ch, float cl, double cd, float eh, float el, double ed, int& odd) {
-    if (PH == 0) {
-        float p = __fmul_rn(ch, eh);
-        float e = __fmaf_rn(ch, eh, -p);
-        float lo = __fmaf_rn(ch, el, __fmaf_rn(cl, eh, e));
-        float qm = __fmaf_rn(p, 2.0f * GNA_INV_PI_F, GNA_ROUND_MAGIC);
-        odd = __float_as_int(qm) & 1;
-        float q = __fsub_rn(qm, GNA_ROUND_MAGIC);
-        float r = __fmaf_rn(-q, 0.5f * GNA_PI_A, p);
-        r = __fmaf_rn(-q, 0.5f * GNA_PI_B, r);
-        r = __fmaf_rn(-q, 0.5f * GNA_PI_C, r);
-        return __fadd_rn(r, lo);
-    } else {
-        double p = cd * ed;
-        double q = rint(p * (2.0 * GNA_INV_PI_D));
-        odd = ((long long)q) & 1;
-        double r = fma(-q, 0.5 * GNA_PI_DA, p);
-        r = fma(-q, 0.5 * GNA_PI_DB, r);
-        r = fma(-q, 0.5 * GNA_PI_DC, r);
-        return (float)r;
-    }
-}
-
-template <int PH>
-__global__ void k_oscprob_mixed(const double* __restrict__ E, int64_t n, OscConst oc, float* __restrict__ P) {
-    const int64_t k = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (k >= n) return;
-    float eh, el;
-    ff_recip(E[k], eh, el);
-    const double ed = (double)eh + (double)el;
-    const float A21 = oc.Af[0], A31 = oc.Af[1], A32 = oc.Af[2];
-    const float omA21 = oc.one_minus_A21f;
-    for (int r = 0; r < oc.nL; r++) {
-        int o21, o31, o32;
-        const float r21 = reduce_half_pi<PH>(oc.c21h[r], oc.c21l[r], oc.c21[r], eh, el, ed, o21);
-        const float r31 = reduce_half_pi<PH>(oc.c31h[r], oc.c31l[r], oc.c21[r] + oc.c32[r], eh, el, ed, o31);
-        const float r32 = reduce_half_pi<PH>(oc.c32h[r], oc.c32l[r], oc.c32[r], eh, el, ed, o32);
-        const float s21 = sin_poly(r21), s31 = sin_poly(r31), s32 = sin_poly(r32);
-        const float q21 = s21 * s21, q31 = s31 * s31, q32 = s32 * s32;
-        const float S31 = o31 ? 1.0f - q31 : q31;
-        const float S32 = o32 ? 1.0f - q32 : q32;
-        const float base = o21 ? fmaf(A21, q21, omA21) : fmaf(-A21, q21, 1.0f);
-        P[(int64_t)r * n + k] = fmaf(-A32, S32, fmaf(-A31, S31, base));
-    }
-}
-
-cudaError_t launch_oscprob(const double* E, int64_t n, const OscConst& oc, int prec, void* P, cudaStream_t s) {
-    const unsigned blocks = (unsigned)((n + 255) / 256);
-    if (prec == GNA_FP64)
-        k_oscprob64<<<blocks, 256, 0, s>>>(E, n, oc, (double*)P);
-    else if (prec == GNA_MIXED_F64PHASE)
-        k_oscprob_mixed<1><<<blocks, 256, 0, s>>>(E, n, oc, (float*)P);
-    else
-        k_oscprob_mixed<0><<<blocks, 256, 0, s>>>(E, n, oc, (float*)P);
-    return cudaGetLastError();
-}
-
 // ------------------------------------------------------------- step a11 --
 // Batched Levenberg-Marquardt, one thread per data set, NP = 4 (survival
 // chain: s2_12, s2_13, dm2_21, dm2_32) or 6 (any channel: s2_12, s2_13,

@@ -46,27 +46,6 @@ struct PlainChi2Args {
     double* spectra_out;  // [npts][nL][nbins] or NULL
 };
 
-struct OscConst {
-    double c21[GNA_NLMAX], c32[GNA_NLMAX];
-    float c21h[GNA_NLMAX], c21l[GNA_NLMAX], c32h[GNA_NLMAX], c32l[GNA_NLMAX], c31h[GNA_NLMAX], c31l[GNA_NLMAX];
-    double A[3];
-    float Af[3];
-    float one_minus_A21f;
-    int nL;
-};
-
-// Constants of the general-channel kernel: phases q = (21, 31, 32) per
-// baseline (double and hi + lo floats), coefficients -4 Re X and 2 Im X.
-struct OscGenConst {
-    double c[3][GNA_NLMAX];
-    float ch[3][GNA_NLMAX], cl[3][GNA_NLMAX];
-    double cr[3], ci[3];
-    float crf[3], cif[3];
-    double dab;  // delta_ab
-    int nL;
-};
-cudaError_t launch_oscgen(const double* E, int64_t n, const OscGenConst& oc, int prec, void* P, cudaStream_t s);
-
 // Levenberg-Marquardt state of one data set for NP parameters.
 template <int NP>
 struct LMStateT {
@@ -91,7 +70,6 @@ cudaError_t launch_sum_weights(const float4* grid, int nbins, int n, int layout,
 // The plain chain's kernels for one chunk of points: OscProb (+ tangents),
 // weights, bin integration, chi^2 (4 launches, 6 with the tangents).
 cudaError_t launch_plain_chunk(const PlainArgs& a, const PlainChi2Args& ca, cudaStream_t s);
-cudaError_t launch_oscprob(const double* E, int64_t n, const OscConst& oc, int prec, void* P, cudaStream_t s);
 template <int NP>
 cudaError_t launch_lm_init(LMStateT<NP>* st, int npts, double lam0, cudaStream_t s);
 template <int NP>

@@ -1177,3 +1177,36 @@ def test_fp64_general_anchored_chunks(api, nL, channel, n, edges):
     for o in (out, alone):
         check_chi2(o["chi2"][0].item(), ref, data, wl.POISSON, 1e-9, tag="fp64 general %d %d" % (nL, n), plain=False)
     plan.close()
+
+
+@pytest.mark.parametrize("prec", ["fp64", "f64phase", "ff"])
+def test_oscprob_number_ranges(api, prec):
+    """Energies at the edges of the number range, and phases from next to zero
+    to many turns: each against the formula in double."""
+    E = np.array([5.0, 1.0, 2.0, np.nextafter(2.0, 0.0), np.nextafter(1.0, 2.0), 2.0 ** -20, 2.0 ** 20, 3e9, 1e15, 1e30,
+                  1e300, 2.0 ** -1000, -5.0, np.inf, np.nan])
+    L = [0.0, 52.5, 1.7, 1e4]
+    for channel in (None, ("mu", "e"), ("mu", "mu")):
+        th = THETA_FULL
+        if channel is None:
+            P = api.oscprob(dev(E), L, [th[i] for i in (0, 1, 4, 5)], prec).double().cpu().numpy()
+        else:
+            P = api.oscprob_general(dev(E), L, th, *channel, prec=prec).double().cpu().numpy()
+        with np.errstate(all="ignore"):
+            ref = np.array([oracle_prob(*(channel or ("e", "e")), E, Lr, False) for Lr in L])
+            phase = np.array([1266.932679419849 * Lr * (th[4] + th[5]) / np.abs(E) for Lr in L])
+        # double: the phase's rounding, twice its 2^-53; mixed: FP32 polynomials
+        # (2e-7 each) and, in double-float, 2^-44 of the phase up to its 2^12 pi
+        top = {"fp64": 1e9, "f64phase": 1e6, "ff": 1e4}[prec]
+        ok = np.isfinite(ref) & (phase < top)
+        if prec != "fp64":  # 1/E is a pair of floats
+            ok &= (np.abs(E) < 1e18) & (np.abs(E) > 1e-18)
+        tol = {"fp64": 4e-16 + 1e-15 * phase, "f64phase": 6e-7 + 1e-12 * phase, "ff": 6e-7 + 1e-11 * phase}[prec]
+        assert ok[:, :5].any(axis=0).all()
+        assert (np.abs(P - ref)[ok] <= tol[ok]).all()
+        if prec == "fp64":
+            # probabilities next to zero or one: the terms (up to 2x each) are
+            # good to 2^-53 of themselves
+            small = ok & (phase < 1e-2)
+            assert (np.abs(P - ref)[small] <= 1e-15 * phase[small] + (3e-16 if channel != ("mu", "e") else 0)).all()
+            assert np.isnan(P[1:, -1]).all()
