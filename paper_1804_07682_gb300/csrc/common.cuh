@@ -47,6 +47,7 @@ struct BaseConst {
     double klmax;           // largest K L_r
     float wsum;             // sum_r om_r rounded to FP32
     double wsum_lo;         // sum_r om_r - wsum (exact sum of the FP32 weights)
+    double wsum_pair;       // sum_r (om_r + omlo_r)
     int nL;
 };
 

@@ -11,42 +11,17 @@
 namespace gna {
 
 // ------------------------------------------------------------ step a0 ----
-// A real number with its derivatives in (s2_12, s2_13, s2_23, delta):
+// A real number with its derivative in one of (s2_12, s2_13, s2_23, delta):
 // forward-mode differentiation of the written-out mixing matrix.
 struct Dn {
-    double v, d[4];
+    double v, d;
 };
 
-__device__ inline Dn dn_const(double v) {
-    Dn x;
-    x.v = v;
-    for (int q = 0; q < 4; q++) x.d[q] = 0.0;
-    return x;
-}
-__device__ inline Dn dn_var(double v, int q, double dq) {
-    Dn x = dn_const(v);
-    x.d[q] = dq;
-    return x;
-}
-__device__ inline Dn operator+(const Dn& a, const Dn& b) {
-    Dn x;
-    x.v = a.v + b.v;
-    for (int q = 0; q < 4; q++) x.d[q] = a.d[q] + b.d[q];
-    return x;
-}
-__device__ inline Dn operator-(const Dn& a, const Dn& b) {
-    Dn x;
-    x.v = a.v - b.v;
-    for (int q = 0; q < 4; q++) x.d[q] = a.d[q] - b.d[q];
-    return x;
-}
+__device__ inline Dn dn_const(double v) { return Dn{v, 0.0}; }
+__device__ inline Dn operator+(const Dn& a, const Dn& b) { return Dn{a.v + b.v, a.d + b.d}; }
+__device__ inline Dn operator-(const Dn& a, const Dn& b) { return Dn{a.v - b.v, a.d - b.d}; }
 __device__ inline Dn operator-(const Dn& a) { return dn_const(0.0) - a; }
-__device__ inline Dn operator*(const Dn& a, const Dn& b) {
-    Dn x;
-    x.v = a.v * b.v;
-    for (int q = 0; q < 4; q++) x.d[q] = a.d[q] * b.v + a.v * b.d[q];
-    return x;
-}
+__device__ inline Dn operator*(const Dn& a, const Dn& b) { return Dn{a.v * b.v, a.d * b.v + a.v * b.d}; }
 
 // Complex number of such reals.
 struct Cn {
@@ -60,60 +35,50 @@ __device__ inline Cn operator*(const Cn& a, const Cn& b) {
 __device__ inline Cn operator*(const Dn& a, const Cn& b) { return Cn{a * b.re, a * b.im}; }
 __device__ inline Cn conjn(const Cn& a) { return Cn{a.re, -a.im}; }
 
-// Coefficients of P(alpha -> beta) at one point: the mixing matrix in the
-// standard parameterisation written out element by element (U = R23
-// U13(delta) R12), X_ij = U*_ai U_bi U_aj U*_bj for the pairs (21, 31, 32),
-// a = -4 Re X, b = 4 Im X, and for antineutrinos (V = U*, so X -> X*) b -> -b.
-__device__ void general_coefficients(const gna_osc_full& o, int alpha, int beta, int anti, GenConst& gc) {
-    const double s12v = sqrt(o.s2_12), c12v = sqrt(1.0 - o.s2_12);
-    const double s13v = sqrt(o.s2_13), c13v = sqrt(1.0 - o.s2_13);
-    const double s23v = sqrt(o.s2_23), c23v = sqrt(1.0 - o.s2_23);
-    // d sin(theta) / d sin^2(theta) = 1 / (2 sin), d cos / d sin^2 = -1 / (2 cos)
-    const Dn s12 = dn_var(s12v, 0, 0.5 / s12v), c12 = dn_var(c12v, 0, -0.5 / c12v);
-    const Dn s13 = dn_var(s13v, 1, 0.5 / s13v), c13 = dn_var(c13v, 1, -0.5 / c13v);
-    const Dn s23 = dn_var(s23v, 2, 0.5 / s23v), c23 = dn_var(c23v, 2, -0.5 / c23v);
-    double sd, cd;
-    sincos(o.delta_cp, &sd, &cd);
-    const Dn cosd = dn_var(cd, 3, -sd), sind = dn_var(sd, 3, cd);
-    const Cn ep = cn(cosd, sind);   // e^{+i delta}
-    const Cn em = cn(cosd, -sind);  // e^{-i delta}
+// Sines and cosines of the mixing angles and e^{+-i delta}.
+struct Angles {
+    Dn s12, c12, s13, c13, s23, c23;
+    Cn ep, em;
+};
+
+// Row `flavour` of the mixing matrix in the standard parameterisation (U = R23
+// U13(delta) R12), written out element by element.
+__device__ __forceinline__ void pmns_row(const Angles& t, int flavour, Cn (&U)[3]) {
     const Dn zero = dn_const(0.0);
-    const Cn s13ep = s13 * ep;
-    Cn U[3][3];
-    U[0][0] = cn(c12 * c13, zero);
-    U[0][1] = cn(s12 * c13, zero);
-    U[0][2] = s13 * em;
-    U[1][0] = cn(-(s12 * c23), zero) + (-(c12 * s23)) * s13ep;
-    U[1][1] = cn(c12 * c23, zero) + (-(s12 * s23)) * s13ep;
-    U[1][2] = cn(s23 * c13, zero);
-    U[2][0] = cn(s12 * s23, zero) + (-(c12 * c23)) * s13ep;
-    U[2][1] = cn(-(c12 * s23), zero) + (-(s12 * c23)) * s13ep;
-    U[2][2] = cn(c23 * c13, zero);
-    const int pi_[3] = {1, 2, 2}, pj_[3] = {0, 0, 1};
-    gc.dab = (alpha == beta) ? 1.0 : 0.0;
-    for (int k = 0; k < 3; k++) {
-        const int i = pi_[k], j = pj_[k];
-        const Cn X = conjn(U[alpha][i]) * U[beta][i] * U[alpha][j] * conjn(U[beta][j]);
-        const double sb = anti ? -4.0 : 4.0;
-        gc.a[k] = -4.0 * X.re.v;
-        gc.b[k] = sb * X.im.v;
-        gc.af[k] = (float)gc.a[k];
-        gc.bf[k] = (float)gc.b[k];
-        gc.alo[k] = (float)(gc.a[k] - (double)gc.af[k]);
-        gc.blo[k] = (float)(gc.b[k] - (double)gc.bf[k]);
-        for (int q = 0; q < 4; q++) {
-            gc.da[q][k] = -4.0 * X.re.d[q];
-            gc.db[q][k] = sb * X.im.d[q];
-            gc.daf[q][k] = (float)gc.da[q][k];
-            gc.dbf[q][k] = (float)gc.db[q][k];
-        }
+    if (flavour == 0) {
+        U[0] = cn(t.c12 * t.c13, zero);
+        U[1] = cn(t.s12 * t.c13, zero);
+        U[2] = t.s13 * t.em;
+        return;
+    }
+    const Cn s13ep = t.s13 * t.ep;
+    if (flavour == 1) {
+        U[0] = cn(-(t.s12 * t.c23), zero) + (-(t.c12 * t.s23)) * s13ep;
+        U[1] = cn(t.c12 * t.c23, zero) + (-(t.s12 * t.s23)) * s13ep;
+        U[2] = cn(t.s23 * t.c13, zero);
+    } else {
+        U[0] = cn(t.s12 * t.s23, zero) + (-(t.c12 * t.c23)) * s13ep;
+        U[1] = cn(-(t.c12 * t.s23), zero) + (-(t.s12 * t.c23)) * s13ep;
+        U[2] = cn(t.c23 * t.c13, zero);
     }
 }
 
-// One thread per (point, baseline slot): the phase constants as for the
-// survival chain; the point's first thread also forms its coefficients and
-// checks that the mixing parameters lie inside (0, 1) (the derivatives are
-// singular on the boundary).  Zeroes the evaluation's counters.
+__device__ __forceinline__ Cn pick(bool first, const Cn& a, const Cn& b) { return first ? a : b; }
+
+// Sixteen threads per point, one per baseline slot for the phase constants (as
+// for the survival chain).  The coefficients of P(alpha -> beta) --
+// X_ij = U*_ai U_bi U_aj U*_bj for the pairs (21, 31, 32), a = -4 Re X,
+// b = 4 Im X, and for antineutrinos (V = U*, so X -> X*) b -> -b -- are formed
+// by twelve of them, thread 4 k + q the pair k and its derivative in parameter
+// q, the roots and their reciprocals by six, one each.  A warp's FP64
+// instruction takes its SM quarter's pipe for 64 cycles however many threads
+// take part, so the number of instructions in the longest thread is the
+// kernel's time: one thread with all four derivatives and nine matrix elements
+// issued about 900.  GB300, whole evaluations: nu_mu disappearance at one point
+// (400 bins x 513 nodes x 2) 42.6 -> 27 us, 1021 points of nu_mu -> nu_e 165 ->
+// 132 us.  The first thread checks that the mixing parameters lie inside (0, 1)
+// (the derivatives are singular on the boundary).  Zeroes the evaluation's
+// counters.
 __global__ void k_prepare_general(const gna_osc_full* __restrict__ prm, int npts, BaseConst bc, int alpha, int beta,
                                   int anti, PointConst* __restrict__ out, GenConst* __restrict__ gout,
                                   int* __restrict__ zero, int64_t nz, int* __restrict__ status) {
@@ -122,25 +87,75 @@ __global__ void k_prepare_general(const gna_osc_full* __restrict__ prm, int npts
     asm volatile("griddepcontrol.wait;" ::: "memory");
     const int64_t tid = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     for (int64_t k = tid; k < nz; k += (int64_t)gridDim.x * blockDim.x) zero[k] = 0;
-    const int p = (int)(tid / GNA_NLMAX), r = (int)(tid % GNA_NLMAX);
-    if (p >= npts) return;
+    static_assert(GNA_NLMAX == 16, "two points per warp");
+    if (tid / 32 * 2 >= npts) return;  // the warp's first point: whole warps go on
+    const int r = (int)(tid % GNA_NLMAX);
+    const bool live = tid / GNA_NLMAX < npts;
+    const int p = live ? (int)(tid / GNA_NLMAX) : npts - 1;
     const gna_osc_full o = prm[p];
-    PointConst& pc = out[p];
     const double kl = (r < bc.nL) ? bc.kld[r] : 0.0;
     const double c21 = o.dm2_21 * kl, c32 = o.dm2_32 * kl;
-    pc.c21[r] = c21;
-    pc.c32[r] = c32;
-    split_ff(c21, pc.c21h[r], pc.c21l[r]);
-    split_ff(c32, pc.c32h[r], pc.c32l[r]);
+    if (live) {
+        PointConst& pc = out[p];
+        pc.c21[r] = c21;
+        pc.c32[r] = c32;
+        split_ff(c21, pc.c21h[r], pc.c21l[r]);
+        split_ff(c32, pc.c32h[r], pc.c32l[r]);
+    }
+    // roots of s2_12, 1 - s2_12, ... in threads 0 to 5, with 1 / (2 root):
+    // d sin(theta) / d sin^2(theta) = 1 / (2 sin), d cos / d sin^2 = -1 / (2 cos)
+    const double x2 = r < 2 ? o.s2_12 : r < 4 ? o.s2_13 : o.s2_23;
+    const double root = sqrt((r & 1) ? 1.0 - x2 : x2), half = 0.5 / root;
+    const int k = min(r >> 2, 2), q = r & 3;
+    auto angle = [&](int j, int par, double sign) {
+        const double v = __shfl_sync(0xffffffffu, root, j, 16), h = __shfl_sync(0xffffffffu, half, j, 16);
+        return Dn{v, q == par ? sign * h : 0.0};
+    };
+    Angles t;
+    t.s12 = angle(0, 0, 1.0);
+    t.c12 = angle(1, 0, -1.0);
+    t.s13 = angle(2, 1, 1.0);
+    t.c13 = angle(3, 1, -1.0);
+    t.s23 = angle(4, 2, 1.0);
+    t.c23 = angle(5, 2, -1.0);
+    if (!live) return;
+    double sd, cd;
+    sincos(o.delta_cp, &sd, &cd);
+    const Dn cosd{cd, q == 3 ? -sd : 0.0}, sind{sd, q == 3 ? cd : 0.0};
+    t.ep = cn(cosd, sind);
+    t.em = cn(cosd, -sind);
+    Cn Ua[3], Ub[3];
+    pmns_row(t, alpha, Ua);
+    pmns_row(t, beta, Ub);
+    const bool i1 = k == 0, j0 = k != 2;  // (i, j) = (1, 0), (2, 0), (2, 1)
+    const Cn X = conjn(pick(i1, Ua[1], Ua[2])) * pick(i1, Ub[1], Ub[2]) * pick(j0, Ua[0], Ua[1]) *
+                 conjn(pick(j0, Ub[0], Ub[1]));
+    const double sb = anti ? -4.0 : 4.0;
+    GenConst& gc = gout[p];
+    if (r < 12) {
+        const double da = -4.0 * X.re.d, db = sb * X.im.d;
+        gc.da[q][k] = da;
+        gc.db[q][k] = db;
+        gc.daf[q][k] = (float)da;
+        gc.dbf[q][k] = (float)db;
+        if (q == 0) {
+            const double a = -4.0 * X.re.v, b = sb * X.im.v;
+            const float af = (float)a, bf = (float)b;
+            gc.a[k] = a;
+            gc.b[k] = b;
+            gc.af[k] = af;
+            gc.bf[k] = bf;
+            gc.alo[k] = (float)(a - (double)af);
+            gc.blo[k] = (float)(b - (double)bf);
+        }
+    }
     if (r != 0) return;
-    pc.cmax = largest_phase(bc, o.dm2_21, o.dm2_32);
+    out[p].cmax = largest_phase(bc, o.dm2_21, o.dm2_32);
+    gc.dab = (alpha == beta) ? 1.0 : 0.0;
+    gc.wsum = bc.wsum_pair;
     const bool inside = o.s2_12 > 0.0 && o.s2_12 < 1.0 && o.s2_13 > 0.0 && o.s2_13 < 1.0 && o.s2_23 > 0.0 &&
                         o.s2_23 < 1.0 && isfinite(o.delta_cp) && isfinite(o.dm2_21) && isfinite(o.dm2_32);
     if (!inside && status) atomicExch(status, (int)GNA_EINVAL);
-    general_coefficients(o, alpha, beta, anti, gout[p]);
-    double w = 0.0;
-    for (int q = 0; q < bc.nL; q++) w += (double)bc.om[q] + (double)bc.omlo[q];
-    gout[p].wsum = w;
 }
 
 cudaError_t launch_prepare_general(const gna_osc_full* prm, int npts, const BaseConst& bc, int alpha, int beta,

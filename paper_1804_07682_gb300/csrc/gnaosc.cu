@@ -1045,6 +1045,7 @@ static gna_status plan_build(gna_plan* plan, const gna_plan_desc* d, cudaStream_
     bc.wsum_lo = fsum - (double)bc.wsum;
     double fall = 0.0;
     for (int r = 0; r < d->nL; r++) fall += (double)bc.om[r] + (double)bc.omlo[r];
+    bc.wsum_pair = fall;
     plan->wsum_all_lo = fall - (double)bc.wsum;
     // mapping and layouts
     const int ngroups = (d->nbins + 31) / 32;
