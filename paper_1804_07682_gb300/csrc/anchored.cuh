@@ -566,7 +566,7 @@ struct MultiMath {
 };
 
 template <int PH, int NP, bool GRAD>
-__global__ void __maxnreg__(NP == 4 ? 168 : 128) k_nodes_multi(BinArgs a) {
+__global__ void __maxnreg__(NP >= 3 ? 168 : 128) k_nodes_multi(BinArgs a) {
     using M = MultiMath<PH, NP, GRAD>;
     extern __shared__ f32x2p comp_all[];  // [NP * NS][blockDim], then the rings
     f32x2p* comp = comp_all + threadIdx.x;

@@ -1,5 +1,5 @@
 // anchored_launch.cuh -- choice of the chunk-anchored node kernel: one baseline
-// takes two nodes per packed value, more take 2, 4 or 8 baselines at a time
+// takes two nodes per packed value, more take 2, 4, 6 or 8 baselines at a time
 // (beyond 8 the nodes are taken again).
 #pragma once
 
@@ -26,12 +26,23 @@ cudaError_t launch_multi(const BinArgs& a, int grid, int block, cudaStream_t s) 
     return launch_dependent(k_nodes_multi<PH, NP, GRAD>, a, grid, block, s, nodes_smem<NP, GRAD>(block));
 }
 
+// Pairs of baselines taken at a time: up to four, the baselines spread evenly
+// over the passes over the nodes that this takes.  GB300, twelve as 6 + 6
+// instead of 8 + 4: 500 bins x 1000 nodes 43.8 -> 39.0 us, 127 x 67 41.0 -> 34.8.
+inline int baseline_pairs(int nL) {
+    const int passes = (nL + 7) / 8, per = (nL + passes - 1) / passes;
+    return (per + 1) / 2;
+}
+
 template <int PH, bool GRAD>
 cudaError_t launch_nodes_g(const BinArgs& a, int grid, int block, cudaStream_t s) {
     if (a.nL <= 1) return launch_dependent(k_nodes_one<PH, GRAD>, a, grid, block, s, one_smem(block));
-    if (a.nL <= 2) return launch_multi<PH, 1, GRAD>(a, grid, block, s);
-    if (a.nL <= 4) return launch_multi<PH, 2, GRAD>(a, grid, block, s);
-    return launch_multi<PH, 4, GRAD>(a, grid, block, s);
+    switch (baseline_pairs(a.nL)) {
+        case 1: return launch_multi<PH, 1, GRAD>(a, grid, block, s);
+        case 2: return launch_multi<PH, 2, GRAD>(a, grid, block, s);
+        case 3: return launch_multi<PH, 3, GRAD>(a, grid, block, s);
+        default: return launch_multi<PH, 4, GRAD>(a, grid, block, s);
+    }
 }
 
 template <int PH>
@@ -53,9 +64,12 @@ int resident_of(int block, size_t smem) {
 template <int PH, bool GRAD>
 int resident_nodes_g(int nL, int block) {
     if (nL <= 1) return resident_of<k_nodes_one<PH, GRAD>>(block, one_smem(block));
-    if (nL <= 2) return resident_of<k_nodes_multi<PH, 1, GRAD>>(block, nodes_smem<1, GRAD>(block));
-    if (nL <= 4) return resident_of<k_nodes_multi<PH, 2, GRAD>>(block, nodes_smem<2, GRAD>(block));
-    return resident_of<k_nodes_multi<PH, 4, GRAD>>(block, nodes_smem<4, GRAD>(block));
+    switch (baseline_pairs(nL)) {
+        case 1: return resident_of<k_nodes_multi<PH, 1, GRAD>>(block, nodes_smem<1, GRAD>(block));
+        case 2: return resident_of<k_nodes_multi<PH, 2, GRAD>>(block, nodes_smem<2, GRAD>(block));
+        case 3: return resident_of<k_nodes_multi<PH, 3, GRAD>>(block, nodes_smem<3, GRAD>(block));
+        default: return resident_of<k_nodes_multi<PH, 4, GRAD>>(block, nodes_smem<4, GRAD>(block));
+    }
 }
 
 template <int PH>

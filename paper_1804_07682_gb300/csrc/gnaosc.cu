@@ -140,6 +140,7 @@ struct gna_plan {
     int64_t ncounters = 0;
     int maxseg_cap = 2;  // split mapping: partial slots per (point, bin) the plan allocated
     int slices_cap = 0;  // slice mapping: slices per group the plan allocated (0: unavailable)
+    int fit_slices_cap = 0;  // of them, those the fits take (at least 16 nodes each)
     float2* d_slices = nullptr;  // [npts][ngroups][slices][NV][32]
     double* d_edges = nullptr;
     // constants
@@ -339,17 +340,26 @@ int grid_size(const gna_plan* p, int ctas_per_sm, int block, int64_t work_items)
 }
 
 // Slice mapping: S slices of L nodes per group of 32 bins.  All tasks take
-// the same time, so the default S is the one whose last round of tasks over
-// the resident warps wastes least: rounds x (nodes of a slice + a task's own
-// cost in nodes).
+// the same time, so the default S is the one of least cost: rounds of tasks
+// over the resident warps x (nodes of a slice + a task's own cost in nodes),
+// and what the second kernel takes for being there and for each slice.
 struct SliceShape {
     int S, L, ntasks;
 };
 
-// in nodes of the mixed-precision kernels
-constexpr int64_t kTaskCost = 6, kReduceCost = 16;
+// In nodes.  A node takes the mixed kernels longer with more baselines (about
+// 0.1 us at one, 0.4 us at eight, when the warp is alone on its quarter), the
+// second kernel 5 us and 0.05 us a slice whatever their number is.
+struct SliceCost {
+    int64_t task, reduce, slice8;  // slice8: per slice, in eighths
+};
 
-SliceShape slice_shape(gna_plan* p, int64_t resident_warps, int64_t task_cost, int64_t reduce_cost) {
+SliceCost slice_cost(const gna_plan* p) {
+    const int64_t nl = std::min(p->nL, 4);
+    return {6, 16 / nl, 4 / nl};
+}
+
+SliceShape slice_shape(gna_plan* p, int64_t resident_warps, SliceCost c) {
     const int n = p->n_uniform;
     const int64_t pg = (int64_t)p->npts * p->ngroups;
     const int64_t cap = std::max(1, p->slices_cap);
@@ -363,7 +373,7 @@ SliceShape slice_shape(gna_plan* p, int64_t resident_warps, int64_t task_cost, i
             const int64_t len = (n + S - 1) / S, used = (n + len - 1) / len;
             if (used != S) continue;  // same length as a smaller S
             const int64_t rounds = (pg * S + resident_warps - 1) / resident_warps;
-            const int64_t cost = rounds * (len + task_cost) + (S > 1 ? reduce_cost : 0);
+            const int64_t cost = 8 * rounds * (len + c.task) + (S > 1 ? 8 * c.reduce + S * c.slice8 : 0);
             if (best < 0 || cost < best) {
                 best = cost;
                 L = len;
@@ -456,8 +466,8 @@ SliceShape fixed_slice_shape(const gna_plan* p) {
         const int64_t S = std::max<int64_t>(1, (target + pg - 1) / pg);
         L = (n + S - 1) / S;
     }
-    if (p->slices_cap <= 1) L = n;
-    else L = std::max<int64_t>(L, (n + p->slices_cap - 1) / p->slices_cap);
+    if (p->fit_slices_cap <= 1) L = n;
+    else L = std::max<int64_t>(L, (n + p->fit_slices_cap - 1) / p->fit_slices_cap);
     L = std::min<int64_t>(std::max<int64_t>(L, 1), n);
     SliceShape sh;
     sh.L = (int)L;
@@ -496,7 +506,7 @@ gna_status enqueue_fit_nodes(gna_plan* plan, const EpiArgs& ea, cudaStream_t s, 
 gna_status enqueue_nodes64(gna_plan* plan, const EpiArgs& ea, bool grad, bool spec, cudaStream_t s, int* nl) {
     constexpr int kBlock = 128, kCtas = 4;
     SliceShape ssh{1, 0, plan->ntasks};
-    if (plan->uniform) ssh = slice_shape(plan, 16LL * plan->sm_count, 3, 2);
+    if (plan->uniform) ssh = slice_shape(plan, 16LL * plan->sm_count, SliceCost{3, 2, 0});
     if ((int64_t)plan->npts * plan->ngroups * ssh.S >= (1LL << 31)) return fail(plan, GNA_ESHAPE, "too many slice tasks");
     const bool sliced = ssh.S > 1;
     const int NVs = sums64(plan->general, grad) + (spec ? plan->nL : 0);
@@ -533,7 +543,7 @@ gna_status enqueue_eval(gna_plan* plan, const EvalReq& q, cudaStream_t s, int* l
     const int nblock = plan->ph < 2 ? nodes_block(plan->block) : plan->block;
     const int ctas = split || plan->ph == 2 ? 0 : node_ctas_per_sm(plan, grad, nblock);
     if (plan->mapping == MAP_SLICES && !fit) {
-        ssh = slice_shape(plan, (int64_t)plan->sm_count * ctas * (nblock / 32), kTaskCost, kReduceCost);
+        ssh = slice_shape(plan, (int64_t)plan->sm_count * ctas * (nblock / 32), slice_cost(plan));
         if ((int64_t)plan->npts * plan->ngroups * ssh.S >= (1LL << 31)) return fail(plan, GNA_ESHAPE, "too many slice tasks");
     }
     // work counter, per-point and per-bin arrival counters: zeroed by the
@@ -611,7 +621,7 @@ gna_status enqueue_eval_general(gna_plan* plan, const EvalReq& q, cudaStream_t s
                                    : node_ctas_per_sm(plan, grad, nblock);
     SliceShape ssh{1, 0, plan->ntasks};
     if (plan->mapping == MAP_SLICES) {
-        ssh = fit ? fixed_slice_shape(plan) : slice_shape(plan, (int64_t)plan->sm_count * ctas * (nblock / 32), kTaskCost, kReduceCost);
+        ssh = fit ? fixed_slice_shape(plan) : slice_shape(plan, (int64_t)plan->sm_count * ctas * (nblock / 32), slice_cost(plan));
         if ((int64_t)plan->npts * plan->ngroups * ssh.S >= (1LL << 31)) return fail(plan, GNA_ESHAPE, "too many slice tasks");
     }
     const int64_t ncnt = 1 + (int64_t)plan->npts * (1 + plan->ngroups);
@@ -1247,12 +1257,16 @@ static gna_status plan_build(gna_plan* plan, const gna_plan_desc* d, cudaStream_
         TRY(dalloc(plan, (double**)&plan->d_part, plan->part_cap));
     }
     if (plan->uniform && plan->has_bins) {
-        // slices per group: up to 8 tasks per resident warp, at least 16 nodes per
-        // slice (GNA_FP64: eight tasks per SM quarter, four nodes)
+        // slices per group: up to 8 tasks per resident warp (GNA_FP64: per SM
+        // quarter), at least a quad of nodes each: a small point's few quads are
+        // worth a warp each (GB300, 200 bins x 50 nodes x 8
+        // baselines: 28.7 us with 16 nodes a slice, 22.5 with what slice_shape takes;
+        // 40 x 20 x 8: 28.1 and 18.5)
         const int64_t pg = (int64_t)d->npts * ngroups;
         const int64_t by_tasks = ((plan->ph == 2 ? 32LL * plan->sm_count : 8 * warps_est) + pg - 1) / pg;
-        const int64_t by_len = std::max<int64_t>(1, plan->n_uniform / (plan->ph == 2 ? 4 : 16));
+        const int64_t by_len = std::max<int64_t>(1, plan->ph == 2 ? plan->n_uniform / 4 : (plan->n_uniform + 3) / 4);
         plan->slices_cap = (int)std::max<int64_t>(1, std::min(by_tasks, by_len));
+        plan->fit_slices_cap = (int)std::max<int64_t>(1, std::min<int64_t>(plan->slices_cap, plan->n_uniform / 16));
         if (plan->slices_cap > 1)
             TRY(dalloc(plan, &plan->d_slices, (size_t)pg * plan->slices_cap * nv_max * 32));
     }

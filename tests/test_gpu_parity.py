@@ -1210,3 +1210,30 @@ def test_oscprob_number_ranges(api, prec):
             small = ok & (phase < 1e-2)
             assert (np.abs(P - ref)[small] <= 1e-15 * phase[small] + (3e-16 if channel != ("mu", "e") else 0)).all()
             assert np.isnan(P[1:, -1]).all()
+
+
+@pytest.mark.parametrize("nL", [2, 5, 6, 9, 12, 16])
+@pytest.mark.parametrize("nodes", [3, 10, 50, 129])
+def test_baseline_groups_and_short_slices(api, nL, nodes):
+    """Baselines taken 2, 4, 6 or 8 at a time in one or two passes, and slices
+    down to one quad of nodes, against the kernel-per-step FP64 chain."""
+    rng = np.random.default_rng(nL * 100 + nodes)
+    edges = np.linspace(1.8, 8.0, 71)
+    L = list(rng.uniform(1.0, 60.0, nL))
+    th = np.array([[0.307, 0.0218, 7.53e-5, 2.44e-3]])
+    plain = api.Plan(edges, L, nodes_per_bin=nodes, prec="fp64", kind="poisson", with_plain=True)
+    ref0 = plain.eval(plain.params_tensor(th), dev(np.full(70, 1.0)), grad=True, spectra=True, mu=True)
+    data = dev(rng.poisson(1e4 * ref0["mu"].cpu().numpy().ravel() / ref0["mu"].max().item()) * 1.0)
+    norm = 1e4 / ref0["mu"].max().item()
+    out = {}
+    for prec in ("fp64", "ff"):
+        plan = api.Plan(edges, L, nodes_per_bin=nodes, prec=prec, kind="poisson", norm=norm, with_plain=prec == "fp64")
+        out[prec] = plan.eval(plan.params_tensor(th), data, grad=True, spectra=True, plain=prec == "fp64")
+        chi_only = plan.eval(plan.params_tensor(th), data)["chi2"]
+        assert rel(chi_only.cpu().numpy(), out[prec]["chi2"].cpu().numpy()) < 1e-6
+    a, b = out["ff"], out["fp64"]
+    assert rel(a["spectra"].cpu().numpy(), b["spectra"].cpu().numpy()) < 1e-6
+    # chi^2 within 1e-6 of what a relative change of every mu_i makes of it
+    scale = max(b["chi2"].item(), 2 * float(torch.sqrt(data).sum()))
+    assert abs(a["chi2"].item() - b["chi2"].item()) < 1e-6 * scale
+    assert normrel(a["grad"].cpu().numpy(), b["grad"].cpu().numpy()) < 1e-4
