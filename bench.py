@@ -86,13 +86,13 @@ PROFILE_EVERY = 8
 TRAFFIC_CAPTURE = {
     "split": {"sources_sha256": "4e84d90634a932986bddfc3627e81e2c61c0ee248b37d8a2b42cd44e71396f94",
               "bytes": 265113600 + 4114176},
-    "slices": {"sources_sha256": "ee1c2edc308edbe2ecc5ca374d8666315fc1bb510abdc327df76998aaec7e7e2",
-               "bytes": 268506880 + 4611584 + 8178176 + 0},
+    "slices": {"sources_sha256": "758a3ede1b15d5e3d1203945af46e51ec9d5aceb2947f384eeee84720709fbb9",
+               "bytes": 201989376 + 3093760 + 6620928 + 0},
 }
 KERNEL_SOURCES = ["paper_1804_07682_gb300/csrc/common.cuh", "paper_1804_07682_gb300/csrc/fused.cuh",
                   "paper_1804_07682_gb300/csrc/anchored.cuh",
                   "paper_1804_07682_gb300/csrc/epilogue.cuh", "paper_1804_07682_gb300/csrc/ff_consts.h",
-                  "paper_1804_07682_gb300/csrc/slices.cu"]
+                  "paper_1804_07682_gb300/csrc/slices.cuh", "paper_1804_07682_gb300/csrc/slices.cu"]
 KERNEL_NAMES = {"split": "k_fused_split", "slices": "k_nodes_multi (slices) + k_slices_reduce",
                 "bins": "k_nodes_multi + k_point_sums"}
 

@@ -98,11 +98,12 @@ typedef struct {
 } gna_plan_desc;
 
 #define GNA_PLAN_WITH_PLAIN 1  /* also build the FP64 arrays and scratch of gna_chain_eval_plain */
-#define GNA_PLAN_FORCE_SPLIT 2 /* equal node ranges per warp across bins (default in FP64 for >= 1024 nodes/bin) */
-#define GNA_PLAN_FORCE_BINS 4  /* one thread per bin (default for small or per-point grids) */
+#define GNA_PLAN_FORCE_SPLIT 2 /* equal node ranges per warp across bins */
+#define GNA_PLAN_FORCE_BINS 4  /* one thread per bin (default for per-point grids, many points, and GNA_FP64) */
 #define GNA_PLAN_FORCE_SLICES 8 /* one thread per bin and slice of its nodes, slices summed by a
                                    second kernel (default for uniform grids in the mixed
-                                   precisions when points x bin groups are too few to fill the GPU) */
+                                   precisions when points x bin groups are too few to fill the GPU;
+                                   in GNA_FP64 the bins of uniform grids are cut by themselves) */
 #define GNA_PLAN_GENERAL 16     /* the chain for any channel (alpha, beta, anti above), evaluated by
                                    gna_chain_eval_general: up to 8 baselines; in the mixed
                                    precisions the slice mapping on equal node counts and the bin
@@ -421,8 +422,10 @@ gna_status gna_fit_batch_general(gna_plan* plan, gna_osc_full* params, const dou
  * fastest.  The evaluations write the outputs `out` names (device pointers,
  * as for gna_chain_eval: the kernels differ with the outputs requested), or,
  * with out == NULL, chi^2 and the gradient into plan scratch.  The choice can
- * be read back and restored as text ("mapping=slices block=256 nodes=16
- * grid=0 slice=216") for caching between runs.
+ * be read back and restored as text ("mapping=slices block=128 nodes=16
+ * grid=0 slice=216"; slice=0: the plan's own choice; the mixed evaluations
+ * by bins and slices use at most 128 threads per block and round the slice
+ * length up to whole quads of nodes) for caching between runs.
  */
 gna_status gna_plan_autotune(gna_plan* plan, const gna_osc* params, const double* data, int data_per_point,
                              const gna_outputs* out, int reps, void* stream);

@@ -1,8 +1,7 @@
 // kernels_misc.cu -- everything on the device except the fused node loop:
 // parameter preparation (step a0), the Gauss-Legendre rule and energy grids
 // (step a1, configuration stage), the chi^2 epilogue (steps a7-a9), the plain
-// FP64 one-kernel-per-transformation chain, the element-wise OscProb
-// transformation and the Levenberg-Marquardt update.
+// FP64 one-kernel-per-transformation chain and the Levenberg-Marquardt update.
 #include <math.h>
 
 #include "common.cuh"
