@@ -19,8 +19,10 @@ KINDS = {"pearson": N.GNA_PEARSON, "poisson": N.GNA_POISSON, 0: N.GNA_PEARSON, 1
 
 
 def _stream(stream=None) -> int:
-    s = stream if stream is not None else torch.cuda.current_stream()
-    return s.cuda_stream
+    if stream is not None:
+        return stream.cuda_stream
+    # the handle alone: building torch's Stream object takes longer than a launch
+    return torch._C._cuda_getCurrentRawStream(torch.cuda.current_device())
 
 
 def _ptr_any(t: torch.Tensor):
@@ -47,6 +49,27 @@ def _require_cuda():
     if not torch.cuda.is_available():
         raise RuntimeError("the oscillation library needs a CUDA device")
     N.lib()
+
+
+def _require_cuda_for(E):
+    """_require_cuda for a call on E: a CUDA tensor shows that there is a device."""
+    if not E.is_cuda:
+        _require_cuda()
+
+
+def _doubles(a):
+    """(count, argument) of a short host array of doubles: lists and tuples of
+    numbers go straight into a ctypes array (numpy's pointer cast alone takes
+    microseconds), anything else through numpy."""
+    if type(a) in (list, tuple):
+        try:
+            return len(a), (ctypes.c_double * len(a))(*a)
+        except TypeError:
+            pass
+    v = _f64(a)
+    arg = v.ctypes.data_as(ctypes.POINTER(ctypes.c_double))
+    arg._kept = v  # alive as long as the pointer
+    return v.size, arg
 
 
 def _f64(a):
@@ -83,16 +106,16 @@ def oscprob(E: torch.Tensor, L: Sequence[float], theta: Sequence[float], prec: s
             out: Optional[torch.Tensor] = None) -> torch.Tensor:
     """Element-wise OscProb: P(nue_bar -> nue_bar) [nL, n] at energies E (MeV) for baselines L (km).
     E and out may be CUDA tensors or pinned host memory (the kernel reads and writes it in place)."""
-    _require_cuda()
+    _require_cuda_for(E)
     if E.dtype != torch.float64:
         raise ValueError("E must be float64")
     if not E.is_cuda and not E.is_pinned():
         raise ValueError("E must be a CUDA tensor or pinned host memory")
-    Ls = _f64(L)
+    nL, Ls = _doubles(L)
     p = N.GnaOsc(*[float(t) for t in theta])
-    P = _oscprob_out(E, Ls.size, prec, out)
-    code = N.lib().gna_oscprob_ee(_ptr_any(E), E.numel(), Ls.ctypes.data_as(ctypes.POINTER(ctypes.c_double)),
-                                  Ls.size, ctypes.byref(p), PRECISIONS[prec], _ptr_any(P), ctypes.c_void_p(_stream()))
+    P = _oscprob_out(E, nL, prec, out)
+    code = N.lib().gna_oscprob_ee(_ptr_any(E), E.numel(), Ls, nL, ctypes.byref(p), PRECISIONS[prec], _ptr_any(P),
+                                  ctypes.c_void_p(_stream()))
     N.check(code, what="gna_oscprob_ee")
     return P
 
@@ -138,18 +161,18 @@ def oscprob_general(E: torch.Tensor, L: Sequence[float], theta_full: Sequence[fl
     """Element-wise OscProb for any channel: P(alpha -> beta) [nL, n] at energies E (MeV) for
     baselines L (km); theta_full = (s2_12, s2_13, s2_23, delta_cp, dm2_21, dm2_32).  E and out
     may be CUDA tensors or pinned host memory."""
-    _require_cuda()
+    _require_cuda_for(E)
     if E.dtype != torch.float64:
         raise ValueError("E must be float64")
     if not E.is_cuda and not E.is_pinned():
         raise ValueError("E must be a CUDA tensor or pinned host memory")
     a = FLAVOURS.get(alpha, alpha)
     b = FLAVOURS.get(beta, beta)
-    Ls = _f64(L)
+    nL, Ls = _doubles(L)
     p = N.GnaOscFull(*[float(t) for t in theta_full])
-    P = _oscprob_out(E, Ls.size, prec, out)
-    code = N.lib().gna_oscprob(_ptr_any(E), E.numel(), Ls.ctypes.data_as(ctypes.POINTER(ctypes.c_double)),
-                               Ls.size, int(a), int(b), int(bool(anti)), ctypes.byref(p), PRECISIONS[prec], _ptr_any(P),
+    P = _oscprob_out(E, nL, prec, out)
+    code = N.lib().gna_oscprob(_ptr_any(E), E.numel(), Ls, nL, int(a), int(b),
+                               int(bool(anti)), ctypes.byref(p), PRECISIONS[prec], _ptr_any(P),
                                ctypes.c_void_p(_stream()))
     N.check(code, what="gna_oscprob")
     return P
