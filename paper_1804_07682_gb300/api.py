@@ -338,7 +338,7 @@ class Plan:
         o.grad_eta = None if g_eta is None else g_eta.data_ptr()
         fn = self._lib.gna_chain_eval if self.channel is None else self._lib.gna_chain_eval_general
         code = fn(self._h, p.data_ptr(), None if e is None else e.data_ptr(), float(sigma), data.data_ptr(), 0,
-                  ctypes.byref(o), torch.cuda.current_stream().cuda_stream)
+                  ctypes.byref(o), _stream())
         if code != N.GNA_OK:
             self._check(code, "gna_chain_eval")
 
@@ -650,7 +650,7 @@ class OscChi2(torch.autograd.Function):
             raise ValueError("OscChi2: grad_output must be a float64 scalar on the evaluation's device")
         code = ctx.lib.gna_grad_scale(gt.data_ptr(), gt.numel(), None if ge is None else ge.data_ptr(),
                                       0 if ge is None else ge.numel(), go.data_ptr(),
-                                      torch.cuda.current_stream(gt.device).cuda_stream)
+                                      torch._C._cuda_getCurrentRawStream(gt.device.index))
         N.check(code, what="gna_grad_scale")
         return gt, ge, None, None, None
 
