@@ -348,15 +348,16 @@ struct SliceShape {
 };
 
 // In nodes.  A node takes the mixed kernels longer with more baselines (about
-// 0.1 us at one, 0.4 us at eight, when the warp is alone on its quarter), the
-// second kernel 5 us and 0.05 us a slice whatever their number is.
+// 0.1 us at one, 0.4 us at eight, when the warp is alone on its quarter); the
+// second kernel, which also does the bins' epilogue, takes about 1 us more than
+// a whole bin's end, and 0.05 us a slice, whatever their number is.
 struct SliceCost {
     int64_t task, reduce, slice8;  // slice8: per slice, in eighths
 };
 
 SliceCost slice_cost(const gna_plan* p) {
     const int64_t nl = std::min(p->nL, 4);
-    return {6, 16 / nl, 4 / nl};
+    return {6, 8 / nl, 4 / nl};
 }
 
 SliceShape slice_shape(gna_plan* p, int64_t resident_warps, SliceCost c) {
