@@ -1261,7 +1261,7 @@ static gna_status plan_build(gna_plan* plan, const gna_plan_desc* d, cudaStream_
         // slices per group: up to 8 tasks per resident warp (GNA_FP64: per SM
         // quarter), at least a quad of nodes each: a small point's few quads are
         // worth a warp each (GB300, 200 bins x 50 nodes x 8
-        // baselines: 28.7 us with 16 nodes a slice, 22.5 with what slice_shape takes;
+        // baselines: 28.7 us with 16 nodes a slice, 20.5 with what slice_shape takes;
         // 40 x 20 x 8: 28.1 and 18.5)
         const int64_t pg = (int64_t)d->npts * ngroups;
         const int64_t by_tasks = ((plan->ph == 2 ? 32LL * plan->sm_count : 8 * warps_est) + pg - 1) / pg;
