@@ -425,7 +425,11 @@ gna_status gna_fit_batch_general(gna_plan* plan, gna_osc_full* params, const dou
  * be read back and restored as text ("mapping=slices block=128 nodes=16
  * grid=0 slice=216"; slice=0: the plan's own choice; the mixed evaluations
  * by bins and slices use at most 128 threads per block and round the slice
- * length up to whole quads of nodes) for caching between runs.
+ * length up to whole quads of nodes) for caching between runs.  A GNA_FP64
+ * plan whose fits use the split mapping while its evaluations go by bins (the
+ * default for >= 1024 nodes per bin or few points) has " fit=split" at the
+ * text's end; autotuning keeps it, a text that names another mapping than the
+ * plan's without it moves the fits to that mapping too.
  */
 gna_status gna_plan_autotune(gna_plan* plan, const gna_osc* params, const double* data, int data_per_point,
                              const gna_outputs* out, int reps, void* stream);

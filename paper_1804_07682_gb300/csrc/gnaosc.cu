@@ -104,7 +104,7 @@ struct gna_plan {
     int prec = GNA_MIXED_FFPHASE, kind = GNA_PEARSON, flags = 0, max_datasets = 0;
     int mapping = MAP_SPLIT;
     // GNA_FP64 plans evaluate by bins (nodes64.cuh); their fits use the split
-    // mapping where it was the default and none was asked for
+    // mapping where it was the default, until a tuning says otherwise
     bool fit_split = false;
     int sm_count = 0;
     // any-channel plans (GNA_PLAN_GENERAL): P(g_alpha -> g_beta), antineutrinos
@@ -1780,8 +1780,8 @@ gna_status gna_fit_batch_general(gna_plan* plan, gna_osc_full* params, const dou
 gna_status gna_plan_get_tuning(const gna_plan* plan, char* buf, int buflen) {
     if (!plan || !buf || buflen < 1) return GNA_EINVAL;
     static const char* names[3] = {"split", "bins", "slices"};
-    snprintf(buf, buflen, "mapping=%s block=%d nodes=%d grid=%d slice=%d", names[plan->mapping], plan->block, plan->npt,
-             plan->grid_mult, plan->slice_len);
+    snprintf(buf, buflen, "mapping=%s block=%d nodes=%d grid=%d slice=%d%s", names[plan->mapping], plan->block, plan->npt,
+             plan->grid_mult, plan->slice_len, plan->fit_split ? " fit=split" : "");
     return GNA_OK;
 }
 
@@ -1793,6 +1793,7 @@ gna_status gna_plan_set_tuning(gna_plan* plan, const char* text) {
     const char* g = strstr(text, "grid=");
     const char* m = strstr(text, "mapping=");
     const char* c = strstr(text, "slice=");
+    const char* f = strstr(text, "fit=");
     if (b) block = atoi(b + 6);
     if (n) npt = atoi(n + 6);
     if (g) gm = atoi(g + 5);
@@ -1802,6 +1803,13 @@ gna_status gna_plan_set_tuning(gna_plan* plan, const char* text) {
         else if (!strncmp(m + 8, "bins", 4)) mapping = MAP_BINS;
         else if (!strncmp(m + 8, "slices", 6)) mapping = MAP_SLICES;
         else return fail(plan, GNA_EINVAL, "bad mapping in '%s'", text);
+    }
+    // the fits follow another mapping of the evaluations unless the text keeps them on the split one
+    bool fit_split = plan->fit_split && mapping == plan->mapping;
+    if (f) {
+        if (!strncmp(f + 4, "split", 5)) fit_split = true;
+        else return fail(plan, GNA_EINVAL, "bad fit mapping in '%s'", text);
+        if (!plan->has_split || plan->general) return fail(plan, GNA_EINVAL, "the plan has no grid for the split mapping");
     }
     if (block < 32 || block > 256 || (block & 31) || npt < 1 || npt > 1024 || gm < 0 || gm > 64 || sl < 0)
         return fail(plan, GNA_EINVAL, "bad tuning '%s'", text);
@@ -1816,7 +1824,7 @@ gna_status gna_plan_set_tuning(gna_plan* plan, const char* text) {
     plan->npt = npt;
     plan->grid_mult = gm;
     plan->mapping = mapping;
-    if (m) plan->fit_split = false;
+    plan->fit_split = fit_split;
     plan->slice_len = sl;
     destroy_graph(plan);
     return GNA_OK;
@@ -1829,6 +1837,7 @@ extern "C++" template <typename Eval>
 gna_status time_candidates(gna_plan* plan, const std::vector<std::string>& cand, int reps, cudaStream_t s, Eval eval) {
     char best_t[128];
     gna_plan_get_tuning(plan, best_t, sizeof(best_t));
+    const bool fit_split = plan->fit_split;  // evaluations are timed: the fits' mapping stays
     float best = 1e30f;
     cudaEvent_t e0, e1;
     CU(cudaEventCreate(&e0));
@@ -1850,6 +1859,7 @@ gna_status time_candidates(gna_plan* plan, const std::vector<std::string>& cand,
     cudaEventDestroy(e0);
     cudaEventDestroy(e1);
     gna_status st = gna_plan_set_tuning(plan, best_t);
+    plan->fit_split = fit_split;
     cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess) return fail(plan, GNA_ECUDA, "autotune: %s", cudaGetErrorString(e));
     return st;
@@ -1866,7 +1876,6 @@ gna_status gna_plan_autotune(gna_plan* plan, const gna_osc* params, const double
     std::vector<std::string> cand;
     const int blocks[3] = {64, 128, 256};
     char t[96];
-    const bool nodes128 = plan->ph < 2;  // the bin and slice kernels take blocks of at most 128 threads
     if (plan->has_split) {
         // block size only changes how the equal ranges sit on the SMs; the
         // minimum range length matters only for workloads smaller than the GPU
@@ -1877,12 +1886,16 @@ gna_status gna_plan_autotune(gna_plan* plan, const gna_osc* params, const double
                 cand.push_back(t);
             }
     }
-    if (plan->has_bins)
-        for (int b : blocks) {
-            if (nodes128 && b > 128) continue;
+    if (plan->has_bins && plan->ph == 2) {
+        // nodes64.cuh has one block size: the block and nodes of this text are the fits'
+        snprintf(t, sizeof(t), "mapping=bins block=%d nodes=%d", plan->block, plan->npt);
+        cand.push_back(t);
+    } else if (plan->has_bins) {
+        for (int b : {64, 128}) {  // the bin and slice kernels take blocks of at most 128 threads
             snprintf(t, sizeof(t), "mapping=bins block=%d nodes=1", b);
             cand.push_back(t);
         }
+    }
     if (plan->has_bins && plan->uniform && plan->ph < 2 && plan->slices_cap > 1) {
         // the chosen slice length, and lengths for about 1, 2 and 4 tasks per
         // 16 warps on each SM

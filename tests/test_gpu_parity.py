@@ -1237,3 +1237,37 @@ def test_baseline_groups_and_short_slices(api, nL, nodes):
     scale = max(b["chi2"].item(), 2 * float(torch.sqrt(data).sum()))
     assert abs(a["chi2"].item() - b["chi2"].item()) < 1e-6 * scale
     assert normrel(a["grad"].cpu().numpy(), b["grad"].cpu().numpy()) < 1e-4
+
+
+@pytest.mark.parametrize("nbins,n", [(200, 50), (40, 1031)])
+def test_fp64_fits_keep_their_mapping_through_tuning(api, nbins, n):
+    """The fits of a default GNA_FP64 plan run in the split mapping while its
+    evaluations go by bins: reading the tuning and setting it back, and
+    autotuning the evaluations, change no bit of a fit."""
+    edges, L = np.linspace(1.8, 8.0, nbins + 1), [52.5, 30.0]
+    th = np.array(wl.TRUTH)
+    Nn = oracle.norm_for_total(edges, n, L, wl.TRUTH)
+    data = dev(wl.pseudo_datasets(Nn * (oracle.baseline_weights(L) @ oracle.binned(edges, n, L, wl.TRUTH)), 2, 5))
+    plan = api.Plan(edges, L, nodes_per_bin=n, npts=2, norm=Nn, prec="fp64", kind="poisson", max_datasets=2)
+
+    def fit():
+        p, c = plan.fit(plan.params_tensor(np.repeat(1.02 * th[None], 2, 0)), data, iters=6)
+        return np.concatenate([p.cpu().numpy().ravel(), c.cpu().numpy()])
+
+    first = fit()
+    plan.tuning = plan.tuning
+    assert np.array_equal(first, fit())
+    assert plan.tuning.startswith("mapping=bins") and plan.tuning.endswith("fit=split")
+    if plan.autotune(plan.params_tensor(np.repeat(th[None], 2, 0)), data[0].contiguous(), reps=2).startswith("mapping=bins"):
+        assert np.array_equal(first, fit())
+    plan.tuning = "mapping=split block=256 nodes=16"  # named: evaluations and fits
+    assert np.array_equal(first, fit())
+    plan.tuning = "mapping=bins"
+    assert "fit" not in plan.tuning
+    by_bins = fit()
+    assert rel(by_bins, first) < 1e-6
+    plan.tuning = "fit=split"
+    assert np.array_equal(first, fit())
+    with pytest.raises(N.GnaError):
+        plan.tuning = "fit=slices"
+    plan.close()
