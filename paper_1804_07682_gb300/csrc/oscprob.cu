@@ -57,7 +57,7 @@ namespace {
 // ------------------------------------------------------------------ FP64 --
 // The double path, for the elements outside turns.cuh's range: energies that
 // are not positive normal numbers, phases of more than 2^30 half-turns or next
-// to zero.
+// to zero, and probabilities next to zero.
 __device__ __noinline__ double osc_double(const OscConst& oc, int r, double E) {
     const double e = 1.0 / E;
     const double s21 = sin(oc.c21[r] * e), s32 = sin(oc.c32[r] * e), s31 = sin((oc.c21[r] + oc.c32[r]) * e);
@@ -96,6 +96,13 @@ struct ElemTurns {
     }
 };
 
+// The integers carry P to a few units of 2^-61 of its largest value, whatever
+// its own size is.  The formula in double is a sum of squares where P has a
+// zero (two equal splittings or one that vanishes, maximal mixing): it stays
+// at or above zero there and its error, about 2^-50 sqrt(P), falls with P.
+// The two errors meet at 2^-16; below it P is taken from the formula.
+constexpr int64_t kSmallTurns = 1ll << (61 - 16);
+
 // Everything in 64-bit integers (turns.cuh): what bounds it is the issue of
 // some eighty wide integer multiplies and their shifts and additions per
 // probability, in place of three double sines (27 FP64 instructions each, at
@@ -132,7 +139,7 @@ __global__ void __launch_bounds__(256) k_osc_fp64(const double* __restrict__ E, 
             }
             double p = __ll2double_rn(v);  // P 2^(61 + scale)
             if (v != 0) p = __hiloint2double(__double2hiint(p) - ((61 + oc.t.scale) << 20), __double2loint(p));
-            if (!in) p = osc_double(oc, r, e);
+            if (!in || v < kSmallTurns) p = osc_double(oc, r, e);
             P[(int64_t)r * n + k] = p;
         }
     }

@@ -1271,3 +1271,34 @@ def test_fp64_fits_keep_their_mapping_through_tuning(api, nbins, n):
     with pytest.raises(N.GnaError):
         plan.tuning = "fit=slices"
     plan.close()
+
+
+def test_oscprob_fp64_next_to_its_zeros(api):
+    """P(mu -> e) with dm2_21 = 0 vanishes where x32 is a multiple of pi, and
+    the survival probability at maximal mixing where x21 is an odd multiple of
+    pi / 2: P stays at or above zero there and follows the closed form."""
+    ld = np.longdouble
+    K = ld(10) ** 3 / (4 * ld("0.1973269804"))
+    rng = np.random.default_rng(8)
+    off = np.concatenate([10.0 ** rng.uniform(-12, -0.5, 20000), [0.0]]) * rng.choice([-1.0, 1.0], 20001)
+    pi = ld("3.14159265358979323846264338327950288")
+    for form, x0, L in (("mu-e", pi, 810.0), ("mu-e", 7 * pi, 1300.0), ("max", pi / 2, 52.5), ("max", 7 * pi / 2, 180.0)):
+        c = K * (ld(2.44e-3) if form == "mu-e" else ld(7.53e-5)) * ld(L)
+        E = (c / (x0 + off)).astype(np.float64)
+        if form == "mu-e":
+            s13, s23 = 0.0218, 0.545
+            P = api.oscprob_general(dev(E), [L], (0.307, s13, s23, 0.7, 0.0, 2.44e-3), "mu", "e", prec="fp64")
+            A, x = 4 * ld(s23) * ld(s13) * (1 - ld(s13)), c / E.astype(ld)
+        else:
+            P = api.oscprob(dev(E), [L], (0.5, 0.0, 7.53e-5, 0.0), "fp64")
+            A, x = ld(1), c / E.astype(ld) - pi / 2
+        P, s = P[0].cpu().numpy(), np.abs(np.sin(x))
+        ref = A * s * s
+        # the phase is good to 4 roundings of 2^-53, in the closed form and the
+        # library's constants; the sum of up to three terms to 2^-50 of itself
+        dx = 4 * 2.0 ** -53 * float(x0)
+        tol = A * (2 * s * dx + dx * dx) + 2.0 ** -50 * ref
+        if form == "max":  # one minus a square: 2^-52 of one
+            tol = tol + 2.0 ** -52
+        assert (P >= 0).all(), (form, float(x0), P.min())
+        assert (np.abs(P - ref) <= tol).all(), (form, float(x0), float((np.abs(P - ref) / tol).max()))
