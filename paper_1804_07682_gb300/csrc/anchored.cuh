@@ -794,7 +794,8 @@ __global__ void __maxnreg__(112) k_nodes_one(BinArgs a) {
                     for (int j = ka; j < kb; j++) {
                         in.wait();
                         const NodePair n[2] = {in.pair(0), in.pair(1)};
-                        w.add(add2(n[0].w, n[1].w));
+                        w.add(n[0].w);
+                        w.add(n[1].w);
                         x.pairs(n, nah, nal);
                         in.done();
                     }

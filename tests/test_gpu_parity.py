@@ -1302,3 +1302,33 @@ def test_oscprob_fp64_next_to_its_zeros(api):
             tol = tol + 2.0 ** -52
         assert (P >= 0).all(), (form, float(x0), P.min())
         assert (np.abs(P - ref) <= tol).all(), (form, float(x0), float((np.abs(P - ref) / tol).max()))
+
+
+@pytest.mark.parametrize("prec", ["f64phase", "ff"])
+@pytest.mark.parametrize("nL", [1, 2])
+@pytest.mark.parametrize("general", [False, True])
+@pytest.mark.parametrize("n", [7, 64, 129])
+def test_chunk_weights_where_p_vanishes(api, general, nL, prec, n):
+    """Maximal two-flavour mixing at an oscillation minimum: P is the square of
+    a small angle, and the prediction what is left of the bin's weight when the
+    chunks' weights are taken from it: their sums hold to 2^-38 of the weight."""
+    K = 1e3 / (4 * 0.1973269804)
+    L, dm = 52.5, 7.53e-5
+    E0 = K * dm * L / (np.pi / 2)
+    e = np.linspace(E0 * (1 - 1e-5), E0 * (1 + 1e-5), 34)
+    mid = 0.5 * (e[1:] + e[:-1])
+    if general:  # nu_e survival of the any-channel chain (mixing inside (0, 1))
+        th, kw = [0.5, 1e-15, 0.5, 0.3, dm, 1e-12], dict(channel=("e", "e", False))
+    else:
+        th, kw = [0.5, 0.0, dm, 0.0], {}
+    plan = api.Plan(e, [L] * nL, nodes_per_bin=n, prec=prec, kind="poisson", **kw)
+    p, d = plan.params_tensor(th), dev(np.ones(33))
+    mu = (plan.eval_general if general else plan.eval)(p, d, grad=True, mu=True)["mu"][0].cpu().numpy()
+    plan.status()
+    plan.close()
+    W = np.exp(0.87 - 0.16 * mid - 0.091 * mid * mid) * np.diff(e)
+    x = K * dm * L / np.linspace(e[:-1], e[1:], 33)
+    ref = W * (np.cos(x) ** 2).mean(axis=0)  # P <= 2.5e-10
+    # 2^-38 of the weight from the sums; the reduced phase of pi holds to 2^-24
+    # of the largest offset, 1.6e-5 (its square to 2^-23)
+    assert (np.abs(mu - ref) <= W * (2.0 ** -38 + 2.0 ** -22 * 2.5e-10)).all(), float((np.abs(mu - ref) / W).max())
