@@ -1332,3 +1332,34 @@ def test_chunk_weights_where_p_vanishes(api, general, nL, prec, n):
     # 2^-38 of the weight from the sums; the reduced phase of pi holds to 2^-24
     # of the largest offset, 1.6e-5 (its square to 2^-23)
     assert (np.abs(mu - ref) <= W * (2.0 ** -38 + 2.0 ** -22 * 2.5e-10)).all(), float((np.abs(mu - ref) / W).max())
+
+
+@pytest.mark.parametrize("prec", ["f64phase", "ff"])
+@pytest.mark.parametrize("channel", [None, ("mu", "mu", False)])
+@pytest.mark.parametrize("mapping", ["bins", "slices"])
+@pytest.mark.parametrize("norm,top", [(1e60, 15.0), (1e-30, 15.0), (1e-44, 15.0), (1e-60, 15.0), (1e-20, 30.0), (1e33, 36.0)])
+def test_normalisations_of_any_size(api, prec, channel, mapping, norm, top):
+    """Normalisations and predictions outside the range of a float: the
+    prediction scales with the normalisation (up to 36 MeV the spectrum falls
+    by 45 orders of magnitude), and so do the derivatives by the nuisances
+    where the prediction is a float (their residual is one)."""
+    e = np.linspace(1.8, top, 41)
+    L, th = [52.5, 30.0], [0.307, 0.0218, 7.53e-5, 2.44e-3]
+    if channel:
+        th = [0.307, 0.0218, 0.545, 0.7, 7.53e-5, 2.44e-3]
+    out = {}
+    for N_, pr in ((1.0, "fp64"), (norm, prec)):
+        plan = api.Plan(e, L, nodes_per_bin=20, norm=N_, prec=pr, kind="poisson", channel=channel,
+                        mapping=None if pr == "fp64" or (channel and mapping == "slices") else mapping)
+        f = plan.eval if channel is None else plan.eval_general
+        o = f(plan.params_tensor(th), dev(np.zeros(40)), eta=dev(np.linspace(-0.5, 1.0, 40)), sigma=0.0, grad=True,
+              grad_eta=True, mu=True)
+        out[pr] = o["mu"][0].cpu().numpy(), o["grad_eta"][0].cpu().numpy()
+        plan.status()
+        plan.close()
+    ref, got = out["fp64"], out[prec]
+    # weights are FP32: below 2^-126 they keep 2^-149 of one each (2 MeV wide bins, 20 nodes)
+    low = 20 * 2.0 ** -149
+    a_float = (ref[0] * norm > 1e-37) & (ref[0] * norm < 1e38) & (ref[0] > 1e-37)
+    for a, b, ok in zip(got, ref, (np.ones(40, bool), a_float)):
+        assert (np.abs(a / norm - b) <= 2e-6 * np.abs(b) + 4 * low)[ok].all(), (a / norm, b)
