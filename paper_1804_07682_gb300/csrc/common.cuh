@@ -33,7 +33,8 @@ struct PointConst {
     double dA12[3];  // d A_ij / d sin^2 theta12
     double dA13[3];  // d A_ij / d sin^2 theta13
     float Af[3], dA12f[3], dA13f[3];
-    float Alo[3];    // A - (double)Af: the amplitudes enter P as hi + lo
+    // A - (double)Af and the derivatives' likewise: they enter P as hi + lo
+    float Alo[3], dA12lo[3], dA13lo[3];
     float cmax;      // largest |c| of the point's phases (rounded up)
 };
 
@@ -42,6 +43,7 @@ struct BaseConst {
     float om[GNA_NLMAX];    // omega_r rounded to FP32
     float omlo[GNA_NLMAX];  // omega_r - om_r (FP32)
     float wkl[GNA_NLMAX];   // 2 omega_r K L_r: d sin^2 D / d dm2 = sin 2D K L / E
+    float wkllo[GNA_NLMAX]; // 2 omega_r K L_r - wkl_r
     double omd[GNA_NLMAX];  // omega_r (FP64)
     double kld[GNA_NLMAX];  // K L_r (FP64)
     double klmax;           // largest K L_r

@@ -140,8 +140,7 @@ struct GenSums {
 // Sums over the baselines: T, V weighted by omega_r, Y by omega_r K L_r, Z by
 // 2 omega_r K L_r.
 struct GenTaskSums {
-    float2 T[3], V[3];
-    float Y[3], Z[3];
+    float2 T[3], V[3], Y[3], Z[3];
 };
 
 template <bool GRAD>
@@ -151,8 +150,8 @@ __device__ __forceinline__ void store_gen_sums(const GenTaskSums& q, float2* pp)
         pp[j * 32] = q.T[j];
         pp[(3 + j) * 32] = q.V[j];
         if constexpr (GRAD) {
-            pp[(6 + j) * 32] = make_float2(q.Y[j], 0.f);
-            pp[(9 + j) * 32] = make_float2(q.Z[j], 0.f);
+            pp[(6 + j) * 32] = q.Y[j];
+            pp[(9 + j) * 32] = q.Z[j];
         }
     }
 }
@@ -169,11 +168,13 @@ __device__ __forceinline__ BinSums<GRAD ? 6 : 0> gen_bin_sums(const GenConst& c,
     }
     b.M = M;
     if constexpr (GRAD) {
-        float U[3], C[3];
+        float U[3], C[3], Y[3], Z[3];
 #pragma unroll
         for (int j = 0; j < 3; j++) {
             U[j] = 0.5f * (q.T[j].x + q.T[j].y);
             C[j] = 0.5f * (q.V[j].x + q.V[j].y);
+            Y[j] = q.Y[j].x + q.Y[j].y;
+            Z[j] = q.Z[j].x + q.Z[j].y;
         }
 #pragma unroll
         for (int p = 0; p < 4; p++) {
@@ -182,9 +183,9 @@ __device__ __forceinline__ BinSums<GRAD ? 6 : 0> gen_bin_sums(const GenConst& c,
             for (int j = 0; j < 3; j++) b.d[p] = fmaf(c.daf[p][j], U[j], fmaf(c.dbf[p][j], C[j], b.d[p]));
         }
         // pairs 0 = 21, 1 = 31, 2 = 32; x31 moves with both splittings
-        const float t31 = fmaf(c.af[1], q.Y[1], 0.5f * c.bf[1] * q.Z[1]);
-        b.d[4] = fmaf(c.af[0], q.Y[0], fmaf(0.5f * c.bf[0], q.Z[0], t31));
-        b.d[5] = fmaf(c.af[2], q.Y[2], fmaf(0.5f * c.bf[2], q.Z[2], t31));
+        const float t31 = fmaf(c.af[1], Y[1], 0.5f * c.bf[1] * Z[1]);
+        b.d[4] = fmaf(c.af[0], Y[0], fmaf(0.5f * c.bf[0], Z[0], t31));
+        b.d[5] = fmaf(c.af[2], Y[2], fmaf(0.5f * c.bf[2], Z[2], t31));
     }
     return b;
 }
@@ -322,8 +323,8 @@ __global__ void __maxnreg__(128) k_gen_one(GenArgs ga) {
             q.T[v] = g.T[v];
             q.V[v] = g.V[v];
             // omega = 1 for one baseline: wkl = 2 K L
-            q.Y[v] = 0.5f * a.bc.wkl[0] * __fsub_rn(g.Y[v].s, g.Y[v].c);
-            q.Z[v] = a.bc.wkl[0] * __fsub_rn(g.Z[v].s, g.Z[v].c);
+            q.Y[v] = ff_mul(0.5f * a.bc.wkl[0], 0.5f * a.bc.wkllo[0], kahan_to_ff(g.Y[v]));
+            q.Z[v] = ff_mul(a.bc.wkl[0], a.bc.wkllo[0], kahan_to_ff(g.Z[v]));
         }
         if (!whole) store_gen_sums<GRAD>(q, a.part + (int64_t)t * a.NVs * 32 + lane);
         else finish_gen_bins<GRAD>(ga, k.p, k.b, q, bin, lane);
@@ -458,8 +459,7 @@ __global__ void __maxnreg__(NP == 2 ? 168 : 128) k_gen_multi(GenArgs ga) {
         GenTaskSums q;
 #pragma unroll
         for (int j = 0; j < 3; j++) {
-            q.T[j] = q.V[j] = make_float2(0.f, 0.f);
-            q.Y[j] = q.Z[j] = 0.f;
+            q.T[j] = q.V[j] = q.Y[j] = q.Z[j] = make_float2(0.f, 0.f);
         }
         for (int r0 = 0; r0 < a.nL; r0 += 2 * NP) {
             M x;
@@ -536,8 +536,8 @@ __global__ void __maxnreg__(NP == 2 ? 168 : 128) k_gen_multi(GenArgs ga) {
                     q.T[j] = ff_add(q.T[j], ff_mul(a.bc.om[r], a.bc.omlo[r], g.T[j]));
                     q.V[j] = ff_add(q.V[j], ff_mul(a.bc.om[r], a.bc.omlo[r], g.V[j]));
                     if constexpr (GRAD) {
-                        q.Y[j] = fmaf(0.5f * a.bc.wkl[r], __fsub_rn(g.Y[j].s, g.Y[j].c), q.Y[j]);
-                        q.Z[j] = fmaf(a.bc.wkl[r], __fsub_rn(g.Z[j].s, g.Z[j].c), q.Z[j]);
+                        q.Y[j] = ff_add(q.Y[j], ff_mul(0.5f * a.bc.wkl[r], 0.5f * a.bc.wkllo[r], kahan_to_ff(g.Y[j])));
+                        q.Z[j] = ff_add(q.Z[j], ff_mul(a.bc.wkl[r], a.bc.wkllo[r], kahan_to_ff(g.Z[j])));
                     }
                 }
             }
@@ -566,8 +566,8 @@ __global__ void __launch_bounds__(W * 32) k_gen_slices_reduce(const float2* __re
         }
         if (ea.has_grad) {
             for (int j = 0; j < 3; j++) {
-                q.Y[j] = fin[(6 + j) * 32 + lane].x + fin[(6 + j) * 32 + lane].y;
-                q.Z[j] = fin[(9 + j) * 32 + lane].x + fin[(9 + j) * 32 + lane].y;
+                q.Y[j] = fin[(6 + j) * 32 + lane];
+                q.Z[j] = fin[(9 + j) * 32 + lane];
             }
             float2 regs[7];
             if (i < ea.nbins) bin_terms<6>(ea, p, i, gen_bin_sums<true>(gc[p], in.sumw, q), nullptr, in, regs);

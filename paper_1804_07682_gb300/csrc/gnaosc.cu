@@ -1049,7 +1049,7 @@ static gna_status plan_build(gna_plan* plan, const gna_plan_desc* d, cudaStream_
         bc.klmax = std::max(bc.klmax, bc.kld[r]);
         bc.om[r] = (float)plan->omega[r];
         bc.omlo[r] = (float)(plan->omega[r] - (double)bc.om[r]);
-        bc.wkl[r] = (float)(2.0 * plan->omega[r] * bc.kld[r]);
+        split_ff(2.0 * plan->omega[r] * bc.kld[r], bc.wkl[r], bc.wkllo[r]);
         fsum += (double)bc.om[r];  // exact: a handful of floats summed in double
     }
     bc.wsum = (float)fsum;

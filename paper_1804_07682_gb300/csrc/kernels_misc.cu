@@ -49,7 +49,8 @@ __global__ void k_prepare_points(const gna_osc* __restrict__ prm, int npts, Base
     const double c12 = 1.0 - s12, c13 = 1.0 - s13, m12 = 1.0 - 2.0 * s12, m13 = 1.0 - 2.0 * s13;
     double k0, f0, f1, f2 = 1.0, f3 = 1.0;
     static_assert(offsetof(PointConst, dA13) == offsetof(PointConst, A) + 6 * sizeof(double) &&
-                      offsetof(PointConst, dA13f) == offsetof(PointConst, Af) + 6 * sizeof(float),
+                      offsetof(PointConst, dA13f) == offsetof(PointConst, Af) + 6 * sizeof(float) &&
+                      offsetof(PointConst, dA13lo) == offsetof(PointConst, Alo) + 6 * sizeof(float),
                   "A, dA12, dA13 in a row, and so their FP32 copies");
     switch (r) {
         case 0: k0 = 4.0, f0 = s12, f1 = c12, f2 = c13, f3 = c13; break;   // A21
@@ -68,8 +69,8 @@ __global__ void k_prepare_points(const gna_osc* __restrict__ prm, int npts, Base
         char* const base = reinterpret_cast<char*>(&pc);
         *reinterpret_cast<double*>(base + offsetof(PointConst, A) + r * sizeof(double)) = a;
         *reinterpret_cast<float*>(base + offsetof(PointConst, Af) + r * sizeof(float)) = af;
+        *reinterpret_cast<float*>(base + offsetof(PointConst, Alo) + r * sizeof(float)) = alo;
     }
-    if (r < 3) pc.Alo[r] = alo;
     if (r == 0) {
         pc.cmax = largest_phase(bc, o.dm2_21, o.dm2_32);
         // the parameters live on the device: a point outside the physical domain

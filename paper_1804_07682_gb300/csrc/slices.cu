@@ -32,7 +32,7 @@ __global__ void __launch_bounds__(W * 32) k_slices_reduce(const float2* __restri
         const int from = ea.has_grad ? 6 : 3;
         for (int r = 0; r < ea.nspec; r++) sp[r] = fin[(from + r) * 32 + lane];
         if (ea.has_grad) {
-            for (int j = 0; j < 3; j++) q.N[j] = fin[(3 + j) * 32 + lane].x + fin[(3 + j) * 32 + lane].y;
+            for (int j = 0; j < 3; j++) q.N[j] = fin[(3 + j) * 32 + lane];
             float2 regs[5];
             if (i < ea.nbins) bin_terms<4>(ea, p, i, bin_sums<true>(pcs + p, in.sumw, q), sp, in, regs);
             group_done_terms<4>(ea, p, g, lane, regs);

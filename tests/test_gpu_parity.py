@@ -1363,3 +1363,54 @@ def test_normalisations_of_any_size(api, prec, channel, mapping, norm, top):
     a_float = (ref[0] * norm > 1e-37) & (ref[0] * norm < 1e38) & (ref[0] > 1e-37)
     for a, b, ok in zip(got, ref, (np.ones(40, bool), a_float)):
         assert (np.abs(a / norm - b) <= 2e-6 * np.abs(b) + 4 * low)[ok].all(), (a / norm, b)
+
+
+def derivative_errors(api, e, L, n, prec, channel=None, e_scale=1.0, seed=1):
+    """rms over 64 points of the errors of mu and of its derivatives by the
+    parameters, one bin, in units of their own rms: Pearson's chi^2 of no
+    counts is mu, so its gradient is d mu.  Against GNA_FP64."""
+    rng = np.random.default_rng(seed)
+    th = np.array(THETA_FULL) * (1 + rng.uniform(-0.05, 0.05, (64, 6)))
+    if channel is None:
+        th = th[:, [0, 1, 4, 5]]
+    out = []
+    for p in (prec, "fp64"):
+        plan = api.Plan(e, L, nodes_per_bin=n, npts=64, prec=p, kind="pearson", channel=channel, e_scale=e_scale)
+        o = (plan.eval if channel is None else plan.eval_general)(plan.params_tensor(th), dev(np.zeros(1)), grad=True, mu=True)
+        out.append(np.concatenate([o["mu"].cpu().numpy(), o["grad"].cpu().numpy()], axis=1))
+        plan.close()
+    a, b = out
+    return np.sqrt(((a - b) ** 2).mean(axis=0) / (b ** 2).mean(axis=0))
+
+
+def s12_cancellation(e, L, seed=1):
+    """Over derivative_errors' points: rms of the absolute terms of d mu / d
+    s2_12 over rms of their sum (survival chain, one bin)."""
+    rng = np.random.default_rng(seed)
+    th = np.array(THETA_FULL) * (1 + rng.uniform(-0.05, 0.05, (64, 6)))
+    s12, s13, d21, d32 = (th[:, k, None] for k in (0, 1, 4, 5))
+    x, w = np.polynomial.legendre.leggauss(64)
+    E = 0.5 * (e[0] + e[1]) + 0.5 * (e[1] - e[0]) * x
+    w = w * np.exp(0.87 - 0.16 * E - 0.091 * E * E)
+    om = oracle.baseline_weights(np.array(L))
+    S = [sum(o * (w * np.sin(1266.932679419849 * d * Lr / E) ** 2).sum(axis=1) for o, Lr in zip(om, L))
+         for d in (d21, d21 + d32, d32)]
+    s12, c13, s13 = s12[:, 0], 1 - s13[:, 0], s13[:, 0]
+    t = 4 * np.array([(1 - 2 * s12) * c13 ** 2 * S[0], -c13 * s13 * S[1], c13 * s13 * S[2]])
+    return np.sqrt((np.abs(t).sum(axis=0) ** 2).mean() / (t.sum(axis=0) ** 2).mean())
+
+
+@pytest.mark.parametrize("prec", ["f64phase", "ff"])
+@pytest.mark.parametrize("n", [50, 262, 1000])
+@pytest.mark.parametrize("nL", [1, 8])
+def test_derivatives_are_contracted_in_pairs(api, nL, n, prec):
+    """The derivative by s2_12 takes two pairs' sums with opposite signs: it is
+    formed from float pairs, as the prediction.  Four FP32 roundings of the
+    result (2^-25 each, rms: 6e-8; 9e-8 allowed), and of the terms the sums'
+    own errors: below 1e-8 each (the terms in FP32 would add 2.5e-8)."""
+    L = [23.2, 11.4, 44.9, 18.3, 45.1, 0.9, 22.2, 19.3][:nL]
+    for lo, w in ((3.004, 0.4028), (7.265, 0.0145), (9.77, 0.4028)):
+        e = np.array([lo, lo + w])
+        mu, s12, s13, dm21, _ = derivative_errors(api, e, L, n, prec)
+        k = s12_cancellation(e, L)
+        assert mu < 5e-8 and s12 < 9e-8 + 1e-8 * k and s13 < 9e-8 and dm21 < 9e-8, (lo, k, mu, s12, s13, dm21)
