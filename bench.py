@@ -39,11 +39,11 @@ SM_COUNT, FP32_LANES, SM_MAX_MHZ = 152, 128, 2070.0
 def fp32_ops_general(nL: int, grad: bool) -> int:
     """Algorithmic FP32 operations (FMA = 1) per energy node of the any-channel
     chain's chunk-anchored node kernels: per (node, baseline) two phases by one
-    FMA each from the chunk's anchor 2, sin and cos - 1 of both 20, the third
-    pair by the addition formulas 6, weighted sums 6 (12 with the gradient);
+    FMA each from the chunk's anchor 2, sin and cos - 1 of both 20, what the
+    third pair has beyond them 4, weighted sums 6 (12 with the gradient);
     per node the offset of 1/E 3, W/E 1, the sum of W 4 and of W/E 1 (with the
     gradient).  Anchors and the additions of a chunk's sums are not counted."""
-    return nL * (40 if grad else 34) + 8 + (1 if grad else 0)
+    return nL * (38 if grad else 32) + 8 + (1 if grad else 0)
 
 
 def fp32_ops_per_node(nL: int, grad: bool, spec: bool) -> int:

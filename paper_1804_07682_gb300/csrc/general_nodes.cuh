@@ -18,8 +18,17 @@
 // where H = sum W h, S = sum W s, C = sum W: the large part is C, summed with
 // compensation, and the rest carries an error relative to itself.
 //
+// The CP terms cancel further: b_21 = b_32 = -b_31, and V_21 + V_32 - V_31 is a
+// product of three sines.  So of the third pair a node adds only what
+// s_31 = s_21 + s_32 + (s_21 h_32 + h_21 s_32) and
+// h_31 = h_21 + h_32 + (h_21 h_32 - s_21 s_32) have beyond the other two, and
+// a chunk's sums S, H of pair 31 are put together from the three in float
+// pairs: the roundings of S_21 and S_32 drop out (P(e -> tau), 5.8 MeV at 4.2
+// GeV, 810 and 295 km: 8.2e-8 of the prediction with s_31 summed by itself,
+// 1.1e-8 so).
+//
 // What bounds it: the FP32 pipe.  Operations per (node, baseline), gradient
-// on: phases 2, sines and cosines 20, addition 6, sums 12 = 40 (reducing each
+// on: phases 2, sines and cosines 20, addition 4, sums 12 = 38 (reducing each
 // node's phases, with sin^2, cos^2 and sin cos of three phases: 120-150).
 #pragma once
 
@@ -51,6 +60,18 @@ __device__ __forceinline__ void sinhq2(const f32x2 (&r)[N], f32x2 (&s)[N], f32x2
     GNA_STEP(h[i] = mul2(c[i], u[i]))
     GNA_STEP(s[i] = fma2(s[i], p[i], r[i]))
 #undef GNA_STEP
+}
+
+// What sin and cos - 1 of r1 + r2 have beyond those of r1 and r2.
+__device__ __forceinline__ void angle_rest2(f32x2 s1, f32x2 h1, f32x2 s2, f32x2 h2, f32x2& s, f32x2& h) {
+    s = fma2(h1, s2, mul2(s1, h2));
+    h = fma2(neg2(s1), s2, mul2(h1, h2));
+}
+
+// a + b + c as a float pair.
+__device__ __forceinline__ float2 sum3(float a, float b, float c) {
+    const float2 s = ff_add(make_float2(a, 0.f), make_float2(b, 0.f));
+    return ff_add(s, make_float2(c, 0.f));
 }
 
 // Doubled phase of baseline r's pair 21 or 32 modulo pi/2, and the quadrant
@@ -86,16 +107,16 @@ struct QuadrantSums {
     float2 T, V;  // {big, part} with the pair's low part of C apart
     float Tl, Vl;
 };
-__device__ __forceinline__ QuadrantSums quadrant_sums(unsigned q, float S, float H, float2 c) {
+__device__ __forceinline__ QuadrantSums quadrant_sums(unsigned q, float2 S, float2 H, float2 c) {
     QuadrantSums r;
     const bool odd = q & 1u;
     const float k = odd ? 1.0f : (q & 2u) ? 2.0f : 0.0f;
     const float st = ((q + 1u) & 2u) ? 1.0f : -1.0f;  // T: -H, +S, +H, -S
     const float sv = (q & 2u) ? -1.0f : 1.0f;         // V: S, C + H, -S, -(C + H)
-    r.T = make_float2(k * c.x, st * (odd ? S : H));
-    r.Tl = k * c.y;
-    r.V = make_float2(odd ? sv * c.x : 0.f, sv * (odd ? H : S));
-    r.Vl = odd ? sv * c.y : 0.f;
+    r.T = make_float2(k * c.x, st * (odd ? S.x : H.x));
+    r.Tl = fmaf(k, c.y, st * (odd ? S.y : H.y));
+    r.V = make_float2(odd ? sv * c.x : 0.f, sv * (odd ? H.x : S.x));
+    r.Vl = sv * (odd ? c.y + H.y : S.y);
     return r;
 }
 __device__ __forceinline__ float quadrant_Y(unsigned q, float SE, float HE, float e) {
@@ -125,8 +146,16 @@ struct GenSums {
             kzero(Z[j]);
         }
     }
+    // a chunk's sums of the three pairs, [1] the third's beyond the other two; q21, q32: quadrants
+    __device__ __forceinline__ void add(unsigned q21, unsigned q32, const float (&S)[3], const float (&H)[3],
+                                        const float (&SE)[3], const float (&HE)[3], float2 c, float e) {
+        add(0, q21, make_float2(S[0], 0.f), make_float2(H[0], 0.f), SE[0], HE[0], c, e);
+        add(1, (q21 + q32) & 3u, sum3(S[0], S[2], S[1]), sum3(H[0], H[2], H[1]), SE[0] + SE[2] + SE[1],
+            HE[0] + HE[2] + HE[1], c, e);
+        add(2, q32, make_float2(S[2], 0.f), make_float2(H[2], 0.f), SE[2], HE[2], c, e);
+    }
     // a chunk's sums of pair j
-    __device__ __forceinline__ void add(int j, unsigned q, float S, float H, float SE, float HE, float2 c, float e) {
+    __device__ __forceinline__ void add(int j, unsigned q, float2 S, float2 H, float SE, float HE, float2 c, float e) {
         const QuadrantSums r = quadrant_sums(q, S, H, c);
         T[j] = ff_add(T[j], big_sum(r.T, r.Tl));
         V[j] = ff_add(V[j], big_sum(r.V, r.Vl));
@@ -208,12 +237,11 @@ __device__ __forceinline__ void gen_single(const PointConst* pc, int r, float eh
     const f32x2 y[1] = {pack2(phase_q<PH>(pc, r, false, eh, el, q21), phase_q<PH>(pc, r, true, eh, el, q32))};
     f32x2 s[1], h[1], s3, h3;
     sinhq2(y, s, h);
-    angle_add2<true>(dup2(s[0].x), dup2(h[0].x), dup2(s[0].y), dup2(h[0].y), s3, h3);
+    angle_rest2(dup2(s[0].x), dup2(h[0].x), dup2(s[0].y), dup2(h[0].y), s3, h3);
     const float We = W * eh;
-    const float2 c = make_float2(W, 0.f);
-    g.add(0, q21, W * s[0].x, W * h[0].x, We * s[0].x, We * h[0].x, c, We);
-    g.add(1, (q21 + q32) & 3u, W * s3.x, W * h3.x, We * s3.x, We * h3.x, c, We);
-    g.add(2, q32, W * s[0].y, W * h[0].y, We * s[0].y, We * h[0].y, c, We);
+    const float S[3] = {W * s[0].x, W * s3.x, W * s[0].y}, H[3] = {W * h[0].x, W * h3.x, W * h[0].y};
+    const float SE[3] = {We * s[0].x, We * s3.x, We * s[0].y}, HE[3] = {We * h[0].x, We * h3.x, We * h[0].y};
+    g.add(q21, q32, S, H, SE, HE, make_float2(W, 0.f), We);
 }
 
 // ---------------------------------------------------- one baseline -------
@@ -231,7 +259,7 @@ struct GenOneMath {
         const f32x2 r[2] = {fma2(c21, d, a21), fma2(c32, d, a32)};
         f32x2 s[2], h[2], s3, h3;
         sinhq2(r, s, h);
-        angle_add2<true>(s[0], h[0], s[1], h[1], s3, h3);
+        angle_rest2(s[0], h[0], s[1], h[1], s3, h3);
         H[0] = fma2(n.w, h[0], H[0]);
         H[1] = fma2(n.w, h3, H[1]);
         H[2] = fma2(n.w, h[1], H[2]);
@@ -301,11 +329,15 @@ __global__ void __maxnreg__(128) k_gen_one(GenArgs ga) {
                 }
                 const float2 c = w.total();
                 const float es = e.x + e.y;
-                const unsigned q[3] = {q21, (q21 + q32) & 3u, q32};
+                float S[3], H[3], SE[3], HE[3];
 #pragma unroll
-                for (int v = 0; v < 3; v++)
-                    g.add(v, q[v], x.S[v].x + x.S[v].y, x.H[v].x + x.H[v].y, x.SE[v].x + x.SE[v].y,
-                          x.HE[v].x + x.HE[v].y, c, es);
+                for (int v = 0; v < 3; v++) {
+                    S[v] = x.S[v].x + x.S[v].y;
+                    H[v] = x.H[v].x + x.H[v].y;
+                    SE[v] = x.SE[v].x + x.SE[v].y;
+                    HE[v] = x.HE[v].x + x.HE[v].y;
+                }
+                g.add(q21, q32, S, H, SE, HE, c, es);
                 x.zero();
             } else {
                 in.wait();
@@ -380,7 +412,7 @@ struct GenMultiMath {
 #pragma unroll
         for (int i = 0; i < NP; i++) {
             f32x2 s3, h3;
-            angle_add2<true>(s[2 * i], h[2 * i], s[2 * i + 1], h[2 * i + 1], s3, h3);
+            angle_rest2(s[2 * i], h[2 * i], s[2 * i + 1], h[2 * i + 1], s3, h3);
             const f32x2 sj[3] = {s[2 * i], s3, s[2 * i + 1]}, hj[3] = {h[2 * i], h3, h[2 * i + 1]};
 #pragma unroll
             for (int j = 0; j < 3; j++) {
@@ -498,14 +530,18 @@ __global__ void __maxnreg__(NP == 2 ? 168 : 128) k_gen_multi(GenArgs ga) {
 #pragma unroll
                         for (int half = 0; half < 2; half++) {
                             const unsigned b = quads >> (8 * i + 4 * half), q21 = b & 3u, q32 = (b >> 2) & 3u;
-                            const unsigned qj[3] = {q21, (q21 + q32) & 3u, q32};
                             GenSums<GRAD> g;
                             if (ka == 0) g.zero();
                             else g = load_gen<NS, GRAD>(comp, stride, i, half);
+                            float S[3], H[3], SE[3], HE[3];
 #pragma unroll
-                            for (int j = 0; j < 3; j++)
-                                g.add(j, qj[j], half ? x.S[i][j].y : x.S[i][j].x, half ? x.H[i][j].y : x.H[i][j].x,
-                                      half ? x.SE[i][j].y : x.SE[i][j].x, half ? x.HE[i][j].y : x.HE[i][j].x, c, es);
+                            for (int j = 0; j < 3; j++) {
+                                S[j] = half ? x.S[i][j].y : x.S[i][j].x;
+                                H[j] = half ? x.H[i][j].y : x.H[i][j].x;
+                                SE[j] = half ? x.SE[i][j].y : x.SE[i][j].x;
+                                HE[j] = half ? x.HE[i][j].y : x.HE[i][j].x;
+                            }
+                            g.add(q21, q32, S, H, SE, HE, c, es);
                             save_gen<NS, GRAD>(comp, stride, i, half, g);
                         }
                     x.zero();

@@ -1414,3 +1414,16 @@ def test_derivatives_are_contracted_in_pairs(api, nL, n, prec):
         mu, s12, s13, dm21, _ = derivative_errors(api, e, L, n, prec)
         k = s12_cancellation(e, L)
         assert mu < 5e-8 and s12 < 9e-8 + 1e-8 * k and s13 < 9e-8 and dm21 < 9e-8, (lo, k, mu, s12, s13, dm21)
+
+
+@pytest.mark.parametrize("prec", ["f64phase", "ff"])
+@pytest.mark.parametrize("n", [8, 100, 1000])
+@pytest.mark.parametrize("channel", [("e", "tau", False), ("mu", "e", True)])
+def test_cp_terms_cancel_exactly(api, channel, n, prec):
+    """At short baselines the three CP terms sin y_21 + sin y_32 - sin y_31 of
+    an appearance channel are fifteen times what is left of them: roundings of
+    the single sums (2^-24 of each, 8e-8 of mu and more) must not remain.  What
+    remains is that of T and of what pair 31 has beyond the others, 2^-25."""
+    for lo, w in ((4167.0, 5.8), (3345.0, 5.8), (2426.0, 22.5)):
+        mu = derivative_errors(api, np.array([lo, lo + w]), [810.0, 295.0], n, prec, channel, 1e-3)[0]
+        assert mu < (3e-8 if n >= 100 else 6e-8), (lo, mu)  # few nodes: their own roundings do not average
