@@ -53,7 +53,7 @@ typedef enum {
     GNA_OK = 0,
     GNA_EINVAL = 1,   /* bad argument value or NULL pointer */
     GNA_ESHAPE = 2,   /* sizes inconsistent with the plan or out of range */
-    GNA_ENOMEM = 3,   /* device or pinned-host allocation failed (plan creation only) */
+    GNA_ENOMEM = 3,   /* device or pinned-host allocation failed (plan creation, first fit) */
     GNA_ECUDA = 4,    /* a CUDA runtime call failed */
     GNA_ETIMEOUT = 5, /* reserved: no call waits on a device flag */
     GNA_ESTATE = 6    /* call not valid in the plan's current state */
@@ -91,7 +91,8 @@ typedef struct {
     double e_scale;             /* spectrum S(E * e_scale): 1 for MeV, 1e-3 for GeV */
     gna_precision prec;
     gna_chi2_kind kind;
-    int max_datasets;           /* >= npts when each point has its own data row (fits); 0 = npts */
+    int max_datasets;           /* >= npts when each point has its own data row (fits); 0 = npts, and what
+                                   only fits need (16 bytes per node, mixed precisions) waits for the first */
     int flags;                  /* GNA_PLAN_* bits below */
     int alpha, beta;            /* with GNA_PLAN_GENERAL: the channel P(alpha -> beta), 0 = e, 1 = mu, 2 = tau */
     int anti;                   /* with GNA_PLAN_GENERAL: 1 for antineutrinos, 0 for neutrinos */
@@ -397,7 +398,10 @@ gna_status gna_chain_eval_plain(gna_plan* plan, const gna_osc* params, const dou
  *   chi2_out: device [npts] best chi^2
  *   lambda0: initial damping (e.g. 1e-3)
  * With use_graph != 0 one iteration is captured once into a CUDA graph and
- * replayed `iters` times.  Asynchronous on `stream`.
+ * replayed `iters` times.  Asynchronous on `stream`, but for the first fit of
+ * a mixed-precision plan created with max_datasets = 0: it allocates and
+ * builds the fits' node layout on a stream of the plan's and waits for it
+ * (also while `stream` is being captured); GNA_ENOMEM if there is no room.
  */
 gna_status gna_fit_batch(gna_plan* plan, gna_osc* params, const double* data, int iters, double lambda0,
                          double* chi2_out, int use_graph, void* stream);

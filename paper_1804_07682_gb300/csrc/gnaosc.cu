@@ -117,7 +117,7 @@ struct gna_plan {
     // autotuner can choose the mapping
     bool has_split = false, has_bins = false;
     float4* grid_split = nullptr;
-    float4* grid_bins = nullptr;
+    float4* grid_bins = nullptr;  // the fits' (bin and slice mappings): built by the first fit, or with the plan
     // quads of nodes for the anchored kernels (survival chain, mixed precisions,
     // bin and slice mappings), and their whole-bin tasks
     char* grid_rec = nullptr;
@@ -130,6 +130,8 @@ struct gna_plan {
     int* d_gn = nullptr;
     int* d_gid = nullptr;  // [npts] grid of each point (NULL: one grid for all)
     int ngrids = 0, ngroups = 0;
+    std::vector<int> gn;                    // orders of the grids
+    std::vector<const double*> gl_x, gl_w;  // their Gauss-Legendre rules (device)
     int* d_tasks = nullptr;
     int ntasks = 0;
     float* d_step = nullptr;  // [ngrids][ngroups] largest step of 1/E between neighbouring nodes
@@ -1000,6 +1002,27 @@ gna_status gna_plan_info(const gna_plan* plan, int64_t* nodes, int64_t* points, 
     return GNA_OK;
 }
 
+// The node layout of the mixed fits' bin and slice mappings (16 bytes a node
+// beside the evaluations' 12): with the plan where it announces data sets of
+// its own for its points, else by the first fit.
+static gna_status build_fit_grid(gna_plan* plan, cudaStream_t s) {
+    if (plan->ph == 2 || !plan->has_bins || plan->grid_bins) return GNA_OK;
+    const int nbins_pad = plan->ngroups * 32;
+    int64_t len = 0;
+    for (int n : plan->gn) len += (int64_t)nbins_pad * n;
+    float4* grid = nullptr;
+    TRY(dalloc(plan, &grid, len));
+    int64_t off = 0;
+    for (int g = 0; g < plan->ngrids; g++) {
+        CU(launch_build_grid(plan->nbins, nbins_pad, plan->d_edges, plan->gn[g], plan->gl_x[g], plan->gl_w[g], plan->e_scale,
+                             1, grid + off, nullptr, nullptr, nullptr, s));
+        off += (int64_t)nbins_pad * plan->gn[g];
+    }
+    CU(cudaStreamSynchronize(s));
+    plan->grid_bins = grid;
+    return GNA_OK;
+}
+
 static gna_status plan_build(gna_plan* plan, const gna_plan_desc* d, cudaStream_t s) {
     int dev = 0;
     CU(cudaGetDevice(&dev));
@@ -1099,6 +1122,7 @@ static gna_status plan_build(gna_plan* plan, const gna_plan_desc* d, cudaStream_
     std::vector<int> gn(plan->counts.begin(), plan->counts.end());
     std::sort(gn.begin(), gn.end());
     gn.erase(std::unique(gn.begin(), gn.end()), gn.end());
+    plan->gn = gn;
     plan->ngrids = (int)gn.size();
     std::vector<int> gid(d->npts);
     for (int p = 0; p < d->npts; p++)
@@ -1134,7 +1158,6 @@ static gna_status plan_build(gna_plan* plan, const gna_plan_desc* d, cudaStream_
         if (want64) TRY(dalloc(plan, &plan->grid64_split, len_split));
     }
     if (plan->has_bins) {
-        if (plan->ph < 2) TRY(dalloc(plan, &plan->grid_bins, len_bins));
         if (quads) TRY(dalloc(plan, &plan->grid_rec, nquads * kQuadBytes));
         if (want64) TRY(dalloc(plan, &plan->grid64_bins, len_bins));
     }
@@ -1166,24 +1189,22 @@ static gna_status plan_build(gna_plan* plan, const gna_plan_desc* d, cudaStream_
     TRY(dalloc(plan, &glx, gl_total));
     TRY(dalloc(plan, &glw, gl_total));
     TRY(dalloc(plan, &tmp, 2 * (size_t)orders.back()));
-    std::map<int, int64_t> gl_off;
     int64_t go = 0;
-    for (int n : orders) {
-        gl_off[n] = go;
+    for (int n : orders) {  // (the orders are the grids')
+        plan->gl_x.push_back(glx + go);
+        plan->gl_w.push_back(glw + go);
         CU(launch_gl(n, glx + go, glw + go, tmp, s));
         go += n;
     }
     // energy grids
     if (plan->has_split) {
-        const int n = plan->n_uniform;
-        CU(launch_build_grid(d->nbins, d->nbins, plan->d_edges, n, glx + gl_off[n], glw + gl_off[n], plan->e_scale, 0,
+        CU(launch_build_grid(d->nbins, d->nbins, plan->d_edges, gn[0], plan->gl_x[0], plan->gl_w[0], plan->e_scale, 0,
                              plan->grid_split, nullptr, plan->grid64_split, plan->plain64, s));
     }
     if (plan->has_bins)
         for (int g = 0; g < plan->ngrids; g++) {
-            const int n = gn[g];
-            CU(launch_build_grid(d->nbins, nbins_pad, plan->d_edges, n, glx + gl_off[n], glw + gl_off[n],
-                                 plan->e_scale, 1, plan->grid_bins ? plan->grid_bins + goff[g] : nullptr,
+            CU(launch_build_grid(d->nbins, nbins_pad, plan->d_edges, gn[g], plan->gl_x[g], plan->gl_w[g],
+                                 plan->e_scale, 1, nullptr,
                                  quads ? plan->grid_rec + qoff[g] * kQuadBytes : nullptr,
                                  plan->grid64_bins ? plan->grid64_bins + goff[g] : nullptr,
                                  (plan->plain64 && !plan->has_split) ? plan->plain64 + plain_goff[g] : nullptr, s));
@@ -1195,8 +1216,8 @@ static gna_status plan_build(gna_plan* plan, const gna_plan_desc* d, cudaStream_
         for (int g = 0; g < plan->ngrids; g++) {
             double* sw = plan->d_sumW + (size_t)g * d->nbins;
             float2* swf = plan->d_sumWf + (size_t)g * d->nbins;
-            if (plan->has_split) CU(launch_sum_weights(plan->grid_split, d->nbins, gn[g], 0, sw, swf, s));
-            else CU(launch_sum_weights(plan->grid_bins + goff[g], d->nbins, gn[g], 1, sw, swf, s));
+            if (plan->has_split) CU(launch_sum_weights(plan->grid_split, nullptr, d->nbins, gn[g], sw, swf, s));
+            else CU(launch_sum_weights(nullptr, plan->grid_rec + qoff[g] * kQuadBytes, d->nbins, gn[g], sw, swf, s));
         }
     }
     std::vector<float> step;  // (copied from below: lives until the stream is synchronised)
@@ -1333,6 +1354,7 @@ static gna_status plan_build(gna_plan* plan, const gna_plan_desc* d, cudaStream_
         TRY(dalloc(plan, &plan->d_plainMu, (size_t)max_cnt * d->nL * d->nbins));
         TRY(dalloc(plan, &plan->d_plainDmu, 4 * (size_t)max_cnt * d->nL * d->nbins));
     }
+    if (d->max_datasets > 0) TRY(build_fit_grid(plan, s));
     CU(cudaStreamSynchronize(s));
     CU(cudaGetLastError());
     plan->last_stream = s;
@@ -1707,6 +1729,14 @@ gna_status fit_impl(gna_plan* plan, double* params, const double* data, int iter
     if (!params || !data || !chi2_out) return fail(plan, GNA_EINVAL, "params, data and chi2_out are required");
     if (iters < 1) return fail(plan, GNA_EINVAL, "iters must be >= 1");
     if (plan->max_datasets < plan->npts) return fail(plan, GNA_ESHAPE, "fits need one data row per point");
+    if (plan->mapping != MAP_SPLIT && !plan->grid_bins) {
+        // on a stream of the plan's own, allowed while the caller's is being captured
+        cudaStreamCaptureMode mode = cudaStreamCaptureModeRelaxed;
+        CU(cudaThreadExchangeStreamCaptureMode(&mode));
+        const gna_status st = build_fit_grid(plan, plan->cap_stream);
+        CU(cudaThreadExchangeStreamCaptureMode(&mode));
+        if (st != GNA_OK) return st;
+    }
     plan->last_stream = s;
     CU(launch_lm_init<NP>(lm, plan->npts, lambda0, s));
     EvalReq q{NP == 4 ? (const gna_osc*)params : nullptr, nullptr, 0.0, data, 1, plan->d_chi2_tmp, plan->d_grad_tmp,

@@ -204,17 +204,17 @@ __global__ void k_build_grid(int nbins, int nbins_pad, const double* __restrict_
 
 // Sum of the FP32 node weights of each bin, in double (for the epilogue's
 // exact correction of the constant term): one warp per bin, lane l takes
-// nodes l, l + 32, ... (coalesced in layout 0), then a fixed-order butterfly.
-__global__ void k_sum_weights(const float4* __restrict__ grid, int nbins, int n, int layout, double* __restrict__ out,
-                              float2* __restrict__ outf) {
+// nodes l, l + 32, ..., then a fixed-order butterfly.  The nodes bin-major
+// (grid), or else in quads (rec).
+__global__ void k_sum_weights(const float4* __restrict__ grid, const char* __restrict__ rec, int nbins, int n,
+                              double* __restrict__ out, float2* __restrict__ outf) {
     const int i = (int)(((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5);
     const int lane = threadIdx.x & 31;
     if (i >= nbins) return;
     double s = 0.0;
-    for (int k = lane; k < n; k += 32) {
-        const int64_t pos = (layout == 0) ? (int64_t)i * n + k : (((int64_t)(i >> 5) * n + k) * 32 + (i & 31));
-        s += (double)grid[pos].z;
-    }
+    const float* w = reinterpret_cast<const float*>(rec + (int64_t)(i >> 5) * ((n + 3) >> 2) * (3 * 512)) + 128 + (i & 31) * 4;
+    for (int k = lane; k < n; k += 32)
+        s += (double)(grid ? grid[(int64_t)i * n + k].z : w[(int64_t)(k >> 2) * (3 * 128) + (k & 3)]);
 #pragma unroll
     for (int o = 16; o >= 1; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
     if (lane == 0) {
@@ -223,9 +223,9 @@ __global__ void k_sum_weights(const float4* __restrict__ grid, int nbins, int n,
     }
 }
 
-cudaError_t launch_sum_weights(const float4* grid, int nbins, int n, int layout, double* out, float2* outf,
+cudaError_t launch_sum_weights(const float4* grid, const char* rec, int nbins, int n, double* out, float2* outf,
                                cudaStream_t s) {
-    k_sum_weights<<<(unsigned)(((int64_t)nbins * 32 + 255) / 256), 256, 0, s>>>(grid, nbins, n, layout, out, outf);
+    k_sum_weights<<<(unsigned)(((int64_t)nbins * 32 + 255) / 256), 256, 0, s>>>(grid, rec, nbins, n, out, outf);
     return cudaGetLastError();
 }
 

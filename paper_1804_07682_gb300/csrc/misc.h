@@ -65,7 +65,7 @@ cudaError_t launch_gl(int n, double* x, double* w, double* tmp_ab, cudaStream_t 
 cudaError_t launch_build_grid(int nbins, int nbins_pad, const double* edges, int n, const double* x, const double* w,
                               double e_scale, int layout, float4* ff, char* rec, double2* d64, double2* plain64,
                               cudaStream_t s);
-cudaError_t launch_sum_weights(const float4* grid, int nbins, int n, int layout, double* out, float2* outf,
+cudaError_t launch_sum_weights(const float4* grid, const char* rec, int nbins, int n, double* out, float2* outf,
                                cudaStream_t s);
 // The plain chain's kernels for one chunk of points: OscProb (+ tangents),
 // weights, bin integration, chi^2 (4 launches, 6 with the tangents).

@@ -1427,3 +1427,37 @@ def test_cp_terms_cancel_exactly(api, channel, n, prec):
     for lo, w in ((4167.0, 5.8), (3345.0, 5.8), (2426.0, 22.5)):
         mu = derivative_errors(api, np.array([lo, lo + w]), [810.0, 295.0], n, prec, channel, 1e-3)[0]
         assert mu < (3e-8 if n >= 100 else 6e-8), (lo, mu)  # few nodes: their own roundings do not average
+
+
+@pytest.mark.parametrize("channel", [None, ("mu", "mu", False)])
+def test_fit_layout_waits_for_the_first_fit(api, channel):
+    """A plan that announces no data sets of its own holds 12 bytes per node
+    until it is fitted (the mixed precisions' evaluations read no more), and its
+    fits, captured into a graph too, equal those of a plan that announces them."""
+    e, L, counts = np.linspace(1.8, 8.0, 33), [52.5], [40001, 40004]
+    th = np.array([0.307, 0.0218, 7.53e-5, 2.44e-3] if channel is None else THETA_FULL)
+    start = np.repeat(th[None] * 1.01, 2, 0)
+    bytes_, res = {}, {}
+    for m in (0, 2):
+        plan = api.Plan(e, L, npts=2, node_counts=counts, prec="ff", kind="poisson", norm=1e4, max_datasets=m, channel=channel)
+        f = plan.eval if channel is None else plan.eval_general
+        data = f(plan.params_tensor(np.repeat(th[None], 2, 0)), dev(np.ones(32)), mu=True)["mu"].clone()
+        bytes_[m] = plan.info()["device_bytes"]
+        p, c = plan.params_tensor(start), torch.empty(2, dtype=torch.float64, device="cuda")
+        if m:
+            plan.fit(p, data, iters=3, chi2_out=c)
+        else:
+            p0 = p.clone()
+            graph = torch.cuda.CUDAGraph()
+            with torch.cuda.graph(graph):
+                p.copy_(p0)
+                plan.fit(p, data, iters=3, chi2_out=c, graph=False)
+            graph.replay()
+        res[m] = p.cpu().numpy(), c.cpu().numpy()
+        assert plan.info()["device_bytes"] == bytes_[2] if m else plan.info()["device_bytes"] > bytes_[0]
+        plan.status()
+        plan.close()
+    nodes = 32 * sum(counts)
+    assert bytes_[0] < 12.1 * nodes + 4e6 and bytes_[2] - bytes_[0] == 16 * nodes
+    for a, b in zip(res[0], res[2]):
+        assert np.array_equal(a, b)
