@@ -327,32 +327,10 @@ __device__ __forceinline__ float2 ff_norm(float p, float e) {
     return make_float2(h, __fsub_rn(e, __fsub_rn(h, p)));
 }
 
-// mu = f M and the bin's term outside the pairs' range (a normalisation that
-// is no float, a prediction next to the smallest ones): with mu and d - mu in
-// double, as bin_epilogue.  Out of line: the node loops keep their registers.
-struct WideTerm {
-    double mu;
-    float2 term;
-    float g;
-};
-static __device__ __noinline__ WideTerm wide_term(double f, double M, double d, int kind) {
-    WideTerm w;
-    w.mu = f * M;
-    const double dm = d - w.mu;
-    const float tf = (float)dm / (float)w.mu;
-    double term;
-    if (kind == GNA_PEARSON) {
-        term = dm * (double)tf;
-        w.g = 1.0f - (1.0f + tf) * (1.0f + tf);
-    } else {
-        term = d > 0.0 ? 2.0 * w.mu * (double)poisson_h(tf) : 2.0 * w.mu;
-        w.g = -2.0f * tf;
-    }
-    w.term = to_ff(term);
-    return w;
-}
 // The pairs hold a product f M and its low parts while f and f M are within
-// these bounds (the low part of f M lies 2^-48 below it, normal floats end at 2^-126).
+// these bounds (the low part of f M lies 2^-48 below it, normal floats end at
+// 2^-126); outside them (a normalisation that is no float, a prediction next
+// to the smallest ones) f M and d - f M are formed in double.
 constexpr float kPairMost = 0x1p100f, kPairLeast = 0x1p-76f;
 
 // Bin (p, i): outputs, and the terms to be summed over bins into regs[0..NG]
@@ -378,9 +356,16 @@ __device__ __forceinline__ void bin_terms(const EpiArgs& a, int p, int i, const 
     if (a.eta) split_ff(a.norm * (1.0 + in.e), fh, fl);
     // mu = f M
     const float pr = __fmul_rn(fh, b.M.x);
-    const float2 mu = ff_norm(pr, __fmaf_rn(fh, b.M.y, __fmaf_rn(fl, b.M.x, __fmaf_rn(fh, b.M.x, -pr))));
-    double mu_d = (double)mu.x + (double)mu.y;
-    const float2 dm = ff_add(in.d, make_float2(-mu.x, -mu.y));  // d and mu are close
+    float2 mu = ff_norm(pr, __fmaf_rn(fh, b.M.y, __fmaf_rn(fl, b.M.x, __fmaf_rn(fh, b.M.x, -pr))));
+    float2 dm = ff_add(in.d, make_float2(-mu.x, -mu.y));  // d and mu are close
+    const bool wide = !(fabsf(fh) <= kPairMost && fabsf(fh) >= kPairLeast && fabsf(pr) <= kPairMost &&
+                        fabsf(pr) >= kPairLeast && in.d.x <= kPairMost);
+    double mu_wide = 0.0;
+    if (wide) {
+        mu_wide = (a.eta ? a.norm * (1.0 + in.e) : a.norm) * ((double)b.M.x + (double)b.M.y);
+        mu = to_ff(mu_wide);
+        dm = to_ff(a.data[a.data_per_point ? idx : i] - mu_wide);
+    }
     const float tf = dm.x / mu.x;                               // relative residual, 1e-7 is enough
     float g;
     float2 term;
@@ -394,20 +379,12 @@ __device__ __forceinline__ void bin_terms(const EpiArgs& a, int p, int i, const 
         term = make_float2(t, __fmaf_rn(h2, mu.y, __fmaf_rn(h2, mu.x, -t)));
         g = -2.0f * tf;  // 2 (1 - d / mu)
     }
-    if (!(fabsf(fh) <= kPairMost && fabsf(fh) >= kPairLeast && fabsf(pr) <= kPairMost && fabsf(pr) >= kPairLeast &&
-          in.d.x <= kPairMost)) {
-        const double d = a.data[a.data_per_point ? idx : i];
-        const WideTerm w = wide_term(a.eta ? a.norm * (1.0 + in.e) : a.norm, (double)b.M.x + (double)b.M.y, d, a.kind);
-        mu_d = w.mu;
-        term = w.term;
-        g = w.g;
-    }
     const bool pen = a.penalty != 0;
     if (pen) term = ff_add(term, to_ff(in.e * in.e / (a.sigma * a.sigma)));
     regs[0] = term;
 #pragma unroll
     for (int q = 0; q < NG; q++) regs[1 + q] = make_float2(g * (fh * b.d[q]), 0.f);
-    if (a.mu_out) a.mu_out[idx] = mu_d;
+    if (a.mu_out) a.mu_out[idx] = wide ? mu_wide : (double)mu.x + (double)mu.y;
     if (a.grad_eta_out)
         a.grad_eta_out[idx] = (double)g * a.norm * ((double)b.M.x + (double)b.M.y) + (pen ? 2.0 * in.e / (a.sigma * a.sigma) : 0.0);
 }
