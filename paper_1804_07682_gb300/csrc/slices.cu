@@ -23,6 +23,9 @@ __global__ void __launch_bounds__(W * 32) k_slices_reduce(const float2* __restri
     const int i = g * 32 + lane;
     BinInput in;
     if (w == 0) in = bin_input(ea, p, min(i, ea.nbins - 1));
+    // (and the point's constants, written before the node kernel began)
+    if (w == 0 && lane < (int)(sizeof(PointConst) + 127) / 128)
+        asm volatile("prefetch.global.L1 [%0];" ::"l"(reinterpret_cast<const char*>(pcs + p) + lane * 128));
     const float2* fin = sum_slices<NVM, W>(part, S, NV, w, lane);
     if (w == 0) {
         // the task sums T, N (anchored.cuh), then the per-baseline parts
