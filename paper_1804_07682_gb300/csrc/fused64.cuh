@@ -68,6 +68,7 @@ struct NodeMath64 {
 
 struct SplitArgs64 {
     const double2* grid;
+    int grouped;  // grid: [group of 32 bins][node][lane] as the bin mapping's, else bin-major
     int nbins, n, npts;
     int64_t per;
     int maxseg;
@@ -84,8 +85,7 @@ __global__ void __launch_bounds__(256) k_fused64_split(SplitArgs64 a) {
     constexpr int NV = M::NV;
     const int lane = threadIdx.x & 31;
     const int64_t w = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
-    const int64_t gn = (int64_t)a.nbins * a.n;
-    const int64_t total = gn * a.npts;
+    const int64_t total = (int64_t)a.nbins * a.n * a.npts;
     const int64_t f0 = w * a.per;
     const int64_t f1 = min(total, f0 + a.per);
     int last_p = -1;
@@ -103,7 +103,16 @@ __global__ void __launch_bounds__(256) k_fused64_split(SplitArgs64 a) {
         double acc[NV];
 #pragma unroll
         for (int v = 0; v < NV; v++) acc[v] = 0.0;
-        for (; f < seg_end; f += 32) m.update(a.grid[f % gn], acc);
+        // the lanes' nodes are neighbours in a bin-major grid and 512 bytes apart
+        // in a grouped one: the FP64 pipe covers the loads of either
+        const int64_t qn = q * a.n;
+        if (a.grouped) {
+            const double2* g = a.grid + (int64_t)(i >> 5) * a.n * 32 + (i & 31);
+            for (; f < seg_end; f += 32) m.update(g[(f - qn) * 32], acc);
+        } else {
+            const double2* g = a.grid + (int64_t)i * a.n;
+            for (; f < seg_end; f += 32) m.update(g[f - qn], acc);
+        }
         const int64_t w_first = (q * a.n) / a.per;
         const int64_t w_last = ((q + 1) * a.n - 1) / a.per;
         const int nseg = (int)(w_last - w_first + 1);

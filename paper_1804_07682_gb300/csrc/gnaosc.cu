@@ -571,7 +571,8 @@ gna_status enqueue_eval(gna_plan* plan, const EvalReq& q, cudaStream_t s, int* l
                         plan->d_pc, plan->bc, (float2*)plan->d_part, ea};
             CU(dispatch_split(plan->ph, plan->nl_inst, grad, spec, &a, sh.grid, plan->block, s));
         } else {
-            SplitArgs64 a{plan->grid64_split, plan->nbins, plan->n_uniform, plan->npts, sh.per, sh.maxseg,
+            const bool grouped = !plan->grid64_split;
+            SplitArgs64 a{grouped ? plan->grid64_bins : plan->grid64_split, grouped, plan->nbins, plan->n_uniform, plan->npts, sh.per, sh.maxseg,
                           plan->d_pc, plan->bc, (double*)plan->d_part, ea};
             CU(dispatch_split(2, plan->nl_inst, grad, spec, &a, sh.grid, plan->block, s));
         }
@@ -1155,7 +1156,9 @@ static gna_status plan_build(gna_plan* plan, const gna_plan_desc* d, cudaStream_
     CU(cudaMemcpyAsync(plan->d_edges, d->edges, sizeof(double) * (d->nbins + 1), cudaMemcpyHostToDevice, s));
     if (plan->has_split) {
         if (plan->ph < 2) TRY(dalloc(plan, &plan->grid_split, len_split));
-        if (want64) TRY(dalloc(plan, &plan->grid64_split, len_split));
+        // GNA_FP64: the split kernel reads the bins layout where there is one;
+        // the plain chain takes the bin-major one
+        if (want64 && (!plan->has_bins || want_plain)) TRY(dalloc(plan, &plan->grid64_split, len_split));
     }
     if (plan->has_bins) {
         if (quads) TRY(dalloc(plan, &plan->grid_rec, nquads * kQuadBytes));
@@ -1197,7 +1200,7 @@ static gna_status plan_build(gna_plan* plan, const gna_plan_desc* d, cudaStream_
         go += n;
     }
     // energy grids
-    if (plan->has_split) {
+    if (plan->grid_split || plan->grid64_split) {
         CU(launch_build_grid(d->nbins, d->nbins, plan->d_edges, gn[0], plan->gl_x[0], plan->gl_w[0], plan->e_scale, 0,
                              plan->grid_split, nullptr, plan->grid64_split, plan->plain64, s));
     }

@@ -1461,3 +1461,26 @@ def test_fit_layout_waits_for_the_first_fit(api, channel):
     assert bytes_[0] < 12.1 * nodes + 4e6 and bytes_[2] - bytes_[0] == 16 * nodes
     for a, b in zip(res[0], res[2]):
         assert np.array_equal(a, b)
+
+
+@pytest.mark.parametrize("nbins,n", [(33, 65000), (64, 1031), (40, 50)])
+def test_fp64_split_mapping_reads_either_layout(api, nbins, n):
+    """A default GNA_FP64 plan keeps one copy of its nodes: its split mapping
+    reads the bin mapping's layout, with the same results bit for bit as on a
+    plan that has the split mapping's own."""
+    e, L = np.linspace(1.8, 8.0, nbins + 1), [52.5, 30.0]
+    th = np.repeat(np.array([[0.307, 0.0218, 7.53e-5, 2.44e-3]]), 2, 0)
+    plans = {m: api.Plan(e, L, nodes_per_bin=n, npts=2, norm=1e4, prec="fp64", kind="poisson", max_datasets=2, mapping=m)
+             for m in (None, "split")}
+    assert plans[None].info()["device_bytes"] - plans["split"].info()["device_bytes"] < 16 * 31 * n + 40e6  # bins in groups, slices
+    data = plans["split"].eval(plans["split"].params_tensor(th), dev(np.ones(nbins)), mu=True)["mu"].clone().round()
+    plans[None].tuning = "mapping=split"
+    out = {}
+    for m, plan in plans.items():
+        o = plan.eval(plan.params_tensor(th), data, grad=True, mu=True, spectra=True)
+        p, c = plan.fit(plan.params_tensor(1.01 * th), data, iters=3)
+        out[m] = [x.cpu().numpy() for x in (o["chi2"], o["grad"], o["mu"], o["spectra"], p, c)]
+        plan.status()
+        plan.close()
+    for a, b in zip(out[None], out["split"]):
+        assert np.array_equal(a, b)
