@@ -10,6 +10,7 @@
 // per channel; the kernels evaluate three phases per (baseline, energy).
 #include <algorithm>
 #include <cmath>
+#include <mutex>
 #include <type_traits>
 
 #include "oscprob.h"
@@ -107,8 +108,8 @@ constexpr int64_t kSmallTurns = 1ll << (61 - 16);
 // some eighty wide integer multiplies and their shifts and additions per
 // probability, in place of three double sines (27 FP64 instructions each, at
 // 64 cycles a warp).  The table is read from shared memory with its cosine and
-// sine side by side; the blocks stay and walk over the energies, so that it is
-// loaded once each.  GB300: 4,000,000 energies at one baseline 529 -> 88 us,
+// sine side by side; a limited number of blocks walk over the energies, so that
+// it is loaded once each.  GB300: 4,000,000 energies at one baseline 529 -> 88 us,
 // 3,000,017 at two (mu -> e) 1032 -> 156 us.  Largest error against 113-bit
 // arithmetic, 1.8-12 MeV at 52.5 km: 1.5e-15 -> 5.2e-16; 0.5-5 GeV at 810 km,
 // mu -> e: 1.9e-16 -> 8.2e-17.
@@ -308,12 +309,38 @@ __global__ void __launch_bounds__(256) k_osc_f64phase(const double* __restrict__
     }
 }
 
+// Most blocks of k_osc_fp64: twice what the current device holds at a time
+// (asked once per device).  The second half starts as blocks of the first end
+// and evens them out: 4,000,000 energies 88.2 us, with one wave 90.3; a table
+// load per block is what more of them would cost.
+template <class C>
+cudaError_t osc_blocks(int64_t& blocks) {
+    static std::once_flag once[64];
+    static int count[64];
+    static cudaError_t err[64];
+    int dev = 0;
+    cudaError_t e = cudaGetDevice(&dev);
+    if (e != cudaSuccess) return e;
+    if (dev < 0 || dev >= 64) return cudaErrorInvalidDevice;
+    std::call_once(once[dev], [&] {
+        int sms = 0, per_sm = 0;
+        err[dev] = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+        if (err[dev] == cudaSuccess) err[dev] = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_osc_fp64<C>, 256, 0);
+        count[dev] = 2 * sms * std::max(per_sm, 1);
+    });
+    blocks = count[dev];
+    return err[dev];
+}
+
 template <class C>
 cudaError_t launch(const double* E, int64_t n, const C& oc, int prec, void* P, cudaStream_t s) {
     const int64_t blocks = (n + 255) / 256;
-    if (prec == GNA_FP64)
-        k_osc_fp64<C><<<(unsigned)std::min<int64_t>(blocks, 152 * 8), 256, 0, s>>>(E, n, oc, (double*)P);
-    else if (prec == GNA_MIXED_F64PHASE)
+    if (prec == GNA_FP64) {
+        int64_t most = 0;
+        const cudaError_t e = osc_blocks<C>(most);
+        if (e != cudaSuccess) return e;
+        k_osc_fp64<C><<<(unsigned)std::min(blocks, most), 256, 0, s>>>(E, n, oc, (double*)P);
+    } else if (prec == GNA_MIXED_F64PHASE)
         k_osc_f64phase<C><<<(unsigned)blocks, 256, 0, s>>>(E, n, oc, (float*)P);
     else
         k_osc_ff<C><<<(unsigned)blocks, 256, 0, s>>>(E, n, oc, (float*)P);
