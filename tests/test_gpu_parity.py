@@ -1059,17 +1059,19 @@ def test_general_fits_match_oracle(api, prec):
 @pytest.mark.parametrize("prec", ["f64phase", "ff"])
 @pytest.mark.parametrize("mapping", ["bins", "slices"])
 @pytest.mark.parametrize("nL", [1, 2, 3, 5, 9])
+@pytest.mark.parametrize("inverted", [False, True])
 @pytest.mark.parametrize("n,edges", [(1, (2.0, 9.0)), (3, (2.0, 9.0)), (4, (2.0, 9.0)), (5, (3.0, 3.4)), (33, (3.0, 3.4)),
                                      (130, (3.0, 3.4)), (67, (0.6, 12.0))])
-def test_anchored_chunks(api, prec, mapping, nL, n, edges):
+def test_anchored_chunks(api, prec, mapping, nL, n, edges, inverted):
     # orders around a quad and a chunk of nodes; fine grids (3-3.4 MeV: long
     # chunks), coarse ones (2-9 MeV with up to 5 nodes: every phase reduced)
     # and one that has both and lengths between (0.6-12 MeV); baselines below,
-    # at and beyond the packed instantiations; 37 bins: a ragged group
+    # at and beyond the packed instantiations; 37 bins: a ragged group; either
+    # mass ordering (a negative dm2_32: negative quotients of the phases)
     rng = np.random.default_rng(nL + n)
     e = np.linspace(edges[0], edges[1], 38)
     L = rng.uniform(1.0, 60.0, nL)
-    theta = np.array(wl.TRUTH) * 1.03
+    theta = np.array(wl.TRUTH) * 1.03 * ([1, 1, 1, -1] if inverted else 1)
     Nn = oracle.norm_for_total(e, n, L, wl.TRUTH)
     data = wl.poisson_data(Nn * (oracle.baseline_weights(L) @ oracle.binned(e, n, L, wl.TRUTH)), 7)
     ref = oracle.chain(e, n, L, theta, Nn, data, wl.POISSON)
@@ -1092,15 +1094,16 @@ def test_anchored_chunks(api, prec, mapping, nL, n, edges):
 @pytest.mark.parametrize("prec", ["f64phase", "ff"])
 @pytest.mark.parametrize("nL", [1, 2, 3, 5])
 @pytest.mark.parametrize("channel", [("mu", "e", False), ("mu", "mu", True), ("e", "tau", False)])
+@pytest.mark.parametrize("inverted", [False, True])
 @pytest.mark.parametrize("n,edges", [(1, (600.0, 4000.0)), (3, (600.0, 4000.0)), (5, (1500.0, 2000.0)), (34, (1500.0, 2000.0)),
                                      (131, (1500.0, 2000.0)), (21, (150.0, 3000.0))])
-def test_general_anchored_chunks(api, prec, nL, channel, n, edges):
+def test_general_anchored_chunks(api, prec, nL, channel, n, edges, inverted):
     # as test_anchored_chunks for the any-channel node kernels: single nodes,
-    # quads, chunks and ragged ends, coarse and fine grids, both mappings
+    # quads, chunks and ragged ends, coarse and fine grids, both mappings and orderings
     rng = np.random.default_rng(nL + n)
     e = np.linspace(edges[0], edges[1], 38)
     L = np.array([810.0, 295.0, 735.0, 700.0, 280.0])[:nL]
-    th = np.array(THETA_FULL) * 1.02
+    th = np.array(THETA_FULL) * 1.02 * ([1, 1, 1, 1, 1, -1] if inverted else 1)
     a, b, anti = channel
     mu_rb, _ = oracle.binned_general(e, n, L, THETA_FULL, a, b, anti, 1e-3)
     M = oracle.baseline_weights(L) @ mu_rb
@@ -1125,15 +1128,16 @@ def test_general_anchored_chunks(api, prec, nL, channel, n, edges):
 
 
 @pytest.mark.parametrize("nL", [1, 3, 9])
+@pytest.mark.parametrize("inverted", [False, True])
 @pytest.mark.parametrize("n,edges", [(1, (2.0, 9.0)), (3, (2.0, 9.0)), (5, (3.0, 3.4)), (33, (3.0, 3.4)), (130, (3.0, 3.4)),
                                      (1000, (3.0, 3.4)), (67, (0.6, 12.0))])
-def test_fp64_anchored_chunks(api, nL, n, edges):
+def test_fp64_anchored_chunks(api, nL, n, edges, inverted):
     # GNA_FP64: sincos per node (coarse grids), both lengths of polynomial
-    # (0.6-12 MeV has all three), whole bins and slices
+    # (0.6-12 MeV has all three), whole bins and slices, both mass orderings
     rng = np.random.default_rng(nL + n)
     e = np.linspace(edges[0], edges[1], 38)
     L = rng.uniform(1.0, 60.0, nL)
-    theta = np.array(wl.TRUTH) * 1.03
+    theta = np.array(wl.TRUTH) * 1.03 * ([1, 1, 1, -1] if inverted else 1)
     Nn = oracle.norm_for_total(e, n, L, wl.TRUTH)
     data = wl.poisson_data(Nn * (oracle.baseline_weights(L) @ oracle.binned(e, n, L, wl.TRUTH)), 7)
     ref = oracle.chain(e, n, L, theta, Nn, data, wl.POISSON)
@@ -1155,11 +1159,12 @@ def test_fp64_anchored_chunks(api, nL, n, edges):
 
 @pytest.mark.parametrize("nL", [1, 3])
 @pytest.mark.parametrize("channel", [("mu", "e", False), ("mu", "mu", True)])
+@pytest.mark.parametrize("inverted", [False, True])
 @pytest.mark.parametrize("n,edges", [(1, (600.0, 4000.0)), (5, (1500.0, 2000.0)), (131, (1500.0, 2000.0)), (21, (150.0, 3000.0))])
-def test_fp64_general_anchored_chunks(api, nL, channel, n, edges):
+def test_fp64_general_anchored_chunks(api, nL, channel, n, edges, inverted):
     e = np.linspace(edges[0], edges[1], 38)
     L = np.array([810.0, 295.0, 735.0])[:nL]
-    th = np.array(THETA_FULL) * 1.02
+    th = np.array(THETA_FULL) * 1.02 * ([1, 1, 1, 1, 1, -1] if inverted else 1)
     a, b, anti = channel
     mu_rb, _ = oracle.binned_general(e, n, L, THETA_FULL, a, b, anti, 1e-3)
     M = oracle.baseline_weights(L) @ mu_rb
@@ -1180,21 +1185,22 @@ def test_fp64_general_anchored_chunks(api, nL, channel, n, edges):
 
 
 @pytest.mark.parametrize("prec", ["fp64", "f64phase", "ff"])
-def test_oscprob_number_ranges(api, prec):
+@pytest.mark.parametrize("inverted", [False, True])
+def test_oscprob_number_ranges(api, prec, inverted):
     """Energies at the edges of the number range, and phases from next to zero
-    to many turns: each against the formula in double."""
+    to many turns, in both mass orderings: each against the formula in double."""
     E = np.array([5.0, 1.0, 2.0, np.nextafter(2.0, 0.0), np.nextafter(1.0, 2.0), 2.0 ** -20, 2.0 ** 20, 3e9, 1e15, 1e30,
                   1e300, 2.0 ** -1000, -5.0, np.inf, np.nan])
     L = [0.0, 52.5, 1.7, 1e4]
     for channel in (None, ("mu", "e"), ("mu", "mu")):
-        th = THETA_FULL
+        th = THETA_FULL[:5] + (-THETA_FULL[5] if inverted else THETA_FULL[5],)
         if channel is None:
             P = api.oscprob(dev(E), L, [th[i] for i in (0, 1, 4, 5)], prec).double().cpu().numpy()
         else:
             P = api.oscprob_general(dev(E), L, th, *channel, prec=prec).double().cpu().numpy()
         with np.errstate(all="ignore"):
-            ref = np.array([oracle_prob(*(channel or ("e", "e")), E, Lr, False) for Lr in L])
-            phase = np.array([1266.932679419849 * Lr * (th[4] + th[5]) / np.abs(E) for Lr in L])
+            ref = np.array([oracle_prob(*(channel or ("e", "e")), E, Lr, False, th) for Lr in L])
+            phase = np.array([1266.932679419849 * Lr * (th[4] + abs(th[5])) / np.abs(E) for Lr in L])
         # double: the phase's rounding, twice its 2^-53; mixed: FP32 polynomials
         # (2e-7 each) and, in double-float, 2^-44 of the phase up to its 2^12 pi
         top = {"fp64": 1e9, "f64phase": 1e6, "ff": 1e4}[prec]
@@ -1202,7 +1208,8 @@ def test_oscprob_number_ranges(api, prec):
         if prec != "fp64":  # 1/E is a pair of floats
             ok &= (np.abs(E) < 1e18) & (np.abs(E) > 1e-18)
         tol = {"fp64": 4e-16 + 1e-15 * phase, "f64phase": 6e-7 + 1e-12 * phase, "ff": 6e-7 + 1e-11 * phase}[prec]
-        assert ok[:, :5].any(axis=0).all()
+        # compared: every energy of 1 - 5 MeV at 52.5 and 1.7 km, and no phase at all (0 km)
+        assert ok[:3, :5].all()
         assert (np.abs(P - ref)[ok] <= tol[ok]).all()
         if prec == "fp64":
             # probabilities next to zero or one: the terms (up to 2x each) are
@@ -1484,3 +1491,27 @@ def test_fp64_split_mapping_reads_either_layout(api, nbins, n):
         plan.close()
     for a, b in zip(out[None], out["split"]):
         assert np.array_equal(a, b)
+
+
+@pytest.mark.parametrize("prec", ["fp64", "f64phase", "ff"])
+@pytest.mark.parametrize("zero", [0, 1])
+@pytest.mark.parametrize("nL", [1, 3, 9])
+def test_a_splitting_of_zero(api, nL, zero, prec):
+    # one pair's phases, and their sums, vanish for every baseline: compensated
+    # sums of zeros, chunks as long as they get (33 nodes: one and a rest)
+    rng = np.random.default_rng(nL)
+    e, n = np.linspace(3.0, 3.4, 38), 33
+    L = rng.uniform(1.0, 60.0, nL)
+    theta = np.array(wl.TRUTH)
+    theta[2 + zero] = 0.0
+    Nn = oracle.norm_for_total(e, n, L, wl.TRUTH)
+    data = wl.poisson_data(Nn * (oracle.baseline_weights(L) @ oracle.binned(e, n, L, wl.TRUTH)), 7)
+    ref = oracle.chain(e, n, L, theta, Nn, data, wl.POISSON)
+    plan = api.Plan(e, L, nodes_per_bin=n, norm=Nn, prec=prec, kind="poisson")
+    out = plan.eval(plan.params_tensor(theta), dev(data), grad=True, mu=True, spectra=True)
+    plan.status()
+    plan.close()
+    assert rel(out["mu"][0].cpu().numpy(), ref["mu"]) < TOL[prec]
+    assert rel(out["spectra"][0].cpu().numpy(), ref["mu_rb"]) < TOL[prec]
+    assert normrel(out["grad"][0].cpu().numpy(), ref["grad"][:4]) < GTOL[prec]
+    check_chi2(out["chi2"][0].item(), ref, data, wl.POISSON, TOL[prec], tag="zero splitting %d %d" % (nL, zero), plain=False)
