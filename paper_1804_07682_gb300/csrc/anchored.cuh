@@ -159,6 +159,17 @@ __device__ __forceinline__ void angle_add2(f32x2 s1, f32x2 h1, f32x2 s2, f32x2 h
     h = fma2(neg2(s1), s2, fma2(h1, h2, add2(h1, h2)));
 }
 
+// Multiple q of the unit 1 / inv = a + b (a of 8 bits) nearest to a phase p + lo
+// beyond kFarPhase, where one rounding of p inv no longer gives it: the rounding
+// of p inv and lo are no longer small against the polynomials' range, and the
+// magic number ends at 2^22 (the quotients are doubled phases': twice those of
+// reduce_pi_ff).  Its integer, then the rest's.  Good to q < 2^24.
+constexpr float kFarPhase = 1e5f;
+__device__ __forceinline__ float far_quotient(float p, float lo, float inv, float a, float b) {
+    const float q = rintf(__fmul_rn(p, inv));
+    return q + rintf(__fmul_rn(__fadd_rn(__fmaf_rn(-q, b, __fmaf_rn(-q, a, p)), lo), inv));
+}
+
 // Phase c * e reduced modulo pi (as reduce_pi_ff / reduce_pi_f64) and the
 // parity of the multiple of pi as a float's sign bit.
 __device__ __forceinline__ float reduce_sign_ff(float ch, float cl, float eh, float el, unsigned& sign) {
@@ -167,7 +178,11 @@ __device__ __forceinline__ float reduce_sign_ff(float ch, float cl, float eh, fl
     const float lo = __fmaf_rn(ch, el, __fmaf_rn(cl, eh, e));
     const float qm = __fmaf_rn(p, GNA_INV_PI_F, GNA_ROUND_MAGIC);
     sign = __float_as_uint(qm) << 31;
-    const float q = __fsub_rn(qm, GNA_ROUND_MAGIC);
+    float q = __fsub_rn(qm, GNA_ROUND_MAGIC);
+    if (fabsf(p) > kFarPhase) {
+        q = far_quotient(p, lo, GNA_INV_PI_F, GNA_PI_A, GNA_PI_B2);
+        sign = (unsigned)__float2int_rn(q) << 31;
+    }
     float r = __fmaf_rn(-q, GNA_PI_A, p);
     r = __fmaf_rn(-q, GNA_PI_B2, r);
     return __fadd_rn(r, lo);

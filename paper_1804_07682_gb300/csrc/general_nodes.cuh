@@ -86,7 +86,11 @@ __device__ __forceinline__ float phase_q(const PointConst* pc, int r, bool p32, 
         const float lo = __fmaf_rn(ch, el, __fmaf_rn(cl, eh, e));
         const float qm = __fmaf_rn(p, 2.0f * GNA_INV_PI_F, GNA_ROUND_MAGIC);
         quad = __float_as_uint(qm) & 3u;
-        const float q = __fsub_rn(qm, GNA_ROUND_MAGIC);
+        float q = __fsub_rn(qm, GNA_ROUND_MAGIC);
+        if (fabsf(p) > kFarPhase) {
+            q = far_quotient(p, lo, 2.0f * GNA_INV_PI_F, 0.5f * GNA_PI_A, 0.5f * GNA_PI_B);
+            quad = (unsigned)__float2int_rn(q) & 3u;
+        }
         float x = __fmaf_rn(-q, 0.5f * GNA_PI_A, p);
         x = __fmaf_rn(-q, 0.5f * GNA_PI_B, x);
         return __fadd_rn(x, __fmaf_rn(-q, 0.5f * GNA_PI_C, lo));

@@ -1515,3 +1515,26 @@ def test_a_splitting_of_zero(api, nL, zero, prec):
     assert rel(out["spectra"][0].cpu().numpy(), ref["mu_rb"]) < TOL[prec]
     assert normrel(out["grad"][0].cpu().numpy(), ref["grad"][:4]) < GTOL[prec]
     check_chi2(out["chi2"][0].item(), ref, data, wl.POISSON, TOL[prec], tag="zero splitting %d %d" % (nL, zero), plain=False)
+
+
+@pytest.mark.parametrize("channel", [None, ("mu", "mu", False), ("mu", "e", True)])
+@pytest.mark.parametrize("nL", [1, 3])
+@pytest.mark.parametrize("L", [1e5, 2.2e6, 4.1e6, 7.3e6, 1e7])
+@pytest.mark.parametrize("wide", [False, True])
+def test_double_float_phases_far_out(api, L, nL, channel, wide):
+    """Phases up to 2^22 pi (x about L at 3 MeV) in the double-float mode, on
+    chunks of nodes and on nodes by themselves (wide): their error grows with
+    the phase, q 5.1e-12 from the reduction (q half-turns) and 2^-46 of the
+    phase from the product, and nothing else is added."""
+    e = np.linspace(3.0, 3.0 + (3.0 if wide else 3e2) / L, 33)
+    th = [0.307, 0.0218, 7.53e-5, 2.44e-3] if channel is None else THETA_FULL
+    mu = {}
+    for prec in ("fp64", "ff"):
+        plan = api.Plan(e, L * (1 + 1e-3 * np.arange(nL)), nodes_per_bin=8 if wide else 64, prec=prec, kind="poisson", channel=channel)
+        f = plan.eval if channel is None else plan.eval_general
+        mu[prec] = f(plan.params_tensor(th), dev(np.ones(32)), mu=True)["mu"][0].cpu().numpy()
+        plan.status()
+        plan.close()
+    x = 1266.932679419849 * 2.52e-3 * L * 1.002 / 3.0
+    W = np.exp(0.87 - 0.48 - 0.819) * (e[1] - e[0])
+    assert np.abs(mu["ff"] - mu["fp64"]).max() < W * (1e-7 + 2 * x * (5.2e-12 / np.pi + 2.0 ** -46))
