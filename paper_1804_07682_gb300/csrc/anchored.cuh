@@ -171,7 +171,9 @@ __device__ __forceinline__ float far_quotient(float p, float lo, float inv, floa
 }
 
 // Phase c * e reduced modulo pi (as reduce_pi_ff / reduce_pi_f64) and the
-// parity of the multiple of pi as a float's sign bit.
+// parity of the multiple of pi as a float's sign bit.  FAR: of any size
+// (anchors lie below kFarPhase, chunk_quads).
+template <bool FAR>
 __device__ __forceinline__ float reduce_sign_ff(float ch, float cl, float eh, float el, unsigned& sign) {
     const float p = __fmul_rn(ch, eh);
     const float e = __fmaf_rn(ch, eh, -p);
@@ -179,7 +181,7 @@ __device__ __forceinline__ float reduce_sign_ff(float ch, float cl, float eh, fl
     const float qm = __fmaf_rn(p, GNA_INV_PI_F, GNA_ROUND_MAGIC);
     sign = __float_as_uint(qm) << 31;
     float q = __fsub_rn(qm, GNA_ROUND_MAGIC);
-    if (fabsf(p) > kFarPhase) {
+    if (FAR && fabsf(p) > kFarPhase) {
         q = far_quotient(p, lo, GNA_INV_PI_F, GNA_PI_A, GNA_PI_B2);
         sign = (unsigned)__float2int_rn(q) << 31;
     }
@@ -197,24 +199,27 @@ __device__ __forceinline__ float reduce_sign_f64(double c, double e, unsigned& s
     return (float)fma(-q, GNA_PI_DC, r);
 }
 
-// The phase of baseline r's pair 21 or 32 at 1/E = eh + el: doubled (y) or not (x).
-template <int PH, bool DOUBLED>
+// The doubled phase of baseline r's pair 21 or 32 at 1/E = eh + el.
+template <int PH, bool FAR>
 __device__ __forceinline__ float phase(const PointConst* pc, int r, bool p32, float eh, float el, unsigned& sign) {
-    constexpr float f = DOUBLED ? 2.0f : 1.0f;
     if constexpr (PH == 0) {
         const float ch = p32 ? pc->c32h[r] : pc->c21h[r], cl = p32 ? pc->c32l[r] : pc->c21l[r];
-        return reduce_sign_ff(f * ch, f * cl, eh, el, sign);
+        return reduce_sign_ff<FAR>(2.0f * ch, 2.0f * cl, eh, el, sign);
     } else {
-        return reduce_sign_f64((double)f * (p32 ? pc->c32[r] : pc->c21[r]), (double)eh + (double)el, sign);
+        return reduce_sign_f64(2.0 * (p32 ? pc->c32[r] : pc->c21[r]), (double)eh + (double)el, sign);
     }
 }
 
 // Quads per chunk of a task of nq quads: at most kChunkQuads, and few enough
 // that no node lies further than `swing` from the anchor; 0: a quad's own
-// nodes already do.  Chunks of a task are made about equally long.
-__device__ __forceinline__ int chunk_quads(float cmax, float step, int nq, float swing) {
+// nodes already do, or (double-float phases) phases exceed kFarPhase, which
+// the anchors' reduction does not take.  Chunks of a task are made about
+// equally long.
+template <int PH>
+__device__ __forceinline__ int chunk_quads(float cmax, float2 step, int nq, float swing) {
+    if (PH == 0 && 2.0f * cmax * step.y > kFarPhase) return 0;
     // the anchor is node 2 len of the chunk: a node lies at most 2 len steps from it
-    const float lf = swing / (4.0f * cmax * step);
+    const float lf = swing / (4.0f * cmax * step.x);
     if (!(lf >= 1.0f)) return 0;
     const int most = lf >= (float)kChunkQuads ? kChunkQuads : (int)lf;
     const int nch = (nq + most - 1) / most;
@@ -231,7 +236,7 @@ constexpr int kQuadBytes = 3 * 512;
 struct NodeTask {
     int p, b, nq;     // point, group of 32 bins, quads
     const char* rec;  // first quad
-    float step;       // largest step of 1/E between neighbouring nodes of the group's bins
+    float2 step;      // largest step of 1/E between neighbouring nodes of the group's bins, and largest 1/E
 };
 
 __device__ __forceinline__ NodeTask node_task(const BinArgs& a, int t) {
@@ -468,13 +473,13 @@ struct MultiMath {
             if constexpr (PH == 0) {
                 const float2 l = *reinterpret_cast<const float2*>(pc->c21l + r);
                 const float2 m = *reinterpret_cast<const float2*>(pc->c32l + r);
-                x[0] = reduce_sign_ff(c[2 * i].x, 2.0f * l.x, eh, el, s[0]);
-                x[1] = reduce_sign_ff(c[2 * i].y, 2.0f * l.y, eh, el, s[1]);
-                x[2] = reduce_sign_ff(c[2 * i + 1].x, 2.0f * m.x, eh, el, s[2]);
-                x[3] = reduce_sign_ff(c[2 * i + 1].y, 2.0f * m.y, eh, el, s[3]);
+                x[0] = reduce_sign_ff<false>(c[2 * i].x, 2.0f * l.x, eh, el, s[0]);
+                x[1] = reduce_sign_ff<false>(c[2 * i].y, 2.0f * l.y, eh, el, s[1]);
+                x[2] = reduce_sign_ff<false>(c[2 * i + 1].x, 2.0f * m.x, eh, el, s[2]);
+                x[3] = reduce_sign_ff<false>(c[2 * i + 1].y, 2.0f * m.y, eh, el, s[3]);
             } else {
 #pragma unroll
-                for (int j = 0; j < 4; j++) x[j] = phase<PH, true>(pc, r + (j & 1), j >= 2, eh, el, s[j]);
+                for (int j = 0; j < 4; j++) x[j] = phase<PH, false>(pc, r + (j & 1), j >= 2, eh, el, s[j]);
             }
             a[2 * i] = pack2(x[0], x[1]);
             a[2 * i + 1] = pack2(x[2], x[3]);
@@ -612,7 +617,7 @@ __global__ void __maxnreg__(NP >= 3 ? 168 : 128) k_nodes_multi(BinArgs a) {
         const bool whole = a.S <= 1;
         BinInput bin;
         if (whole) bin = bin_input(a.ea, k.p, min(k.b * 32 + lane, a.nbins - 1));
-        const int len = chunk_quads(pc->cmax, k.step, k.nq, kSwing);
+        const int len = chunk_quads<PH>(pc->cmax, k.step, k.nq, kSwing);
         const bool direct = len == 0;
         const int step = direct ? 1 : len;
         // the spectra's parts, and the sums q between two passes over the nodes
@@ -788,7 +793,7 @@ __global__ void __maxnreg__(112) k_nodes_one(BinArgs a) {
         queue.prefetch();
         NodeTask k = node_task(a, t);
         in.start(k);
-        int len = chunk_quads(a.pcs[k.p].cmax, k.step, k.nq, kSwing);
+        int len = chunk_quads<PH>(a.pcs[k.p].cmax, k.step, k.nq, kSwing);
         float2 an = load_anchor(k, 0, min(max(len, 1), k.nq));
         while (true) {
             int tn = a.ntasks;
@@ -820,8 +825,8 @@ __global__ void __maxnreg__(112) k_nodes_one(BinArgs a) {
                 const int kb = min(k.nq, ka + step);
                 if (!direct) {
                     unsigned q21, q32;
-                    x.a21 = dup2(phase<PH, true>(pc, 0, false, an.x, an.y, q21));
-                    x.a32 = dup2(phase<PH, true>(pc, 0, true, an.x, an.y, q32));
+                    x.a21 = dup2(phase<PH, false>(pc, 0, false, an.x, an.y, q21));
+                    x.a32 = dup2(phase<PH, false>(pc, 0, true, an.x, an.y, q32));
                     const f32x2 nah = dup2(-an.x), nal = dup2(-an.y);
                     if (kb < k.nq) an = load_anchor(k, kb, min(step, k.nq - kb));
                     WeightSum w;
@@ -885,7 +890,7 @@ __global__ void __maxnreg__(112) k_nodes_one(BinArgs a) {
                 t = tn;
                 k = kn;
                 in.start(k);
-                len = chunk_quads(a.pcs[k.p].cmax, k.step, k.nq, kSwing);
+                len = chunk_quads<PH>(a.pcs[k.p].cmax, k.step, k.nq, kSwing);
                 an = load_anchor(k, 0, min(max(len, 1), k.nq));
             }
             float2 sp[1];

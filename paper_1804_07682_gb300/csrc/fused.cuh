@@ -295,7 +295,7 @@ __global__ void __launch_bounds__(256, GNA_SPLIT_MIN_BLOCKS) k_fused_split(Split
 // A whole-bin task of the anchored kernels.
 struct BinTask {
     int p, b, nq;  // point, group, quads of nodes
-    float step;    // largest step of 1/E between neighbouring nodes
+    float2 step;   // largest step of 1/E between neighbouring nodes, and largest 1/E
     int64_t quad;  // first quad in the plan's records
 };
 
@@ -316,7 +316,7 @@ struct BinArgs {
     float2* part;  // slice values [ntasks][NVs][32] (S > 1)
     int NVs;       // values per slice and bin
     int nL, spec;  // baselines, per-baseline sums requested
-    const float* step;  // [ngrids][ngroups] largest step of 1/E between neighbouring nodes
+    const float2* step;  // [ngrids][ngroups] as BinTask's
 };
 
 // The fits' node kernel (grid layout [group][node][lane], each warp load 512

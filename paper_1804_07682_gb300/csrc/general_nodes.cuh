@@ -77,7 +77,7 @@ __device__ __forceinline__ float2 sum3(float a, float b, float c) {
 // Doubled phase of baseline r's pair 21 or 32 modulo pi/2, and the quadrant
 // (mod 4).  The quotient's steps q PI_A / 2 and q PI_B / 2 are exact (12-bit
 // parts); r is rounded once, when the small part is added.
-template <int PH>
+template <int PH, bool FAR>  // FAR: as reduce_sign_ff
 __device__ __forceinline__ float phase_q(const PointConst* pc, int r, bool p32, float eh, float el, unsigned& quad) {
     if constexpr (PH == 0) {
         const float ch = 2.0f * (p32 ? pc->c32h[r] : pc->c21h[r]), cl = 2.0f * (p32 ? pc->c32l[r] : pc->c21l[r]);
@@ -87,7 +87,7 @@ __device__ __forceinline__ float phase_q(const PointConst* pc, int r, bool p32, 
         const float qm = __fmaf_rn(p, 2.0f * GNA_INV_PI_F, GNA_ROUND_MAGIC);
         quad = __float_as_uint(qm) & 3u;
         float q = __fsub_rn(qm, GNA_ROUND_MAGIC);
-        if (fabsf(p) > kFarPhase) {
+        if (FAR && fabsf(p) > kFarPhase) {
             q = far_quotient(p, lo, 2.0f * GNA_INV_PI_F, 0.5f * GNA_PI_A, 0.5f * GNA_PI_B);
             quad = (unsigned)__float2int_rn(q) & 3u;
         }
@@ -238,7 +238,7 @@ __device__ __forceinline__ void finish_gen_bins(const GenArgs& ga, int p, int b,
 template <int PH, bool GRAD>
 __device__ __forceinline__ void gen_single(const PointConst* pc, int r, float eh, float el, float W, GenSums<GRAD>& g) {
     unsigned q21, q32;
-    const f32x2 y[1] = {pack2(phase_q<PH>(pc, r, false, eh, el, q21), phase_q<PH>(pc, r, true, eh, el, q32))};
+    const f32x2 y[1] = {pack2(phase_q<PH, true>(pc, r, false, eh, el, q21), phase_q<PH, true>(pc, r, true, eh, el, q32))};
     f32x2 s[1], h[1], s3, h3;
     sinhq2(y, s, h);
     angle_rest2(dup2(s[0].x), dup2(h[0].x), dup2(s[0].y), dup2(h[0].y), s3, h3);
@@ -297,7 +297,7 @@ __global__ void __maxnreg__(128) k_gen_one(GenArgs ga) {
         const PointConst* pc = a.pcs + k.p;
         BinInput bin;
         if (whole) bin = bin_input(a.ea, k.p, min(k.b * 32 + lane, a.nbins - 1));
-        const int len = chunk_quads(pc->cmax, k.step, k.nq, kSwingQ);
+        const int len = chunk_quads<PH>(pc->cmax, k.step, k.nq, kSwingQ);
         const bool direct = len == 0;
         const int step = direct ? 1 : len;
         GenOneMath<PH, GRAD> x;
@@ -311,8 +311,8 @@ __global__ void __maxnreg__(128) k_gen_one(GenArgs ga) {
             const int kb = min(k.nq, ka + step);
             if (!direct) {
                 unsigned q21, q32;
-                x.a21 = dup2(phase_q<PH>(pc, 0, false, an.x, an.y, q21));
-                x.a32 = dup2(phase_q<PH>(pc, 0, true, an.x, an.y, q32));
+                x.a21 = dup2(phase_q<PH, false>(pc, 0, false, an.x, an.y, q21));
+                x.a32 = dup2(phase_q<PH, false>(pc, 0, true, an.x, an.y, q32));
                 const f32x2 nah = dup2(-an.x), nal = dup2(-an.y);
                 if (kb < k.nq) an = load_anchor(k, kb, min(step, k.nq - kb));
                 WeightSum w;
@@ -400,7 +400,7 @@ struct GenMultiMath {
             unsigned q[4];
             float x[4];
 #pragma unroll
-            for (int j = 0; j < 4; j++) x[j] = phase_q<PH>(pc, r0 + 2 * i + (j & 1), j >= 2, eh, el, q[j]);
+            for (int j = 0; j < 4; j++) x[j] = phase_q<PH, false>(pc, r0 + 2 * i + (j & 1), j >= 2, eh, el, q[j]);
             a[2 * i] = pack2(x[0], x[1]);
             a[2 * i + 1] = pack2(x[2], x[3]);
             quads |= (q[0] | q[2] << 2 | q[1] << 4 | q[3] << 6) << (8 * i);
@@ -489,7 +489,7 @@ __global__ void __maxnreg__(NP == 2 ? 168 : 128) k_gen_multi(GenArgs ga) {
         const PointConst* pc = a.pcs + k.p;
         BinInput bin;
         if (whole) bin = bin_input(a.ea, k.p, min(k.b * 32 + lane, a.nbins - 1));
-        const int len = chunk_quads(pc->cmax, k.step, k.nq, kSwingQ);
+        const int len = chunk_quads<PH>(pc->cmax, k.step, k.nq, kSwingQ);
         const bool direct = len == 0;
         const int step = direct ? 1 : len;
         GenTaskSums q;

@@ -134,7 +134,8 @@ struct gna_plan {
     std::vector<const double*> gl_x, gl_w;  // their Gauss-Legendre rules (device)
     int* d_tasks = nullptr;
     int ntasks = 0;
-    float* d_step = nullptr;  // [ngrids][ngroups] largest step of 1/E between neighbouring nodes
+    // [ngrids][ngroups] largest step of 1/E between neighbouring nodes, and largest 1/E
+    float2* d_step = nullptr;
     int res_ctas[2] = {0, 0}, res_block[2] = {0, 0};  // resident blocks per SM of the node kernel (without, with gradient)
     // [1 + npts + npts*ngroups (+ npts*nbins, split)]: work counter, groups
     // finished per point, bins finished per group, segments finished per bin
@@ -1223,7 +1224,7 @@ static gna_status plan_build(gna_plan* plan, const gna_plan_desc* d, cudaStream_
             else CU(launch_sum_weights(nullptr, plan->grid_rec + qoff[g] * kQuadBytes, d->nbins, gn[g], sw, swf, s));
         }
     }
-    std::vector<float> step;  // (copied from below: lives until the stream is synchronised)
+    std::vector<float2> step;  // (copied from below: lives until the stream is synchronised)
     std::vector<BinTask> desc;
     if (plan->has_bins) {
         // neighbouring zeros of P_n are less than pi / (n + 1/2) apart in
@@ -1235,10 +1236,10 @@ static gna_status plan_build(gna_plan* plan, const gna_plan_desc* d, cudaStream_
                 double w = 0.0;
                 for (int i = b * 32; i < std::min(d->nbins, (b + 1) * 32); i++)
                     w = std::max(w, 0.5 * (d->edges[i + 1] - d->edges[i]) / (d->edges[i] * d->edges[i]));
-                step[(size_t)g * ngroups + b] = (float)(w * M_PI / (gn[g] + 0.5));
+                step[(size_t)g * ngroups + b] = make_float2((float)(w * M_PI / (gn[g] + 0.5)), (float)(1.0 / d->edges[b * 32]));
             }
         TRY(dalloc(plan, &plan->d_step, step.size()));
-        CU(cudaMemcpyAsync(plan->d_step, step.data(), sizeof(float) * step.size(), cudaMemcpyHostToDevice, s));
+        CU(cudaMemcpyAsync(plan->d_step, step.data(), sizeof(float2) * step.size(), cudaMemcpyHostToDevice, s));
     }
     CU(cudaStreamCreateWithFlags(&plan->cap_stream, cudaStreamNonBlocking));
     // task list (bins mapping): (point, group) ordered by decreasing node count

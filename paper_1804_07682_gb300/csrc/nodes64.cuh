@@ -49,7 +49,7 @@ struct Args64 {
     double* part;         // [ntasks][NVs][32] (S > 1)
     int NVs;
     int nL, spec;
-    const float* step;    // [ngrids][ngroups] largest step of 1/E
+    const float2* step;   // [ngrids][ngroups] .x: largest step of 1/E
 };
 
 // Values of a task: T(3), [V(3)], [N(3)], [Z(3)], sum W, [per-baseline parts].
@@ -213,7 +213,7 @@ __global__ void __launch_bounds__(128) k_nodes64(Args64 a) {
         const double2* g = a.grid + a.goff[gi] + ((int64_t)b * n + k0) * 32 + lane;
         const PointConst* pc = a.pcs + p;
         // nodes per chunk: the anchor is node m / 2, at most m / 2 steps from the others
-        const float per = 2.0f * pc->cmax * a.step[(int64_t)gi * a.ngroups + b];
+        const float per = 2.0f * pc->cmax * a.step[(int64_t)gi * a.ngroups + b].x;
         const float ms = 2.0f * 0.015625f / per, ml = 2.0f * 0.25f / per;
         // below eight nodes the anchors cost more than the longer polynomials
         const bool small = ms >= 8.0f;
