@@ -11,25 +11,25 @@
 #define GNA_COS_C2 (4.166396707e-02f)
 #define GNA_COS_C3 (-1.385575277e-03f)
 #define GNA_COS_C4 (2.319028135e-05f)
-// Chunk-anchored loops, |r| <= 1.821796: polynomial error sin 2.33e-08, cos 2.46e-09.
+// Chunk-anchored loops, |r| <= 1.821796: polynomial error sin 2.33e-08, cos 5.25e-09 (cos - 1: 4.22e-09 of itself).
 #define GNA_SINA_C1 (-1.666663587e-01f)
 #define GNA_SINA_C2 (8.332575671e-03f)
 #define GNA_SINA_C3 (-1.977937063e-04f)
 #define GNA_SINA_C4 (2.548287284e-06f)
-#define GNA_COSA_C1 (-4.999999702e-01f)
-#define GNA_COSA_C2 (4.166654870e-02f)
-#define GNA_COSA_C3 (-1.388737932e-03f)
-#define GNA_COSA_C4 (2.471726839e-05f)
-#define GNA_COSA_C5 (-2.540818400e-07f)
-// Chunk-anchored loops, |r| <= 1.186398: polynomial error sin 2.28e-10, cos 3.68e-09.
+#define GNA_COSA_C1 (-5.000000000e-01f)
+#define GNA_COSA_C2 (4.166664928e-02f)
+#define GNA_COSA_C3 (-1.388838165e-03f)
+#define GNA_COSA_C4 (2.475560905e-05f)
+#define GNA_COSA_C5 (-2.590579697e-07f)
+// Chunk-anchored loops, |r| <= 1.186398: polynomial error sin 2.28e-10, cos 1.14e-08 (cos - 1: 2.08e-08 of itself).
 #define GNA_SINQ_C1 (-1.666666567e-01f)
 #define GNA_SINQ_C2 (8.333275095e-03f)
 #define GNA_SINQ_C3 (-1.982997928e-04f)
 #define GNA_SINQ_C4 (2.666453838e-06f)
-#define GNA_COSQ_C1 (-4.999999404e-01f)
-#define GNA_COSQ_C2 (4.166620970e-02f)
-#define GNA_COSQ_C3 (-1.387852593e-03f)
-#define GNA_COSQ_C4 (2.389178371e-05f)
+#define GNA_COSQ_C1 (-5.000000000e-01f)
+#define GNA_COSQ_C2 (4.166652262e-02f)
+#define GNA_COSQ_C3 (-1.388277742e-03f)
+#define GNA_COSQ_C4 (2.405918167e-05f)
 // pi = PI_A + PI_B + PI_C; PI_A and PI_B have 12 significant bits.
 #define GNA_PI_A (3.140625f)
 #define GNA_PI_B (0.00096750259399414062f)

@@ -57,7 +57,9 @@ def fit_sequential(basis, target, weight):
     return np.array(fixed)
 
 
-def fit(R_MAX=R_MAX, N_SIN=N_SIN, N_COS=N_COS):
+def fit(R_MAX=R_MAX, N_SIN=N_SIN, N_COS=N_COS, relative=False):
+    """relative: cos r - 1 to a relative error (where 1 - cos is what is left of
+    a probability next to zero), else cos r to an absolute one."""
     t = np.cos(np.linspace(0, np.pi, 6001))  # Chebyshev points on [-1, 1]
     r = 0.5 * (t + 1) * R_MAX
     r = r[r > 1e-3]
@@ -69,7 +71,7 @@ def fit(R_MAX=R_MAX, N_SIN=N_SIN, N_COS=N_COS):
     # cos: (cos r - 1) / u = C1 + C2 u + ...; absolute error weight u
     fc = (np.cos(r) - 1) / u
     Bc = np.stack([u ** k for k in range(N_COS)], axis=1)
-    cc = fit_sequential(Bc, fc, u)
+    cc = fit_sequential(Bc, fc, 1 / np.abs(fc) if relative else u)
     return cs, cc
 
 
@@ -140,12 +142,14 @@ def main():
     for k, c in enumerate(cc32):
         out.write("#define GNA_COS_C%d (%.9ef)\n" % (k + 1, float(c)))
     for suffix, rmax, ns, nc in ANCHORED:
-        ks, kc = fit(rmax, ns, nc)
-        r = np.linspace(-rmax, rmax, 200001)
+        ks, kc = fit(rmax, ns, nc, relative=True)
+        r = np.linspace(-rmax, rmax, 200000)  # (not 0)
         u = r * r
         e_s = np.abs(r + r * u * sum(float(c) * u ** k for k, c in enumerate(ks)) - np.sin(r)).max()
-        e_c = np.abs(1 + u * sum(float(c) * u ** k for k, c in enumerate(kc)) - np.cos(r)).max()
-        out.write("// Chunk-anchored loops, |r| <= %.6f: polynomial error sin %.2e, cos %.2e.\n" % (rmax, e_s, e_c))
+        h = -2 * np.sin(0.5 * r) ** 2
+        d_c = np.abs(u * sum(float(c) * u ** k for k, c in enumerate(kc)) - h)
+        out.write("// Chunk-anchored loops, |r| <= %.6f: polynomial error sin %.2e, cos %.2e (cos - 1: %.2e of itself).\n"
+                  % (rmax, e_s, d_c.max(), (d_c / -h)[np.abs(r) > 1e-3].max()))
         for k, c in enumerate(ks):
             out.write("#define GNA_SIN%s_C%d (%.9ef)\n" % (suffix, k + 1, float(c)))
         for k, c in enumerate(kc):

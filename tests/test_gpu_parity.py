@@ -1538,3 +1538,32 @@ def test_double_float_phases_far_out(api, L, nL, channel, wide):
     x = 1266.932679419849 * 2.52e-3 * L * 1.002 / 3.0
     W = np.exp(0.87 - 0.48 - 0.819) * (e[1] - e[0])
     assert np.abs(mu["ff"] - mu["fp64"]).max() < W * (1e-7 + 2 * x * (5.2e-12 / np.pi + 2.0 ** -46))
+
+
+@pytest.mark.parametrize("prec", ["f64phase", "ff"])
+@pytest.mark.parametrize("general", [False, True])
+def test_one_minus_cosine_keeps_its_relative_error(api, general, prec):
+    """Near an oscillation minimum at maximal mixing the prediction is a sum of
+    1 - cos r: the polynomial holds to 2.1e-8 of it (any channel; 4.2e-9 in the
+    survival chain), which the mean over bins and points shows; what else there
+    is, roundings of 6e-8 in each of 64 x 40 sums, averages to 2e-9."""
+    K = 1e3 / (4 * 0.1973269804)
+    L, dm = 52.5, 7.53e-5
+    E0 = K * dm * L / (np.pi / 2)
+    e = E0 / (1 + np.linspace(0.15, 0.03, 41) * 2 / np.pi)  # x = pi/2 + 0.03 .. 0.15
+    th = np.array([[0.5, 1e-15, 0.5, 0.3, dm, 1e-12]] if general else [[0.5, 0.0, dm, 0.0]])
+    th = np.repeat(th, 64, 0)
+    th[:, 4 if general else 2] *= 1 + np.linspace(0.0, 1e-3, 64)
+    mu = {}
+    for p in ("fp64", prec):
+        plan = api.Plan(e, [L], nodes_per_bin=33, npts=64, prec=p, kind="poisson", channel=("e", "e", False) if general else None)
+        f = plan.eval_general if general else plan.eval
+        mu[p] = f(plan.params_tensor(th), dev(np.ones(40)), mu=True)["mu"].cpu().numpy()
+        plan.status()
+        plan.close()
+    mean = float((mu[prec] / mu["fp64"] - 1).mean())
+    # the survival chain's double-float reduction rounds p - pi to 2^-29 (r below
+    # 2^-3) with the same low bits at every point, those of pi's second part:
+    # up to twice that over r = 0.06 .. 0.3
+    same = 2 * 2.0 ** -29 / 0.1 if prec == "ff" and not general else 0.0
+    assert abs(mean) < (2.1e-8 if general else 4.2e-9) + 6e-9 + same, mean
