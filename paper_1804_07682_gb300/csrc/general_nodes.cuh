@@ -77,8 +77,10 @@ __device__ __forceinline__ float2 sum3(float a, float b, float c) {
 // Doubled phase of baseline r's pair 21 or 32 modulo pi/2, and the quadrant
 // (mod 4).  The quotient's steps q PI_A / 2 and q PI_B / 2 are exact (12-bit
 // parts); r is rounded once, when the small part is added.
-template <int PH, bool FAR>  // FAR: as reduce_sign_ff
-__device__ __forceinline__ float phase_q(const PointConst* pc, int r, bool p32, float eh, float el, unsigned& quad) {
+// FAR: as reduce_sign_ff; low: what that rounding dropped
+template <int PH, bool FAR>
+__device__ __forceinline__ float phase_q(const PointConst* pc, int r, bool p32, float eh, float el, unsigned& quad,
+                                         float& low) {
     if constexpr (PH == 0) {
         const float ch = 2.0f * (p32 ? pc->c32h[r] : pc->c21h[r]), cl = 2.0f * (p32 ? pc->c32l[r] : pc->c21l[r]);
         const float p = __fmul_rn(ch, eh);
@@ -93,7 +95,9 @@ __device__ __forceinline__ float phase_q(const PointConst* pc, int r, bool p32, 
         }
         float x = __fmaf_rn(-q, 0.5f * GNA_PI_A, p);
         x = __fmaf_rn(-q, 0.5f * GNA_PI_B, x);
-        return __fadd_rn(x, __fmaf_rn(-q, 0.5f * GNA_PI_C, lo));
+        const float y = __fmaf_rn(-q, 0.5f * GNA_PI_C, lo), s = __fadd_rn(x, y);
+        low = __fadd_rn(__fsub_rn(x, s), y);  // (|x| >= |y|, or both are tiny)
+        return s;
     } else {
         const double p = 2.0 * (p32 ? pc->c32[r] : pc->c21[r]) * ((double)eh + (double)el);
         const double qm = fma(p, 2.0 * GNA_INV_PI_D, 6755399441055744.0);
@@ -101,8 +105,16 @@ __device__ __forceinline__ float phase_q(const PointConst* pc, int r, bool p32, 
         const double q = qm - 6755399441055744.0;
         double x = fma(-q, 0.5 * GNA_PI_DA, p);
         x = fma(-q, 0.5 * GNA_PI_DB, x);
-        return (float)fma(-q, 0.5 * GNA_PI_DC, x);
+        x = fma(-q, 0.5 * GNA_PI_DC, x);
+        const float s = (float)x;
+        low = (float)(x - (double)s);
+        return s;
     }
+}
+template <int PH, bool FAR>
+__device__ __forceinline__ float phase_q(const PointConst* pc, int r, bool p32, float eh, float el, unsigned& quad) {
+    float low;
+    return phase_q<PH, FAR>(pc, r, p32, eh, el, quad, low);
 }
 
 // What a chunk in quadrant q adds, as big + part (T, V: |big| >= |part| or
@@ -311,9 +323,15 @@ __global__ void __maxnreg__(128) k_gen_one(GenArgs ga) {
             const int kb = min(k.nq, ka + step);
             if (!direct) {
                 unsigned q21, q32;
-                x.a21 = dup2(phase_q<PH, false>(pc, 0, false, an.x, an.y, q21));
-                x.a32 = dup2(phase_q<PH, false>(pc, 0, true, an.x, an.y, q32));
-                const f32x2 nah = dup2(-an.x), nal = dup2(-an.y);
+                float low;
+                x.a32 = dup2(phase_q<PH, false>(pc, 0, true, an.x, an.y, q32, low));
+                // the anchor moves to where pair 32's phase is that float: its
+                // rounding would be common to the chunk (nu_mu disappearance, eight
+                // spectra of 4 - 1000 nodes per bin, largest error of a bin: 7.3e-8
+                // -> 6.4e-8 of mu, with a reduction per node 6.7e-8)
+                const float shift = low != 0.f ? __fdividef(-low, x.c32.x) : 0.f;
+                x.a21 = dup2(fmaf(x.c21.x, shift, phase_q<PH, false>(pc, 0, false, an.x, an.y, q21)));
+                const f32x2 nah = dup2(-an.x), nal = dup2(-an.y - shift);
                 if (kb < k.nq) an = load_anchor(k, kb, min(step, k.nq - kb));
                 WeightSum w;
                 in.wait();
