@@ -86,8 +86,8 @@ PROFILE_EVERY = 8
 TRAFFIC_CAPTURE = {
     "split": {"sources_sha256": "4e84d90634a932986bddfc3627e81e2c61c0ee248b37d8a2b42cd44e71396f94",
               "bytes": 265113600 + 4114176},
-    "slices": {"sources_sha256": "758a3ede1b15d5e3d1203945af46e51ec9d5aceb2947f384eeee84720709fbb9",
-               "bytes": 201989376 + 3093760 + 6620928 + 0},
+    "slices": {"sources_sha256": "6cb2571b43ea1bb029cd4d96bfe0a44fb6b543e4a0fcc3cc8fe427725c76bb35",
+               "bytes": 204826368 + 3265536 + 6620672 + 0},
 }
 KERNEL_SOURCES = ["paper_1804_07682_gb300/csrc/common.cuh", "paper_1804_07682_gb300/csrc/fused.cuh",
                   "paper_1804_07682_gb300/csrc/anchored.cuh",

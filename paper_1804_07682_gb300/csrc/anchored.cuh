@@ -38,7 +38,7 @@
 // takes half the issue slots, so the loads, address arithmetic and loop
 // control no longer compete with the arithmetic.  An FMA (packed or not) that
 // reads three registers no neighbouring instruction reads runs at two thirds
-// of the rate (25 against 38 T lane operations/s measured): the polynomials
+// of the rate (26 against 39 T lane operations/s measured): the polynomials
 // of all phases in hand are stepped together, so that neighbours share a
 // coefficient.  Nodes come through a ring in shared memory (cp.async): with
 // loads into registers the warps spent half their time waiting for them.

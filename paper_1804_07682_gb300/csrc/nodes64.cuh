@@ -17,7 +17,7 @@
 // nodes lie further apart take sincos per node as before.  Measured (GB300):
 // 1000 bins x 16384 nodes x 8 baselines with gradient 18.9 -> 12.1 ms, 1000 x
 // 262 x 8 825 -> 435 us (the split mapping filled a sixth of the GPU), nu_mu
-// disappearance 400 x 513 x 2 23.6 ms -> 116 us (whole bins: 13 warps); the
+// disappearance 400 x 513 x 2 23.3 ms -> 102 us (whole bins: 13 warps); the
 // FP64 pipe is 89 % busy with 16 warps per SM.
 //
 // Per baseline and pair (y = 2x):

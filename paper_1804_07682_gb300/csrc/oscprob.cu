@@ -285,8 +285,9 @@ __global__ void __launch_bounds__(256) k_osc_ff(const double* __restrict__ E, in
     for (int r = 0; r < oc.nL; r++) P[(int64_t)r * n + k] = mixed_ff(oc, r, eh, el);
 }
 
-// Phases of turns.cuh: no FP64 instruction is left (27 per probability before).
-// GB300: 3,000,017 energies at two baselines (mu -> e) 281 -> 39 us.
+// Phases of turns.cuh: no FP64 instruction (three phases formed and reduced in
+// double take 27).  GB300: 3,000,017 energies at two baselines (mu -> e) 39 us,
+// 281 with phases in double.
 template <class C>
 __global__ void __launch_bounds__(256) k_osc_f64phase(const double* __restrict__ E, int64_t n,
                                                       const __grid_constant__ C oc, float* __restrict__ P) {
