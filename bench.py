@@ -40,10 +40,11 @@ def fp32_ops_general(nL: int, grad: bool) -> int:
     """Algorithmic FP32 operations (FMA = 1) per energy node of the any-channel
     chain's chunk-anchored node kernels: per (node, baseline) two phases by one
     FMA each from the chunk's anchor 2, sin and cos - 1 of both 20, what the
-    third pair has beyond them 4, weighted sums 6 (12 with the gradient);
+    third pair has beyond them 4, weighted sums 6 (12 with the gradient),
+    with one baseline two differences from the anchor's sine and cosine;
     per node the offset of 1/E 3, W/E 1, the sum of W 4 and of W/E 1 (with the
     gradient).  Anchors and the additions of a chunk's sums are not counted."""
-    return nL * (38 if grad else 32) + 8 + (1 if grad else 0)
+    return nL * (38 if grad else 32) + (2 if nL == 1 else 0) + 8 + (1 if grad else 0)
 
 
 def fp32_ops_per_node(nL: int, grad: bool, spec: bool) -> int:

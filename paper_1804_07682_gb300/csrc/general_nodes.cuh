@@ -28,8 +28,9 @@
 // 1.1e-8 so).
 //
 // What bounds it: the FP32 pipe.  Operations per (node, baseline), gradient
-// on: phases 2, sines and cosines 20, addition 4, sums 12 = 38 (reducing each
-// node's phases, with sin^2, cos^2 and sin cos of three phases: 120-150).
+// on: phases 2, sines and cosines 20, addition 4, sums 12 = 38, two more with
+// one baseline (reducing each node's phases, with sin^2, cos^2 and sin cos of
+// three phases: 120-150).
 #pragma once
 
 #include "anchored.cuh"
@@ -66,12 +67,6 @@ __device__ __forceinline__ void sinhq2(const f32x2 (&r)[N], f32x2 (&s)[N], f32x2
 __device__ __forceinline__ void angle_rest2(f32x2 s1, f32x2 h1, f32x2 s2, f32x2 h2, f32x2& s, f32x2& h) {
     s = fma2(h1, s2, mul2(s1, h2));
     h = fma2(neg2(s1), s2, mul2(h1, h2));
-}
-
-// a + b + c as a float pair.
-__device__ __forceinline__ float2 sum3(float a, float b, float c) {
-    const float2 s = ff_add(make_float2(a, 0.f), make_float2(b, 0.f));
-    return ff_add(s, make_float2(c, 0.f));
 }
 
 // Doubled phase of baseline r's pair 21 or 32 modulo pi/2, and the quadrant
@@ -162,13 +157,15 @@ struct GenSums {
             kzero(Z[j]);
         }
     }
-    // a chunk's sums of the three pairs, [1] the third's beyond the other two; q21, q32: quadrants
-    __device__ __forceinline__ void add(unsigned q21, unsigned q32, const float (&S)[3], const float (&H)[3],
-                                        const float (&SE)[3], const float (&HE)[3], float2 c, float e) {
-        add(0, q21, make_float2(S[0], 0.f), make_float2(H[0], 0.f), SE[0], HE[0], c, e);
-        add(1, (q21 + q32) & 3u, sum3(S[0], S[2], S[1]), sum3(H[0], H[2], H[1]), SE[0] + SE[2] + SE[1],
-            HE[0] + HE[2] + HE[1], c, e);
-        add(2, q32, make_float2(S[2], 0.f), make_float2(H[2], 0.f), SE[2], HE[2], c, e);
+    // a chunk's sums of the three pairs, [1] the third's beyond the other two,
+    // S, H of pair 32 as pairs; q21, q32: quadrants
+    __device__ __forceinline__ void add(unsigned q21, unsigned q32, const float (&S)[2], const float (&H)[2], float2 S32,
+                                        float2 H32, const float (&SE)[3], const float (&HE)[3], float2 c, float e) {
+        const float2 s = make_float2(S[0], 0.f), h = make_float2(H[0], 0.f);
+        add(0, q21, s, h, SE[0], HE[0], c, e);
+        add(1, (q21 + q32) & 3u, ff_add(ff_add(s, S32), make_float2(S[1], 0.f)),
+            ff_add(ff_add(h, H32), make_float2(H[1], 0.f)), SE[0] + SE[2] + SE[1], HE[0] + HE[2] + HE[1], c, e);
+        add(2, q32, S32, H32, SE[2], HE[2], c, e);
     }
     // a chunk's sums of pair j
     __device__ __forceinline__ void add(int j, unsigned q, float2 S, float2 H, float SE, float HE, float2 c, float e) {
@@ -255,20 +252,35 @@ __device__ __forceinline__ void gen_single(const PointConst* pc, int r, float eh
     sinhq2(y, s, h);
     angle_rest2(dup2(s[0].x), dup2(h[0].x), dup2(s[0].y), dup2(h[0].y), s3, h3);
     const float We = W * eh;
-    const float S[3] = {W * s[0].x, W * s3.x, W * s[0].y}, H[3] = {W * h[0].x, W * h3.x, W * h[0].y};
+    const float S[2] = {W * s[0].x, W * s3.x}, H[2] = {W * h[0].x, W * h3.x};
     const float SE[3] = {We * s[0].x, We * s3.x, We * s[0].y}, HE[3] = {We * h[0].x, We * h3.x, We * h[0].y};
-    g.add(q21, q32, S, H, SE, HE, make_float2(W, 0.f), We);
+    g.add(q21, q32, S, H, make_float2(W * s[0].y, 0.f), make_float2(W * h[0].y, 0.f), SE, HE, make_float2(W, 0.f), We);
 }
 
 // ---------------------------------------------------- one baseline -------
+// S and H of pair 32 are summed as differences from their values s0, h0 at the
+// anchor, which enter with the chunk's weight: FP32 sums of up to 32 terms near
+// 0.7 (the quadrants' edges) were the largest error of a bin that is one chunk
+// (nu_mu disappearance in 40 - 500 bins of 4 - 2400 nodes, largest error of a
+// bin: 1.8e-7 of mu, 6.0e-8 so; a reduction and a compensated sum per node
+// 7.5e-8; scan of 1021 points 135 -> 138 us).
 template <int PH, bool GRAD>
 struct GenOneMath {
     f32x2 c21, c32, a21, a32;
     f32x2 S[3], H[3], SE[3], HE[3];
+    float s0, h0;
 
     __device__ __forceinline__ void zero() {
 #pragma unroll
         for (int j = 0; j < 3; j++) S[j] = H[j] = SE[j] = HE[j] = f32x2{0.f, 0.f};
+    }
+    // s0, h0: at a32
+    __device__ __forceinline__ void base() {
+        const f32x2 y[1] = {a32};
+        f32x2 s[1], h[1];
+        sinhq2(y, s, h);
+        s0 = s[0].x;
+        h0 = h[0].x;
     }
     __device__ __forceinline__ void pair(const NodePair& n, f32x2 nah, f32x2 nal, f32x2 we) {
         const f32x2 d = add2(add2(n.e, nah), add2(n.l, nal));
@@ -278,10 +290,10 @@ struct GenOneMath {
         angle_rest2(s[0], h[0], s[1], h[1], s3, h3);
         H[0] = fma2(n.w, h[0], H[0]);
         H[1] = fma2(n.w, h3, H[1]);
-        H[2] = fma2(n.w, h[1], H[2]);
+        H[2] = fma2(n.w, add2(h[1], dup2(-h0)), H[2]);
         S[0] = fma2(n.w, s[0], S[0]);
         S[1] = fma2(n.w, s3, S[1]);
-        S[2] = fma2(n.w, s[1], S[2]);
+        S[2] = fma2(n.w, add2(s[1], dup2(-s0)), S[2]);
         if constexpr (GRAD) {
             HE[0] = fma2(we, h[0], HE[0]);
             HE[1] = fma2(we, h3, HE[1]);
@@ -332,6 +344,7 @@ __global__ void __maxnreg__(128) k_gen_one(GenArgs ga) {
                 const float shift = low != 0.f ? __fdividef(-low, x.c32.x) : 0.f;
                 x.a21 = dup2(fmaf(x.c21.x, shift, phase_q<PH, false>(pc, 0, false, an.x, an.y, q21)));
                 const f32x2 nah = dup2(-an.x), nal = dup2(-an.y - shift);
+                x.base();
                 if (kb < k.nq) an = load_anchor(k, kb, min(step, k.nq - kb));
                 WeightSum w;
                 in.wait();
@@ -359,7 +372,8 @@ __global__ void __maxnreg__(128) k_gen_one(GenArgs ga) {
                     SE[v] = x.SE[v].x + x.SE[v].y;
                     HE[v] = x.HE[v].x + x.HE[v].y;
                 }
-                g.add(q21, q32, S, H, SE, HE, c, es);
+                g.add(q21, q32, {S[0], S[1]}, {H[0], H[1]}, ff_add(ff_mul(x.s0, 0.f, c), make_float2(S[2], 0.f)),
+                      ff_add(ff_mul(x.h0, 0.f, c), make_float2(H[2], 0.f)), SE, HE, c, es);
                 x.zero();
             } else {
                 in.wait();
@@ -563,7 +577,8 @@ __global__ void __maxnreg__(NP == 2 ? 168 : 128) k_gen_multi(GenArgs ga) {
                                 SE[j] = half ? x.SE[i][j].y : x.SE[i][j].x;
                                 HE[j] = half ? x.HE[i][j].y : x.HE[i][j].x;
                             }
-                            g.add(q21, q32, S, H, SE, HE, c, es);
+                            g.add(q21, q32, {S[0], S[1]}, {H[0], H[1]}, make_float2(S[2], 0.f), make_float2(H[2], 0.f), SE,
+                                  HE, c, es);
                             save_gen<NS, GRAD>(comp, stride, i, half, g);
                         }
                     x.zero();

@@ -1567,3 +1567,19 @@ def test_one_minus_cosine_keeps_its_relative_error(api, general, prec):
     # up to twice that over r = 0.06 .. 0.3
     same = 2 * 2.0 ** -29 / 0.1 if prec == "ff" and not general else 0.0
     assert abs(mean) < (2.1e-8 if general else 4.2e-9) + 6e-9 + same, mean
+
+
+@pytest.mark.parametrize("prec", ["f64phase", "ff"])
+@pytest.mark.parametrize("channel", [("mu", "mu", True), ("mu", "e", False)])
+@pytest.mark.parametrize("n", [12, 30])
+def test_one_chunk_between_quadrants(api, channel, n, prec):
+    """Bins that are one chunk whose doubled phase 32 lies near 3 pi / 4, where
+    sin r and cos r - 1 are largest: they are summed as differences from the
+    anchor's values.  Left are the nodes' own roundings: three of 2^-25 / sqrt 3
+    in a sine of 0.7, over P = 0.15 (nu_mu -> nu_mu) and averaged over n nodes:
+    1.4e-7 / sqrt n, less where P is a small part of the sines (seen: half of it,
+    0.8e-7 / sqrt n allowed for nu_mu -> nu_e).  Sums of the sines themselves
+    gave 2.4e-7 / sqrt n and 1.8e-7 / sqrt n."""
+    e = np.linspace(2150.0, 2300.0, 13)
+    err = [derivative_errors(api, e[i:i + 2], [810.0], n, prec, channel, 1e-3, seed=i)[0] for i in range(12)]
+    assert np.sqrt(np.mean(np.square(err))) < (1.4e-7 if channel[1] == "mu" else 0.8e-7) / np.sqrt(n), err
